@@ -276,7 +276,8 @@ def kernel_traffic(workload, p, B, kind="decode"):
 # valid while these are unchanged
 KERNEL_SOURCES = {
     "decode": ["decode.cu", "pp_common.cuh", "pp_select.cuh", "pp_kernels.h", "api.cu"],
-    "grouped": ["grouped.cu", "pp_common.cuh", "pp_select.cuh", "pp_tc.cuh", "pp_kernels.h", "api.cu"],
+    "grouped": ["grouped.cu", "union.cu", "pp_common.cuh", "pp_launch.h", "pp_select.cuh", "pp_tc.cuh",
+                "pp_kernels.h", "api.cu"],
 }
 
 

@@ -55,7 +55,7 @@ struct Layout {
     size_t logits, ids, counts, gates, tlog, th, stats;
     // grouped path
     size_t part, bits, gexp, invpos, wcnt, blkcnt, blkbase, offsets, n_items, items, perm_token, perm_gate, H, Y,
-        yacc, overflow;
+        yacc, overflow, dpart;
     size_t total;
 };
 
@@ -95,6 +95,7 @@ Layout layout(const pp_desc& d, int T) {
         L.Y = take((size_t)g.ycap * d.d_model * 2);
         L.yacc = take(Tn * (size_t)d.d_model * 4);
         L.overflow = take(16);
+        L.dpart = take(union_part_floats((int)Tn, d.d_model) * 4);
     }
     L.total = off;
     return L;
@@ -257,6 +258,8 @@ GroupedArgs grouped_args(const pp_desc& d, int T, void* ws, const void* x, const
     a.Y = reinterpret_cast<__nv_bfloat16*>(b + L.Y);
     a.yacc = reinterpret_cast<float*>(b + L.yacc);
     a.overflow = reinterpret_cast<int*>(b + L.overflow);
+    a.dpart = reinterpret_cast<float*>(b + L.dpart);
+    a.bar = &reinterpret_cast<Control*>(b)->bar;
     a.status = &reinterpret_cast<Control*>(b)->status;
     a.timeout_ns = kDefaultTimeoutNs;
     return a;
@@ -414,7 +417,8 @@ pp_status pp_route(const pp_desc* desc, const void* x, int T, const void* W_r, f
     const Ws w = ws_views(*desc, T, ws);
     const float kp = rule_kernel_param(desc->rule, p, desc->n_experts);
     if (use_grouped(*desc, T)) {
-        const GroupedArgs a = grouped_args(*desc, T, ws, x, W_r, nullptr, nullptr, nullptr, kp, *out, nullptr);
+        GroupedArgs a = grouped_args(*desc, T, ws, x, W_r, nullptr, nullptr, nullptr, kp, *out, nullptr);
+        a.bits = nullptr;  // no FFN reads the selection
         return cuda_status(grouped_route(a, st));
     }
     const int ts = decode_ts_limit(*desc);
@@ -443,6 +447,7 @@ pp_status pp_sparse_ffn(const pp_desc* desc, const void* x, int T, const void* W
     const Ws w = ws_views(*desc, T, ws);
     if (use_grouped(*desc, T)) {
         const GroupedArgs a = grouped_args(*desc, T, ws, x, nullptr, W_gate, W_up, W_down, 0.0f, *sel, y);
+        PP_TRY(cuda_status(grouped_load_selection(a, st)));
         return cuda_status(grouped_ffn(a, device_info().sms, st));
     }
     const int ts = decode_ts_limit(*desc);
@@ -472,7 +477,14 @@ pp_status pp_layer(const pp_desc* desc, const void* x, int T, const void* W_r, c
     pp_selection s = sel_out ? *sel_out : pp_selection{w.ids, w.counts, w.gates, nullptr};
     const float kp = rule_kernel_param(desc->rule, p, desc->n_experts);
     if (use_grouped(*desc, T)) {
-        const GroupedArgs a = grouped_args(*desc, T, ws, x, W_r, W_gate, W_up, W_down, kp, s, y);
+        GroupedArgs a = grouped_args(*desc, T, ws, x, W_r, W_gate, W_up, W_down, kp, s, y);
+        if (T <= kUnionMaxT) {
+            if (!sel_out) {  // nobody reads the rank order
+                a.ids = a.counts = nullptr;
+                a.gates = nullptr;
+            }
+            return cuda_status(union_layer(a, true, device_info().sms, st));
+        }
         PP_TRY(cuda_status(grouped_route(a, st)));
         return cuda_status(grouped_ffn(a, device_info().sms, st));
     }

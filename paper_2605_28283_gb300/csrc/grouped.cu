@@ -26,6 +26,7 @@
 // All waits are bounded (PP_ERR_TIMEOUT).
 #include "pp_common.cuh"
 #include "pp_kernels.h"
+#include "pp_launch.h"
 #include "pp_select.cuh"
 #include "pp_tc.cuh"
 
@@ -145,10 +146,15 @@ PP_DEVINL float sum_partials(const float* __restrict__ part, int nsplit, size_t 
     return v;
 }
 
+// The selection is written in two forms: rank order (ids, counts, gates) for
+// the caller, and per expert for the FFN kernels -- bits[t] (E bits in 8
+// words) and gexp[t][e], the gate weight, 0 where e is not activated.  bits is
+// NULL when no FFN follows (pp_route).
 template <int S>
 __global__ void __launch_bounds__(256) select_part_kernel(const float* __restrict__ part, int nsplit, int T, int E,
                                                           float p, int rule, int gate, int32_t* ids, int32_t* counts,
-                                                          float* gates, float* logits_out, unsigned* status) {
+                                                          float* gates, float* logits_out, uint32_t* bits,
+                                                          float* gexp, unsigned* status) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
@@ -159,13 +165,33 @@ __global__ void __launch_bounds__(256) select_part_kernel(const float* __restric
     bool finite = true;
     const int k = warp_select<S>(load, E, p, rule, key, &finite);
     if (!finite && lane == 0) record_status(status, PP_ERR_NONFINITE);
+    float* grow = gexp + (size_t)t * E;
+    if (bits) {
+        for (int e = lane; e < E; e += 32) grow[e] = 0.0f;
+        __syncwarp();  // before the activated experts' weights below
+    }
+    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
     for (int s = 0; s < S; s++) {
         const int r = lane * S + s;
         if (r >= E) continue;
         const bool on = finite && r < k;
-        ids[(size_t)t * E + r] = on ? key_index(key[s]) : -1;
-        gates[(size_t)t * E + r] = on ? gate_of(gate, key[s]) : 0.0f;
+        const int e = on ? key_index(key[s]) : -1;
+        const float gv = on ? gate_of(gate, key[s]) : 0.0f;
+        ids[(size_t)t * E + r] = e;
+        gates[(size_t)t * E + r] = gv;
+        if (on && bits) {
+            grow[e] = gv;
+#pragma unroll
+            for (int i = 0; i < 8; i++) w[i] |= (e >> 5) == i ? 1u << (e & 31) : 0u;
+        }
+    }
+    if (bits) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const uint32_t v = __reduce_or_sync(kFull, w[i]);
+            if (lane == i) bits[(size_t)t * 8 + i] = v;
+        }
     }
     if (lane == 0) counts[t] = k;
     if (logits_out)
@@ -175,7 +201,7 @@ __global__ void __launch_bounds__(256) select_part_kernel(const float* __restric
 __global__ void __launch_bounds__(256) select_part_cta_kernel(const float* __restrict__ part, int nsplit, int T,
                                                               int E, float p, int rule, int gate, int32_t* ids,
                                                               int32_t* counts, float* gates, float* logits_out,
-                                                              unsigned* status) {
+                                                              uint32_t* bits, float* gexp, unsigned* status) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
     __shared__ __align__(16) CtaSelScratch sc;
@@ -186,8 +212,13 @@ __global__ void __launch_bounds__(256) select_part_cta_kernel(const float* __res
     float g;
     const int k = cta_select_fn(load, E, p, rule, true, sc, status, &on, &r, &g);
     const int j = threadIdx.x;
-    write_selection_row(ids + (size_t)t * E, gates + (size_t)t * E, j, E, k, on, r,
-                        on ? (gate == PP_GATE_NONE ? 1.0f : sigmoidf_(g)) : 0.0f);
+    const float gv = on ? (gate == PP_GATE_NONE ? 1.0f : sigmoidf_(g)) : 0.0f;
+    write_selection_row(ids + (size_t)t * E, gates + (size_t)t * E, j, E, k, on, r, gv);
+    if (bits) {
+        const unsigned bal = __ballot_sync(kFull, on);
+        if ((j & 31) == 0) bits[(size_t)t * 8 + (j >> 5)] = bal;
+        if (j < E) gexp[(size_t)t * E + j] = gv;
+    }
     if (j < E && logits_out) logits_out[(size_t)t * E + j] = g;
     if (j == 0) counts[t] = k;
 }
@@ -198,19 +229,30 @@ __global__ void __launch_bounds__(256) select_part_cta_kernel(const float* __res
 __global__ void __launch_bounds__(256) select_part_cut_kernel(const float* __restrict__ part, int nsplit, int T, int E,
                                                               float p, int rule, int gate, int32_t* ids,
                                                               int32_t* counts, float* gates, float* logits_out,
-                                                              unsigned* status) {
+                                                              uint32_t* bits, float* gexp, unsigned* status) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
     __shared__ __align__(16) CutShared sc;
     __shared__ __align__(16) WarpCand cand[256];
+    __shared__ float gx[256];     // gate weight per expert
+    __shared__ uint32_t bw[8];    // activated experts
     const int t = blockIdx.x, j = threadIdx.x;
+    gx[j] = 0.0f;  // ordered before the cut's writes by its barriers
+    if (j < 8) bw[j] = 0u;
     const float g = j < E ? sum_partials(part, nsplit, (size_t)T * E, (size_t)t * E + j) : -INFINITY;
     int32_t* idr = ids + (size_t)t * E;
     float* gtr = gates + (size_t)t * E;
     const int k = cta_mass_cut(g, E, p, rule, sc, cand, status, [&](int r, int e, float ge) {
+        const float gv = gate == PP_GATE_NONE ? 1.0f : sigmoidf_(ge);
         idr[r] = e;
-        gtr[r] = gate == PP_GATE_NONE ? 1.0f : sigmoidf_(ge);
-    }, [] {});
+        gtr[r] = gv;
+        gx[e] = gv;
+        atomicOr(&bw[e >> 5], 1u << (e & 31));
+    }, [] {});  // its last barrier orders gx and bw before the reads below
+    if (bits) {
+        if (j < 8) bits[(size_t)t * 8 + j] = bw[j];
+        if (j < E) gexp[(size_t)t * E + j] = gx[j];
+    }
     for (int r = k + j; r < E; r += 256) {
         idr[r] = -1;
         gtr[r] = 0.0f;
@@ -378,164 +420,6 @@ __global__ void __launch_bounds__(kDispBlock) dispatch_scatter_kernel(const uint
             perm_gate[pos] = gexp[(size_t)t * E + e];
             invpos[(size_t)t * E + e] = pos;
         }
-    }
-}
-
-// All of the dispatch for T <= 256 tokens in one CTA of 1024 threads (small
-// batches are latency-bound: four kernels with a serial loop over the
-// experts cost more than their work).  Shared memory holds, per expert, the
-// 256-bit mask of the tokens that activated it; an assignment (t, e) lands
-// at offsets[e] + (tokens below t in e's mask), so tokens stay in ascending
-// order within each expert, as in the multi-block path; work items hold at
-// most item_rows rows.  Writes the same
-// outputs as that path (bits, offsets, work items, perm_token, perm_gate,
-// invpos) and clears the overflow flag of the down projection.  Gates of a
-// repeated id add up (with three or more copies the order of the additions
-// is not fixed).
-constexpr int kSmallDispatchMaxT = 256;
-
-__global__ void __launch_bounds__(1024) dispatch_small_kernel(const int32_t* __restrict__ ids,
-                                                              const int32_t* __restrict__ counts,
-                                                              const float* __restrict__ gates, int T, int E,
-                                                              uint32_t* bits, int* offsets, WorkItem* items,
-                                                              int* n_items, int* perm_token, float* perm_gate,
-                                                              int* invpos, int* overflow, int item_rows,
-                                                              unsigned* status) {
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    __shared__ uint32_t mask[kMaxExperts][8];              // tokens of expert e
-    __shared__ uint32_t dup[kSmallDispatchMaxT][8];        // entry (t, r) repeats an earlier id of token t
-    __shared__ int off_s[kMaxExperts + 1], item_s[kMaxExperts + 1];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < kMaxExperts * 8; i += blockDim.x) {
-        (&mask[0][0])[i] = 0u;
-        (&dup[0][0])[i] = 0u;
-    }
-    if (tid == 0) *overflow = 0;
-    __syncthreads();
-    // warp w takes tokens w + 32 i, lane r their entries r, r + 32, ...; the
-    // count and entry r = lane of each of the warp's tokens are read once, all
-    // loads independent (the three passes below reuse them)
-    constexpr int kTokPerWarp = kSmallDispatchMaxT / 32;
-    int ck[kTokPerWarp], ce[kTokPerWarp];
-    float cg[kTokPerWarp];
-#pragma unroll
-    for (int i = 0; i < kTokPerWarp; i++) {
-        const int t = warp + 32 * i;
-        ck[i] = 0;
-        ce[i] = -1;
-        cg[i] = 0.0f;
-        if (t < T) {
-            ck[i] = counts[t];
-            if (lane < E) {
-                ce[i] = ids[(size_t)t * E + lane];
-                cg[i] = gates[(size_t)t * E + lane];
-            }
-        }
-    }
-    // token masks
-#pragma unroll
-    for (int i = 0; i < kTokPerWarp; i++) {
-        const int t = warp + 32 * i;
-        if (t >= T) break;
-        int k = ck[i];
-        if (k < 0 || k > E) {
-            if (lane == 0) record_status(status, PP_ERR_INVALID_ARG);
-            k = k < 0 ? 0 : E;
-        }
-        ck[i] = k;
-        for (int r = lane; r < k; r += 32) {
-            const int e = r == lane ? ce[i] : ids[(size_t)t * E + r];
-            if (e < 0 || e >= E) {
-                record_status(status, PP_ERR_INVALID_ARG);
-                continue;
-            }
-            const uint32_t bit = 1u << (t & 31);
-            if (atomicOr(&mask[e][t >> 5], bit) & bit) atomicOr(&dup[t][r >> 5], 1u << (r & 31));
-        }
-    }
-    __syncthreads();
-    // per-expert counts -> offsets and work items (warp 0 scans, 8 experts per lane)
-    if (warp == 0) {
-        int c[8], m[8], cs = 0, ms = 0;
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-            const int e = lane * 8 + q;
-            int n = 0;
-            if (e < E)
-#pragma unroll
-                for (int w = 0; w < 8; w++) n += __popc(mask[e][w]);
-            c[q] = n;
-            m[q] = (n + item_rows - 1) / item_rows;
-            cs += n;
-            ms += m[q];
-        }
-        int ci = cs, mi = ms;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int cv = __shfl_up_sync(kFull, ci, o), mv = __shfl_up_sync(kFull, mi, o);
-            if (lane >= o) {
-                ci += cv;
-                mi += mv;
-            }
-        }
-        int ce = ci - cs, me = mi - ms;
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-            off_s[lane * 8 + q] = ce;
-            item_s[lane * 8 + q] = me;
-            ce += c[q];
-            me += m[q];
-        }
-        if (lane == 31) {
-            off_s[kMaxExperts] = ci;
-            item_s[kMaxExperts] = mi;
-        }
-    }
-    __syncthreads();
-    if (tid < E) {
-        const int e = tid, o = off_s[e], n = off_s[e + 1] - o;
-        offsets[e] = o;
-        int it = item_s[e];
-        for (int a0 = 0; a0 < n; a0 += item_rows) items[it++] = WorkItem{e, o + a0, min(item_rows, n - a0), 0};
-    }
-    if (tid == 0) {
-        offsets[E] = off_s[kMaxExperts];
-        *n_items = item_s[kMaxExperts];
-    }
-    // bits[t][w]: bit i of word w = token t activated expert 32 w + i
-    for (int q = tid; q < T * 8; q += blockDim.x) {
-        const int t = q >> 3, w = q & 7;
-        uint32_t v = 0;
-        for (int i = 0; i < 32 && 32 * w + i < E; i++) v |= ((mask[32 * w + i][t >> 5] >> (t & 31)) & 1u) << i;
-        bits[(size_t)t * 8 + w] = v;
-    }
-    // scatter: the first entry of each (t, e) writes its slot, repeats add
-    // their gate afterwards
-    for (int pass = 0; pass < 2; pass++) {
-#pragma unroll
-        for (int i = 0; i < kTokPerWarp; i++) {
-            const int t = warp + 32 * i;
-            if (t >= T) break;
-            const int k = ck[i];
-            for (int r = lane; r < k; r += 32) {
-                const int e = r == lane ? ce[i] : ids[(size_t)t * E + r];
-                if (e < 0 || e >= E) continue;
-                const bool rep = (dup[t][r >> 5] >> (r & 31)) & 1u;
-                if (rep != (pass == 1)) continue;
-                int pos = off_s[e] + __popc(mask[e][t >> 5] & ((1u << (t & 31)) - 1u));
-                for (int w = 0; w < (t >> 5); w++) pos += __popc(mask[e][w]);
-                const float gv = r == lane ? cg[i] : gates[(size_t)t * E + r];
-                if (pass == 0) {
-                    perm_token[pos] = t;
-                    perm_gate[pos] = gv;
-                    invpos[(size_t)t * E + e] = pos;
-                } else {
-                    atomicAdd(&perm_gate[pos], gv);
-                }
-            }
-        }
-        __syncthreads();
     }
 }
 
@@ -720,17 +604,14 @@ __global__ void __launch_bounds__(kGuThreads, 1)
 PP_DEVINL bool jt_first_overflow(const WorkItem& w, long long ycap) { return (long long)w.a0 + w.cnt > ycap; }
 
 // ============================================================== grouped down
-// Persistent over (work item, column part) pairs: the njt 256-wide slices of
-// d are cut into nsub parts (more, smaller tasks than items when a batch is
-// small, so that every SM streams W_down); per task the H tile is loaded
-// once and the part's slices stream through the B ring.  Two 256-column
-// TMEM accumulators overlap the reduction epilogue with the next slice's
-// MMAs.
+// Persistent over work items: an item's H tile is loaded once and the njt
+// 256-wide slices of d stream through the B ring.  Two 256-column TMEM
+// accumulators overlap the reduction epilogue with the next slice's MMAs.
 __global__ void __launch_bounds__(kTcThreads, 1)
     down_gemm_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
                      const __grid_constant__ CUtensorMap map_y, const WorkItem* __restrict__ items,
                      const int* __restrict__ n_items_p,
-                     const int* __restrict__ perm_token, int d, int njt, int nsub, __nv_bfloat16* Y, long long ycap,
+                     const int* __restrict__ perm_token, int d, int njt, __nv_bfloat16* Y, long long ycap,
                      float* yacc, int* overflow, unsigned* status, uint64_t lim) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
@@ -743,13 +624,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __shared__ uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], afull, aempty;
     __shared__ uint32_t taddr_s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tasks = *n_items_p * nsub;
-    // slices [jt0, jt1) of task v (item v / nsub, part v % nsub)
-    auto slices = [&](int v, int& jt0, int& jt1) {
-        const int sp = v % nsub;
-        jt0 = sp * njt / nsub;
-        jt1 = (sp + 1) * njt / nsub;
-    };
+    const int n_items = *n_items_p;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; i++) {
             mbar_init(&full[i], 1);
@@ -775,14 +650,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (warp == 0) {
         if (lane == 0) {
             int it = 0, ii = 0;
-            for (int v = blockIdx.x; v < n_tasks; v += gridDim.x, ii++) {
-                const WorkItem w = items[v / nsub];
-                int jt0, jt1;
-                slices(v, jt0, jt1);
+            for (int v = blockIdx.x; v < n_items; v += gridDim.x, ii++) {
+                const WorkItem w = items[v];
                 if (ii >= 1) mbar_wait(&aempty, (uint32_t)(ii - 1) & 1u, status, lim);
                 mbar_arrive_expect_tx(&afull, kTileBytesA);
                 tma_load_2d(tileA, &map_h, 0, w.a0, &afull);
-                for (int jt = jt0; jt < jt1; jt++, it++) {
+                for (int jt = 0; jt < njt; jt++, it++) {
                     const int s = it % kStages;
                     if (it >= kStages) mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, status, lim);
                     mbar_arrive_expect_tx(&full[s], kTileB);
@@ -795,11 +668,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16_m128(256);
             int it = 0, acc = 0, ii = 0;
-            for (int v = blockIdx.x; v < n_tasks; v += gridDim.x, ii++) {
-                int jt0, jt1;
-                slices(v, jt0, jt1);
+            for (int v = blockIdx.x; v < n_items; v += gridDim.x, ii++) {
                 mbar_wait(&afull, (uint32_t)ii & 1u, status, lim);
-                for (int jt = jt0; jt < jt1; jt++, it++, acc++) {
+                for (int jt = 0; jt < njt; jt++, it++, acc++) {
                     const int a = acc & 1;
                     if (acc >= 2) mbar_wait(&tempty[a], (uint32_t)((acc >> 1) - 1) & 1u, status, lim);
                     const int s = it % kStages;
@@ -820,10 +691,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         // its 32 rows in the 128-byte swizzle (conflict-free row writes)
         unsigned char* stage = smem + kTileBytesA + (size_t)kStages * kTileB + (size_t)q * 16384;
         int acc = 0;
-        for (int v = blockIdx.x; v < n_tasks; v += gridDim.x) {
-            const WorkItem w = items[v / nsub];
-            int jt0, jt1;
-            slices(v, jt0, jt1);
+        for (int v = blockIdx.x; v < n_items; v += gridDim.x) {
+            const WorkItem w = items[v];
             const bool live = row < w.cnt;
             const bool group_live = 32 * q < w.cnt;  // any live row in this warp's 32 rows
             // all 32 rows live and inside Y: the group's rows go out as 2-D bulk stores
@@ -834,7 +703,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             float* yrow = tok >= 0 ? yacc + (size_t)tok * d : nullptr;
             if (tok >= 0 && jt_first_overflow(w, ycap)) *overflow = 1;
             __nv_bfloat16* Yrow = in_buf ? Y + (size_t)arow * d : nullptr;
-            for (int jt = jt0; jt < jt1; jt++, acc++) {
+            for (int jt = 0; jt < njt; jt++, acc++) {
                 const int a = acc & 1;
                 mbar_wait(&tfull[a], (uint32_t)(acc >> 1) & 1u, status, lim);
                 tc_fence_after();
@@ -909,299 +778,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// ========================================================== small batches
-// Operand-swapped grouped GEMMs for items of at most kSwN tokens (batches of
-// up to kSwapMaxT tokens, where an expert sees a few tokens): the weights are the
-// M = 128 operand and the item's tokens the N = kSwN operand.  A pipeline
-// stage is then 16 KB of weights + 2 KB of token rows (a 128-token tile would
-// spend half of every stage on padding rows), so about twice as many weight
-// bytes are in flight per SM.
-constexpr int kSwN = 16;
-constexpr int kSwapMaxT = 128;  // batches above this keep 128-row items (experts see more tokens)
-constexpr int kSwTileW = 128 * 128;   // 128 weight rows x 64 bf16
-constexpr int kSwTileX = kSwN * 128;  // kSwN token rows x 64 bf16
-
-// Gate/up (SwiGLU): D[128 x kSwN] = [64 gate rows; 64 up rows of expert e]
-// . x_tokens^T over K = d.  TMEM lanes 0-63 hold the gate sums of neurons
-// 0-63, lanes 64-127 the up sums; the warps reading the up lanes hand them to
-// the gate warps through shared memory, which write h = silu(g) * u * gate.
-__global__ void __launch_bounds__(kTcThreads, 1)
-    gu_swap_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_wg,
-                   const __grid_constant__ CUtensorMap map_wu, const WorkItem* __restrict__ items,
-                   const int* __restrict__ n_items_p, const int* __restrict__ perm_token,
-                   const float* __restrict__ perm_gate, int nk, __nv_bfloat16* H, unsigned* status, uint64_t lim) {
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    constexpr int kStages = 11;
-    constexpr int kStage = kSwTileW + kSwTileX;  // 18 KB, a multiple of 1024
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t full[kStages], empty[kStages], tfull[2], tempty[2];
-    __shared__ uint32_t taddr_s;
-    __shared__ float up_s[2][32][kSwN + 1];  // up sums of neurons 0-31 / 32-63 for the gate warps
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_items = *n_items_p;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; i++) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
-        }
-        for (int i = 0; i < 2; i++) {
-            mbar_init(&tfull[i], 1);
-            mbar_init(&tempty[i], 4);
-        }
-        fence_mbar_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(&taddr_s, 32);  // two kSwN-column accumulators
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = taddr_s;
-
-    if (warp == 0) {
-        int it = 0;
-        // the next item and its token rows are read one item ahead
-        WorkItem wn = blockIdx.x < n_items ? items[blockIdx.x] : WorkItem{0, 0, 1, 0};
-        int tokn = blockIdx.x < n_items ? perm_token[wn.a0 + min(lane & (kSwN - 1), wn.cnt - 1)] : 0;
-        for (int wi = blockIdx.x; wi < n_items; wi += gridDim.x) {
-            const WorkItem w = wn;
-            // lane i < kSwN: the item's i-th token row (padding repeats the last)
-            const int tok = tokn;
-            if (wi + (int)gridDim.x < n_items) {
-                wn = items[wi + gridDim.x];
-                tokn = perm_token[wn.a0 + min(lane & (kSwN - 1), wn.cnt - 1)];
-            }
-            const int ng = (w.cnt + 3) >> 2;  // gather4 groups of live rows
-            const int r0 = __shfl_sync(kFull, tok, (4 * lane) & 31), r1 = __shfl_sync(kFull, tok, (4 * lane + 1) & 31);
-            const int r2 = __shfl_sync(kFull, tok, (4 * lane + 2) & 31), r3 = __shfl_sync(kFull, tok, (4 * lane + 3) & 31);
-            for (int kc = 0; kc < nk; kc++, it++) {
-                const int s = it % kStages;
-                unsigned char* st = smem + (size_t)s * kStage;
-                if (lane == 0) {
-                    if (it >= kStages) mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, status, lim);
-                    mbar_arrive_expect_tx(&full[s], (uint32_t)(kSwTileW + ng * 512));
-                }
-                __syncwarp();
-                if (lane < ng) tma_gather4(st + kSwTileW + lane * 512, &map_x1, kc * 64, r0, r1, r2, r3, &full[s]);
-                if (lane == 0) {
-                    tma_load_2d(st, &map_wg, kc * 64, w.e * 64, &full[s]);
-                    tma_load_2d(st + 64 * 128, &map_wu, kc * 64, w.e * 64, &full[s]);
-                }
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16_m128(kSwN);
-            int it = 0, acc = 0;
-            for (int wi = blockIdx.x; wi < n_items; wi += gridDim.x, acc++) {
-                const int a = acc & 1;
-                if (acc >= 2) mbar_wait(&tempty[a], (uint32_t)((acc >> 1) - 1) & 1u, status, lim);
-                tc_fence_after();
-                for (int kc = 0; kc < nk; kc++, it++) {
-                    const int s = it % kStages;
-                    mbar_wait(&full[s], (uint32_t)(it / kStages) & 1u, status, lim);
-                    tc_fence_after();
-                    unsigned char* st = smem + (size_t)s * kStage;
-                    umma_k64(tmem + (uint32_t)(a * kSwN), st, st + kSwTileW, idesc, kc > 0);
-                    umma_commit(&empty[s]);
-                }
-                umma_commit(&tfull[a]);
-            }
-        }
-        __syncwarp();
-    } else {
-        const int q = warp & 3;  // TMEM lanes 32 q .. 32 q + 31
-        int acc = 0;
-        for (int wi = blockIdx.x; wi < n_items; wi += gridDim.x, acc++) {
-            const WorkItem w = items[wi];
-            const int a = acc & 1;
-            const float gw_l = lane < w.cnt ? perm_gate[w.a0 + lane] : 0.0f;  // gate weight of token `lane`
-            mbar_wait(&tfull[a], (uint32_t)(acc >> 1) & 1u, status, lim);
-            tc_fence_after();
-            uint32_t v[kSwN];
-            tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(a * kSwN), v);
-            tmem_ld_wait();
-            if (q >= 2) {
-#pragma unroll
-                for (int t = 0; t < kSwN; t++) up_s[q - 2][lane][t] = __uint_as_float(v[t]);
-            }
-            named_bar_sync(1, 128);
-            if (q < 2) {
-                const int n = 32 * q + lane;  // this lane's neuron
-#pragma unroll
-                for (int t = 0; t < kSwN; t++) {
-                    const float gw = __shfl_sync(kFull, gw_l, t);
-                    if (t < w.cnt) {
-                        const float h = act_h(PP_ACT_SWIGLU, up_s[q][lane][t], __uint_as_float(v[t])) * gw;
-                        H[(size_t)(w.a0 + t) * 64 + n] = __float2bfloat16_rn(h);
-                    }
-                }
-            }
-            named_bar_sync(1, 128);  // up_s is free for the next item
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[a]);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, 32);
-}
-
-// Down projection: per task (item, part of the ceil(d / 128) row tiles),
-// D[128 x kSwN] = W_down[128 rows, 64 columns of expert e] . H_item^T; the
-// item's kSwN H rows stay in shared memory for the task while the W_down
-// tiles stream through the ring (two H buffers, so that the next task's
-// tiles follow without a gap).  Lane = output row, column t = token: Y row
-// a0 + t (or, past ycap, a reduction into yacc) receives it.
-__global__ void __launch_bounds__(kTcThreads, 1)
-    down_swap_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
-                     const WorkItem* __restrict__ items, const int* __restrict__ n_items_p,
-                     const int* __restrict__ perm_token, int d, int nrt, int nsub, __nv_bfloat16* Y, long long ycap,
-                     float* yacc, int* overflow, unsigned* status, uint64_t lim) {
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    constexpr int kStages = 12;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    unsigned char* tileH = smem;                // 2 x kSwTileX bytes (1024-aligned)
-    unsigned char* ring = smem + 2 * 2048;      // kStages x kSwTileW
-    __shared__ uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], hfull[2], hempty[2];
-    __shared__ uint32_t taddr_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tasks = *n_items_p * nsub;
-    auto tiles = [&](int v, int& r0, int& r1) {  // row tiles [r0, r1) of task v
-        const int sp = v % nsub;
-        r0 = sp * nrt / nsub;
-        r1 = (sp + 1) * nrt / nsub;
-    };
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; i++) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
-        }
-        for (int i = 0; i < 2; i++) {
-            mbar_init(&tfull[i], 1);
-            mbar_init(&tempty[i], 4);
-        }
-        for (int i = 0; i < 2; i++) {
-            mbar_init(&hfull[i], 1);
-            mbar_init(&hempty[i], 1);
-        }
-        fence_mbar_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(&taddr_s, 32);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = taddr_s;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            int it = 0, ii = 0;
-            WorkItem wn = blockIdx.x < n_tasks ? items[blockIdx.x / nsub] : WorkItem{0, 0, 0, 0};
-            for (int v = blockIdx.x; v < n_tasks; v += gridDim.x, ii++) {
-                const WorkItem w = wn;
-                if (v + (int)gridDim.x < n_tasks) wn = items[(v + gridDim.x) / nsub];  // next task's item, early
-                int r0, r1;
-                tiles(v, r0, r1);
-                const int hb = ii & 1;
-                if (ii >= 2) mbar_wait(&hempty[hb], (uint32_t)((ii >> 1) - 1) & 1u, status, lim);
-                mbar_arrive_expect_tx(&hfull[hb], kSwTileX);
-                tma_load_2d(tileH + hb * 2048, &map_h, 0, w.a0, &hfull[hb]);
-                for (int rt = r0; rt < r1; rt++, it++) {
-                    const int s = it % kStages;
-                    if (it >= kStages) mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, status, lim);
-                    mbar_arrive_expect_tx(&full[s], kSwTileW);
-                    tma_load_2d(ring + (size_t)s * kSwTileW, &map_wd, w.e * 64, rt * 128, &full[s]);
-                }
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16_m128(kSwN);
-            int it = 0, acc = 0, ii = 0;
-            for (int v = blockIdx.x; v < n_tasks; v += gridDim.x, ii++) {
-                int r0, r1;
-                tiles(v, r0, r1);
-                const int hb = ii & 1;
-                mbar_wait(&hfull[hb], (uint32_t)(ii >> 1) & 1u, status, lim);
-                for (int rt = r0; rt < r1; rt++, it++, acc++) {
-                    const int a = acc & 1;
-                    if (acc >= 2) mbar_wait(&tempty[a], (uint32_t)((acc >> 1) - 1) & 1u, status, lim);
-                    const int s = it % kStages;
-                    mbar_wait(&full[s], (uint32_t)(it / kStages) & 1u, status, lim);
-                    tc_fence_after();
-                    umma_k64(tmem + (uint32_t)(a * kSwN), ring + (size_t)s * kSwTileW, tileH + hb * 2048, idesc,
-                             false);
-                    umma_commit(&empty[s]);
-                    umma_commit(&tfull[a]);
-                }
-                umma_commit(&hempty[hb]);
-            }
-        }
-        __syncwarp();
-    } else {
-        const int q = warp & 3;
-        int acc = 0;
-        for (int v = blockIdx.x; v < n_tasks; v += gridDim.x) {
-            const WorkItem w = items[v / nsub];
-            int r0, r1;
-            tiles(v, r0, r1);
-            // token of assignment row a0 + lane (for rows past ycap)
-            const long long arow_l = (long long)w.a0 + lane;
-            const int tok_l = lane < w.cnt && arow_l >= ycap ? perm_token[arow_l] : -1;
-            const bool spill = (long long)w.a0 + w.cnt > ycap;  // some of the item's rows go to yacc
-            if (lane == 0 && spill) *overflow = 1;
-            for (int rt = r0; rt < r1; rt++, acc++) {
-                const int a = acc & 1;
-                mbar_wait(&tfull[a], (uint32_t)(acc >> 1) & 1u, status, lim);
-                tc_fence_after();
-                uint32_t val[kSwN];
-                tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(a * kSwN), val);
-                tmem_ld_wait();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[a]);
-                const int row = rt * 128 + 32 * q + lane;  // output element of d
-                if (!spill) {  // every row of the item is kept: only its cnt columns are stored
-                    if (row < d) {
-                        __nv_bfloat16* yp = Y + (size_t)w.a0 * d + row;
-#pragma unroll
-                        for (int t = 0; t < kSwN; t++) {
-                            if (t >= w.cnt) break;
-                            yp[(size_t)t * d] = __float2bfloat16_rn(__uint_as_float(val[t]));
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int t = 0; t < kSwN; t++) {
-                        const int tk = __shfl_sync(kFull, tok_l, t);
-                        if (t < w.cnt && row < d) {
-                            const long long arow = (long long)w.a0 + t;
-                            if (arow < ycap)
-                                Y[(size_t)arow * d + row] = __float2bfloat16_rn(__uint_as_float(val[t]));
-                            else
-                                atomicAdd(&yacc[(size_t)tk * d + row], __uint_as_float(val[t]));
-                        }
-                    }
-                }
-            }
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, 32);
-}
-
 // =================================================================== combine
 // y[t] = the sum of token t's assignment rows Y[pos] in ascending expert
 // order, plus yacc[t] when the down projection overflowed (yacc is then
@@ -1265,62 +841,6 @@ __global__ void __launch_bounds__(128) combine_kernel(const uint32_t* __restrict
 // ====================================================================== host
 namespace {
 
-// Launch with programmatic dependent launch allowed: the kernel may be
-// scheduled while its predecessor on the stream finishes, and waits for it
-// in griddepcontrol.wait (pdl_wait) before touching memory.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-    if (e == cudaErrorNotSupported) {
-        (void)cudaGetLastError();
-        cfg.numAttrs = 0;
-        e = cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-    }
-    return e;
-}
-
-// Launch through launch_pdl; returns the error from the enclosing function.
-#define PP_LAUNCH(...)                                   \
-    do {                                                 \
-        const cudaError_t le_ = launch_pdl(__VA_ARGS__); \
-        if (le_ != cudaSuccess) return le_;              \
-    } while (0)
-
-
-// bf16 [outer][inner] row-major, SW128 boxes.  `promote` is the L2 fill
-// granularity: 256 B where the neighbouring 128 B of a row is read next by
-// the same CTA (K-major operand streams), 128 B where it belongs to another
-// expert that may not be selected (the 64-column blocks of W_down).
-bool encode_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer, uint32_t box_inner,
-               uint32_t box_outer, CUtensorMapL2promotion promote = CU_TENSOR_MAP_L2_PROMOTION_L2_256B) {
-    auto enc = tensor_map_encoder();
-    if (!enc) return false;
-    const cuuint64_t dims[2] = {inner, outer};
-    const cuuint64_t strides[1] = {inner * 2};
-    const cuuint32_t box[2] = {box_inner, box_outer};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, promote,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-template <typename K>
-cudaError_t set_smem(K kern, size_t bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-int router_ne(int E) { return E <= 32 ? 32 : E <= 64 ? 64 : E <= 128 ? 128 : E <= 160 ? 160 : E <= 192 ? 192 : E <= 224 ? 224 : 256; }
-
 template <int NE>
 cudaError_t launch_router(const CUtensorMap& mx, const CUtensorMap& mwr, int T, int E, int nk, int kpb, int nsplit,
                           float* part, unsigned* status, uint64_t lim, cudaStream_t st) {
@@ -1342,8 +862,7 @@ GroupedPlan grouped_plan(int T, int d, int E, int sms) {
     const int ns = std::max(1, std::min(sms / mt, std::min(g.nk / 4, 64)));
     g.kpb = (g.nk + ns - 1) / ns;
     g.nsplit = (g.nk + g.kpb - 1) / g.kpb;
-    const int rows = T <= kSwapMaxT ? kSwN : 128;  // rows per work item
-    g.max_items = (int)std::min<long long>((long long)T * E / rows + E + 1, (long long)T * E);
+    g.max_items = (int)std::min<long long>((long long)T * E / 128 + E + 1, (long long)T * E);  // 128-row items
     g.nnz_max = (long long)T * E;
     g.ycap = (long long)T * std::min(E, 64);  // assignment rows kept for the combine
     return g;
@@ -1367,66 +886,57 @@ cudaError_t grouped_route(const GroupedArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     if ((a.rule == PP_SEL_MIN_PREFIX || a.rule == PP_SEL_PAPER) && a.p < 1.0f) {
         PP_LAUNCH(select_part_cut_kernel, dim3(a.T), dim3(256), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                  a.gate, a.ids, a.counts, a.gates, a.logits_out, a.status);
+                  a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status);
         return cudaGetLastError();
     }
     if (a.T <= kCtaSelectMaxTokens) {
         PP_LAUNCH(select_part_cta_kernel, dim3(a.T), dim3(256), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-            a.gate, a.ids, a.counts, a.gates, a.logits_out, a.status);
+            a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status);
         return cudaGetLastError();
     }
     const dim3 grid((a.T + 7) / 8), block(256);
     switch (sel_slots_for(a.E)) {
         case 1: PP_LAUNCH(select_part_kernel<1>, dim3(grid), dim3(block), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.status); break;
+                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status); break;
         case 2: PP_LAUNCH(select_part_kernel<2>, dim3(grid), dim3(block), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.status); break;
+                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status); break;
         case 4: PP_LAUNCH(select_part_kernel<4>, dim3(grid), dim3(block), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.status); break;
+                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status); break;
         default: PP_LAUNCH(select_part_kernel<8>, dim3(grid), dim3(block), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.status); break;
+                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status); break;
     }
     return cudaGetLastError();
 }
 
+cudaError_t grouped_load_selection(const GroupedArgs& a, cudaStream_t st) {
+    PP_LAUNCH(dispatch_bits_kernel, dim3((a.T + 7) / 8), dim3(256), 0, st, a.ids, a.counts, a.gates, a.T, a.E, a.bits,
+              a.gexp, a.status);
+    return cudaGetLastError();
+}
+
 cudaError_t grouped_ffn(const GroupedArgs& a, int sms, cudaStream_t st) {
+    if (a.T <= kUnionMaxT) return union_layer(a, false, sms, st);
     const GroupedPlan& g = a.plan;
     const bool gated = a.act == PP_ACT_SWIGLU;
     cudaError_t e;
     // dispatch
-    if (a.T <= kSmallDispatchMaxT) {
-        PP_LAUNCH(dispatch_small_kernel, dim3(1), dim3(1024), 0, st, a.ids, a.counts, a.gates, a.T, a.E, a.bits,
-            a.offsets, reinterpret_cast<WorkItem*>(a.items), a.n_items, a.perm_token, a.perm_gate, a.invpos,
-            a.overflow, a.T <= kSwapMaxT ? kSwN : 128, a.status);
-    } else {
-        const int nblk = (a.T + kDispBlock - 1) / kDispBlock;
-        PP_LAUNCH(dispatch_bits_kernel, dim3((a.T + 7) / 8), dim3(256), 0, st, a.ids, a.counts, a.gates, a.T, a.E,
-            a.bits, a.gexp, a.status);
-        PP_LAUNCH(dispatch_count_kernel, dim3(nblk), dim3(kDispBlock), 0, st, a.bits, a.T, a.E, a.wcnt, a.blkcnt);
-        PP_LAUNCH(dispatch_scan_kernel, dim3(1), dim3(kMaxExperts), 0, st, a.blkcnt, nblk, a.E, a.offsets, a.blkbase,
-            reinterpret_cast<WorkItem*>(a.items), a.n_items, a.overflow);
-        PP_LAUNCH(dispatch_scatter_kernel, dim3(nblk, std::min(8, a.E)), dim3(kDispBlock), 0, st, a.bits, a.gexp, a.T, a.E, a.wcnt,
-            a.blkbase, a.perm_token, a.perm_gate, a.invpos);
-    }
+    const int nblk = (a.T + kDispBlock - 1) / kDispBlock;
+    PP_LAUNCH(dispatch_count_kernel, dim3(nblk), dim3(kDispBlock), 0, st, a.bits, a.T, a.E, a.wcnt, a.blkcnt);
+    PP_LAUNCH(dispatch_scan_kernel, dim3(1), dim3(kMaxExperts), 0, st, a.blkcnt, nblk, a.E, a.offsets, a.blkbase,
+              reinterpret_cast<WorkItem*>(a.items), a.n_items, a.overflow);
+    PP_LAUNCH(dispatch_scatter_kernel, dim3(nblk, std::min(8, a.E)), dim3(kDispBlock), 0, st, a.bits, a.gexp, a.T,
+              a.E, a.wcnt, a.blkbase, a.perm_token, a.perm_gate, a.invpos);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // grouped gate/up
-    CUtensorMap mx1, mwg, mwu, mh, mwd;
-    if (!encode_2d(&mx1, a.x, a.d, a.T, 64, 1) || !encode_2d(&mwu, a.Wu, a.d, (uint64_t)a.E * 64, 64, 64) ||
+    CUtensorMap mwg, mwu, mh, mwd;
+    if (!encode_2d(&mwu, a.Wu, a.d, (uint64_t)a.E * 64, 64, 64) ||
         !encode_2d(&mwg, gated ? a.Wg : a.Wu, a.d, (uint64_t)a.E * 64, 64, 64) ||
         !encode_2d(&mh, a.H, 64, (uint64_t)g.nnz_max + 128, 64, 128) ||
         !encode_2d(&mwd, a.Wd, (uint64_t)a.E * 64, a.d, 64, 256, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
         return cudaErrorInvalidValue;
     const int grid = std::max(1, std::min(sms, g.max_items));
     const WorkItem* items = reinterpret_cast<const WorkItem*>(a.items);
-    // batches of up to kSwapMaxT tokens: items of at most kSwN rows and the
-    // operand-swapped kernels (weights as the M = 128 operand)
-    const bool small = a.T <= kSwapMaxT;
-    if (gated && small) {
-        const size_t smem = 11 * (size_t)(kSwTileW + kSwTileX) + 1024;
-        if ((e = set_smem(gu_swap_kernel, smem)) != cudaSuccess) return e;
-        PP_LAUNCH(gu_swap_kernel, dim3(grid), dim3(kTcThreads), smem, st, mx1, mwg, mwu, items, a.n_items,
-            a.perm_token, a.perm_gate, g.nk, a.H, a.status, a.timeout_ns);
-    } else if (gated) {
+    if (gated) {
         const size_t smem = 6 * (size_t)(kTileBytesA + 128 * 128) + 1024;
         if ((e = set_smem(gu_gemm_kernel<128>, smem)) != cudaSuccess) return e;
         PP_LAUNCH(gu_gemm_kernel<128>, dim3(grid), dim3(kGuThreads), smem, st,
@@ -1440,37 +950,14 @@ cudaError_t grouped_ffn(const GroupedArgs& a, int sms, cudaStream_t st) {
             g.nk, a.act, a.H, a.status, a.timeout_ns);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // grouped down + scatter-add
-    if (small) {
-        CUtensorMap mh16, mwd128;
-        if (!encode_2d(&mh16, a.H, 64, (uint64_t)g.nnz_max + 128, 64, kSwN) ||
-            !encode_2d(&mwd128, a.Wd, (uint64_t)a.E * 64, a.d, 64, 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
-            return cudaErrorInvalidValue;
-        const size_t smem = 2 * 2048 + 12 * (size_t)kSwTileW + 1024;
-        if ((e = set_smem(down_swap_kernel, smem)) != cudaSuccess) return e;
-        // each item's ceil(d / 128) row tiles cut into up to 4 tasks, so that
-        // every SM streams W_down
-        const int nrt = (a.d + 127) / 128;
-        const int nsub = std::min(4, nrt);
-        const int grid6 = std::max(1, (int)std::min<long long>(sms, (long long)g.max_items * nsub));
-        PP_LAUNCH(down_swap_kernel, dim3(grid6), dim3(kTcThreads), smem, st, mh16, mwd128, items, a.n_items,
-            a.perm_token, a.d, nrt, nsub, a.Y, g.ycap, a.yacc, a.overflow, a.status, a.timeout_ns);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    } else {
-        // A tile, the 4-stage W_down ring, 4 x 16 KB store staging
-        const size_t smem = (size_t)kTileBytesA + 4 * (size_t)256 * 128 + 4 * (size_t)16384 + 1024;
-        CUtensorMap my;
-        if (!encode_2d(&my, a.Y, a.d, (uint64_t)g.ycap, 64, 32)) return cudaErrorInvalidValue;
-        if ((e = set_smem(down_gemm_kernel, smem)) != cudaSuccess) return e;
-        // up to 256 tokens: about one 128-row item per expert, fewer than the
-        // SMs can share evenly, so each item's columns are cut into 4 tasks
-        const int njt = (a.d + 255) / 256;
-        const int nsub = a.T <= kSmallDispatchMaxT ? std::min(4, njt) : 1;
-        const int grid6 = std::max(1, (int)std::min<long long>(sms, (long long)g.max_items * nsub));
-        PP_LAUNCH(down_gemm_kernel, dim3(grid6), dim3(kTcThreads), smem, st, mh, mwd, my, items, a.n_items, a.perm_token,
-            a.d, njt, nsub, a.Y, g.ycap, a.yacc, a.overflow, a.status, a.timeout_ns);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    // grouped down: A tile, the 4-stage W_down ring, 4 x 16 KB store staging
+    const size_t smem = (size_t)kTileBytesA + 4 * (size_t)256 * 128 + 4 * (size_t)16384 + 1024;
+    CUtensorMap my;
+    if (!encode_2d(&my, a.Y, a.d, (uint64_t)g.ycap, 64, 32)) return cudaErrorInvalidValue;
+    if ((e = set_smem(down_gemm_kernel, smem)) != cudaSuccess) return e;
+    PP_LAUNCH(down_gemm_kernel, dim3(grid), dim3(kTcThreads), smem, st, mh, mwd, my, items, a.n_items, a.perm_token, a.d,
+              (a.d + 255) / 256, a.Y, g.ycap, a.yacc, a.overflow, a.status, a.timeout_ns);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     PP_LAUNCH(combine_kernel, dim3(a.T, (a.d + 1023) / 1024), dim3(128), 0, st, a.bits, a.invpos, a.Y, g.ycap,
         a.yacc, a.overflow, a.T, a.E, a.d, reinterpret_cast<__nv_bfloat16*>(a.y));
     return cudaGetLastError();

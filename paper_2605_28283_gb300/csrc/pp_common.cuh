@@ -28,7 +28,9 @@ constexpr int kMaxGrid = 256;  // CTAs of a fused decode launch (one per SM)
 struct Control {
     unsigned status;           // sticky pp_status of the device side
     unsigned wait_flag;        // never written: target of pp_debug_wait_timeout
-    unsigned pad[62];
+    unsigned pad[30];
+    unsigned long long bar;    // grid barrier arrivals of the union kernel
+    unsigned pad2[30];
     unsigned epoch[kMaxGrid];  // launches of the fused decode kernel seen by CTA b
 };
 static_assert(sizeof(Control) == 1280, "control block is 1280 bytes");
@@ -143,6 +145,11 @@ PP_DEVINL void named_bar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Arrive on a named barrier without waiting for it.
+PP_DEVINL void named_bar_arrive(int id, int nthreads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
 // ---------------------------------------------------------- tagged words
 PP_DEVINL unsigned ld_acquire_gpu(const unsigned* p) {
     unsigned v;
@@ -208,6 +215,38 @@ PP_DEVINL float wait_tagged(const unsigned long long* p, unsigned tag, unsigned*
     }
     return word_value(w);
 }
+
+// --------------------------------------------------------------- grid barrier
+// Barrier of all CTAs of a cooperative launch on one 64-bit arrival counter
+// (it only grows: every launch adds a multiple of its CTA count).  One thread
+// of a CTA reads the counter once, early in the launch (grid_bar_base), and
+// keeps the target of the next barrier; an arrival is one reduction without a
+// reply, and the waiters poll the counter itself.  What the CTA wrote before
+// its arrival (and a barrier of the CTA) is visible to what it reads after the
+// wait.  Waits are bounded.
+PP_DEVINL unsigned long long grid_bar_base(const unsigned long long* count, unsigned nctas) {
+    const unsigned long long v = ld_relaxed_u64(count);
+    return v - v % nctas;  // at most nctas - 1 of this launch's CTAs have arrived so far
+}
+
+PP_DEVINL void grid_arrive(unsigned long long* count) {
+    asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(count) : "memory");
+}
+
+PP_DEVINL bool grid_wait(const unsigned long long* count, unsigned long long target, unsigned* status,
+                         uint64_t limit_ns) {
+    uint64_t t0 = 0;
+    while (true) {
+        unsigned long long v;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
+        if (v >= target) return true;
+        if (poll_give_up(t0, status, limit_ns)) return false;
+    }
+}
+
+// Order generic-proxy accesses of global memory before it with async-proxy
+// (TMA) accesses after it.
+PP_DEVINL void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // ------------------------------------------------------------------- bf16
 PP_DEVINL float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }

@@ -163,14 +163,32 @@ struct GroupedArgs {
     __nv_bfloat16* H;   // [nnz_max + 128][64]
     __nv_bfloat16* Y;   // [ycap][d] assignment outputs
     float* yacc;        // [T][d] overflow accumulator, zero at rest
+    float* dpart;       // partial down-projection tiles (union path)
     int* overflow;      // set when any assignment went to yacc
+    unsigned long long* bar;  // grid barrier counter (union path)
     unsigned* status;
     uint64_t timeout_ns;
 };
 
+// -------------------------------------- union path (up to kUnionMaxT tokens)
+constexpr int kUnionMaxT = 256;
+constexpr int kUnionMaxGrid = 152;
+size_t union_part_floats(int T, int d);  // of GroupedArgs.dpart
+
 GroupedPlan grouped_plan(int T, int d, int E, int sms);
 cudaError_t grouped_route(const GroupedArgs& a, cudaStream_t st);
+// The FFN over a.bits / a.gexp (the selection as the FFN kernels read it,
+// written by grouped_route, or by grouped_load_selection from a.ids, a.counts
+// and a.gates).
+cudaError_t grouped_load_selection(const GroupedArgs& a, cudaStream_t st);
 cudaError_t grouped_ffn(const GroupedArgs& a, int sms, cudaStream_t st);
+// The whole layer (do_route), or the FFN alone over a.bits / a.gexp, in one
+// cooperative launch; a.T <= kUnionMaxT.  a.ids, a.counts, a.gates may be NULL.
+cudaError_t union_layer(const GroupedArgs& a, bool do_route, int sms, cudaStream_t st);
+// Columns of the router's MMA for E experts.
+inline int router_ne(int E) {
+    return E <= 32 ? 32 : E <= 64 ? 64 : E <= 128 ? 128 : E <= 160 ? 160 : E <= 192 ? 192 : E <= 224 ? 224 : 256;
+}
 
 // ------------------------------------------------ MoEfication (Sec. 2.2)
 // Balanced k-means over the neurons' input weights (host, offline); shapes

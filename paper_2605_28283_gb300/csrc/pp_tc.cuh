@@ -115,6 +115,11 @@ PP_DEVINL void tma_gather4(void* dst, const CUtensorMap* map, int col, int r0, i
         : "memory");
 }
 
+// Fetch a tensor map (a kernel parameter) ahead of its first use.
+PP_DEVINL void tma_prefetch_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 // 16-byte cp.async global -> shared through L2 (not L1); src_bytes = 0
 // writes 16 zero bytes instead of reading.  Completion: cp_async_commit
 // closes a group, cp_async_wait<N> waits until at most N groups are pending.
