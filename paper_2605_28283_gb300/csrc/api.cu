@@ -56,6 +56,8 @@ struct Layout {
     // grouped path
     size_t part, bits, gexp, invpos, wcnt, blkcnt, blkbase, offsets, n_items, items, perm_token, perm_gate, H, Y,
         yacc, overflow, dpart;
+    // fp32 calls of more tokens than a fused decode launch takes (bits and gexp too)
+    size_t h32;
     size_t total;
 };
 
@@ -96,6 +98,11 @@ Layout layout(const pp_desc& d, int T) {
         L.yacc = take(Tn * (size_t)d.d_model * 4);
         L.overflow = take(16);
         L.dpart = take(union_part_floats((int)Tn, d.d_model) * 4);
+    }
+    if (d.dtype == PP_F32) {
+        L.bits = take(Tn * 8 * 4);
+        L.gexp = take(Tn * E * 4);
+        L.h32 = take((size_t)std::min<size_t>(Tn, kFfn32Slice) * E * kDExpert * 4);
     }
     L.total = off;
     return L;
@@ -167,6 +174,9 @@ struct Ws {
     float* gates;
     unsigned long long* tlog;
     unsigned long long* th;
+    uint32_t* bits;  // fp32
+    float* gexp;     // fp32
+    float* h32;      // fp32
 };
 
 Ws ws_views(const pp_desc& d, int T, void* ws) {
@@ -175,7 +185,8 @@ Ws ws_views(const pp_desc& d, int T, void* ws) {
     return Ws{reinterpret_cast<Control*>(b), reinterpret_cast<float*>(b + L.logits),
               reinterpret_cast<int32_t*>(b + L.ids), reinterpret_cast<int32_t*>(b + L.counts),
               reinterpret_cast<float*>(b + L.gates), reinterpret_cast<unsigned long long*>(b + L.tlog),
-              reinterpret_cast<unsigned long long*>(b + L.th)};
+              reinterpret_cast<unsigned long long*>(b + L.th), reinterpret_cast<uint32_t*>(b + L.bits),
+              reinterpret_cast<float*>(b + L.gexp), reinterpret_cast<float*>(b + L.h32)};
 }
 
 bool make_down_map(const pp_desc& d, const void* Wd, int R6, CUtensorMap* map) {
@@ -332,6 +343,34 @@ pp_status decode_call(const pp_desc& d, const void* x, int t0, int n, const void
     return cuda_status(decode_launch(a, plan, d.dtype, TS, di.sms, st));
 }
 
+RouteArgs route_args(const pp_desc& d, const void* x, int T, const void* Wr, float kp, const pp_selection& s, const Ws& w,
+                     bool for_ffn32) {
+    return RouteArgs{x,        Wr,      T,        d.d_model,  d.n_experts, d.rule,
+                     d.gate,   kp,      s.ids,    s.counts,   s.gates,     s.logits,
+                     for_ffn32 ? w.bits : nullptr, for_ffn32 ? w.gexp : nullptr, &w.ctrl->status};
+}
+
+// The fp32 FFN of T tokens over w.gexp, kFfn32Slice tokens at a time.
+pp_status ffn32_call(const pp_desc& d, const void* x, int T, const void* Wg, const void* Wu, const void* Wd, void* y,
+                     const Ws& w, cudaStream_t st) {
+    for (int t0 = 0; t0 < T; t0 += kFfn32Slice) {
+        Ffn32Args a{};
+        a.x = static_cast<const float*>(x) + (size_t)t0 * d.d_model;
+        a.Wg = static_cast<const float*>(Wg);
+        a.Wu = static_cast<const float*>(Wu);
+        a.Wd = static_cast<const float*>(Wd);
+        a.gexp = w.gexp + (size_t)t0 * d.n_experts;
+        a.h = w.h32;
+        a.y = static_cast<float*>(y) + (size_t)t0 * d.d_model;
+        a.T = std::min(kFfn32Slice, T - t0);
+        a.d = d.d_model;
+        a.E = d.n_experts;
+        a.act = d.act;
+        PP_TRY(cuda_status(ffn32(a, st)));
+    }
+    return PP_OK;
+}
+
 }  // namespace
 
 float rule_kernel_param(int rule, float p, int E) {
@@ -425,10 +464,7 @@ pp_status pp_route(const pp_desc* desc, const void* x, int T, const void* W_r, f
     if (ts == 0) return PP_ERR_SHAPE;
     if (T <= ts)
         return decode_call(*desc, x, 0, T, W_r, nullptr, nullptr, nullptr, kp, out, true, false, nullptr, w, st);
-    float* lg = out->logits ? out->logits : w.logits;
-    PP_TRY(cuda_status(router_launch(desc->dtype, x, T, desc->d_model, W_r, desc->n_experts, lg, st)));
-    return cuda_status(select_launch(lg, T, desc->n_experts, kp, desc->rule, desc->gate, out->ids, out->counts,
-                                     out->gates, &w.ctrl->status, st));
+    return cuda_status(route_tokens(desc->dtype, route_args(*desc, x, T, W_r, kp, *out, w, false), st));
 }
 
 pp_status pp_sparse_ffn(const pp_desc* desc, const void* x, int T, const void* W_gate, const void* W_up,
@@ -452,6 +488,19 @@ pp_status pp_sparse_ffn(const pp_desc* desc, const void* x, int T, const void* W
     }
     const int ts = decode_ts_limit(*desc);
     if (ts == 0) return PP_ERR_SHAPE;
+    if (desc->dtype == PP_F32 && T > ts) {
+        GroupedArgs a{};
+        a.ids = sel->ids;
+        a.counts = sel->counts;
+        a.gates = sel->gates;
+        a.T = T;
+        a.E = desc->n_experts;
+        a.bits = w.bits;
+        a.gexp = w.gexp;
+        a.status = &w.ctrl->status;
+        PP_TRY(cuda_status(grouped_load_selection(a, st)));
+        return ffn32_call(*desc, x, T, W_gate, W_up, W_down, y, w, st);
+    }
     for (int t0 = 0; t0 < T; t0 += ts) {
         const int n = std::min(ts, T - t0);
         PP_TRY(decode_call(*desc, x, t0, n, nullptr, W_gate, W_up, W_down, 0.0f, sel, false, true, y, w, st));
@@ -492,10 +541,16 @@ pp_status pp_layer(const pp_desc* desc, const void* x, int T, const void* W_r, c
     if (ts == 0) return PP_ERR_SHAPE;
     if (T <= ts)
         return decode_call(*desc, x, 0, T, W_r, W_gate, W_up, W_down, kp, sel_out, true, true, y, w, st);
-    float* lg = s.logits ? s.logits : w.logits;
-    PP_TRY(cuda_status(router_launch(desc->dtype, x, T, desc->d_model, W_r, desc->n_experts, lg, st)));
-    PP_TRY(cuda_status(select_launch(lg, T, desc->n_experts, kp, desc->rule, desc->gate, s.ids, s.counts, s.gates,
-                                     &w.ctrl->status, st)));
+    if (desc->dtype == PP_F32) {
+        RouteArgs r = route_args(*desc, x, T, W_r, kp, s, w, true);
+        if (!sel_out) {  // nobody reads the rank order
+            r.ids = r.counts = nullptr;
+            r.gates = nullptr;
+        }
+        PP_TRY(cuda_status(route_tokens(desc->dtype, r, st)));
+        return ffn32_call(*desc, x, T, W_gate, W_up, W_down, y, w, st);
+    }
+    PP_TRY(cuda_status(route_tokens(desc->dtype, route_args(*desc, x, T, W_r, kp, s, w, false), st)));
     for (int t0 = 0; t0 < T; t0 += ts) {
         const int n = std::min(ts, T - t0);
         PP_TRY(decode_call(*desc, x, t0, n, nullptr, W_gate, W_up, W_down, 0.0f, &s, false, true, y, w, st));

@@ -125,9 +125,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 }
 
 // ================================================================= selection
-// Selection from K-split partial logits (summed in split order).  Up to
-// kCtaSelectMaxTokens tokens take one CTA each (the counting selection);
-// beyond, one warp per token (the warp sort).
+// Selection from K-split partial logits (summed in split order).  The
+// cumulative-mass cut, and the other rules up to kCtaSelectMaxTokens tokens,
+// take one CTA per token; the others one warp per token (the warp sort).
 constexpr int kCtaSelectMaxTokens = 256;
 
 // Logit = sum over s of part[s * stride + off], added in split order; the
@@ -198,67 +198,20 @@ __global__ void __launch_bounds__(256) select_part_kernel(const float* __restric
         for (int j = lane; j < E; j += 32) logits_out[(size_t)t * E + j] = load(j);
 }
 
+// One CTA per token.
 __global__ void __launch_bounds__(256) select_part_cta_kernel(const float* __restrict__ part, int nsplit, int T,
                                                               int E, float p, int rule, int gate, int32_t* ids,
                                                               int32_t* counts, float* gates, float* logits_out,
                                                               uint32_t* bits, float* gexp, unsigned* status) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
-    __shared__ __align__(16) CtaSelScratch sc;
+    __shared__ __align__(16) SelScratch sc;
     const int t = blockIdx.x;
-    auto load = [&](int j) { return sum_partials(part, nsplit, (size_t)T * E, (size_t)t * E + j); };
-    bool on;
-    int r;
-    float g;
-    const int k = cta_select_fn(load, E, p, rule, true, sc, status, &on, &r, &g);
-    const int j = threadIdx.x;
-    const float gv = on ? (gate == PP_GATE_NONE ? 1.0f : sigmoidf_(g)) : 0.0f;
-    write_selection_row(ids + (size_t)t * E, gates + (size_t)t * E, j, E, k, on, r, gv);
-    if (bits) {
-        const unsigned bal = __ballot_sync(kFull, on);
-        if ((j & 31) == 0) bits[(size_t)t * 8 + (j >> 5)] = bal;
-        if (j < E) gexp[(size_t)t * E + j] = gv;
-    }
-    if (j < E && logits_out) logits_out[(size_t)t * E + j] = g;
-    if (j == 0) counts[t] = k;
-}
-
-// Cumulative-mass cut (MIN_PREFIX / PAPER with p < 1) of any number of
-// tokens: one CTA per token runs the three-barrier cut of the fused decode
-// kernel on the summed partial logits.
-__global__ void __launch_bounds__(256) select_part_cut_kernel(const float* __restrict__ part, int nsplit, int T, int E,
-                                                              float p, int rule, int gate, int32_t* ids,
-                                                              int32_t* counts, float* gates, float* logits_out,
-                                                              uint32_t* bits, float* gexp, unsigned* status) {
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    __shared__ __align__(16) CutShared sc;
-    __shared__ __align__(16) WarpCand cand[256];
-    __shared__ float gx[256];     // gate weight per expert
-    __shared__ uint32_t bw[8];    // activated experts
-    const int t = blockIdx.x, j = threadIdx.x;
-    gx[j] = 0.0f;  // ordered before the cut's writes by its barriers
-    if (j < 8) bw[j] = 0u;
-    const float g = j < E ? sum_partials(part, nsplit, (size_t)T * E, (size_t)t * E + j) : -INFINITY;
-    int32_t* idr = ids + (size_t)t * E;
-    float* gtr = gates + (size_t)t * E;
-    const int k = cta_mass_cut(g, E, p, rule, sc, cand, status, [&](int r, int e, float ge) {
-        const float gv = gate == PP_GATE_NONE ? 1.0f : sigmoidf_(ge);
-        idr[r] = e;
-        gtr[r] = gv;
-        gx[e] = gv;
-        atomicOr(&bw[e >> 5], 1u << (e & 31));
-    }, [] {});  // its last barrier orders gx and bw before the reads below
-    if (bits) {
-        if (j < 8) bits[(size_t)t * 8 + j] = bw[j];
-        if (j < E) gexp[(size_t)t * E + j] = gx[j];
-    }
-    for (int r = k + j; r < E; r += 256) {
-        idr[r] = -1;
-        gtr[r] = 0.0f;
-    }
-    if (j < E && logits_out) logits_out[(size_t)t * E + j] = g;
-    if (j == 0) counts[t] = k;
+    const size_t row = (size_t)t * E;
+    const SelOut o{ids + row, counts + t, gates + row, logits_out ? logits_out + row : nullptr,
+                   bits ? bits + (size_t)t * 8 : nullptr, gexp + row};
+    select_token_cta([&](int j) { return sum_partials(part, nsplit, (size_t)T * E, row + j); }, E, p, rule, gate, sc, o,
+                     status);
 }
 
 // ================================================================== dispatch
@@ -884,12 +837,8 @@ cudaError_t grouped_route(const GroupedArgs& a, cudaStream_t st) {
         default: e = launch_router<256>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, a.status, a.timeout_ns, st); break;
     }
     if (e != cudaSuccess) return e;
-    if ((a.rule == PP_SEL_MIN_PREFIX || a.rule == PP_SEL_PAPER) && a.p < 1.0f) {
-        PP_LAUNCH(select_part_cut_kernel, dim3(a.T), dim3(256), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                  a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status);
-        return cudaGetLastError();
-    }
-    if (a.T <= kCtaSelectMaxTokens) {
+    const bool mass_cut = (a.rule == PP_SEL_MIN_PREFIX || a.rule == PP_SEL_PAPER) && a.p < 1.0f;
+    if (mass_cut || a.T <= kCtaSelectMaxTokens) {
         PP_LAUNCH(select_part_cta_kernel, dim3(a.T), dim3(256), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
             a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status);
         return cudaGetLastError();

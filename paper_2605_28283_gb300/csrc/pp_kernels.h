@@ -109,8 +109,30 @@ cudaError_t decode_launch(const DecodeArgs& a, const DecodePlan& p, int dtype, i
 int decode_max_ts(int dtype);
 
 // --------------------------------------------------------- route / select
-cudaError_t router_launch(int dtype, const void* x, int T, int d, const void* Wr, int E,
-                          float* logits, cudaStream_t st);
+// Logits and selection of T tokens on the CUDA cores; any output may be NULL
+// (ids and gates, and bits and gexp, only together).
+struct RouteArgs {
+    const void* x;
+    const void* Wr;
+    int T, d, E, rule, gate;
+    float p;
+    int32_t* ids;
+    int32_t* counts;
+    float* gates;
+    float* logits;
+    uint32_t* bits;
+    float* gexp;
+    unsigned* status;
+};
+cudaError_t route_tokens(int dtype, const RouteArgs& a, cudaStream_t st);
+// fp32 FFN of T tokens over gexp [T][E] (gate weights, 0: not selected).
+struct Ffn32Args {
+    const float *x, *Wg, *Wu, *Wd, *gexp;
+    float *h, *y;  // h: [T][E * 64] scratch
+    int T, d, E, act;
+};
+constexpr int kFfn32Slice = 1024;  // tokens of a call's scratch; more run in slices
+cudaError_t ffn32(const Ffn32Args& a, cudaStream_t st);
 cudaError_t select_launch(const float* logits, int T, int E, float p, int rule, int gate,
                           int32_t* ids, int32_t* counts, float* gates, unsigned* status,
                           cudaStream_t st);

@@ -597,4 +597,73 @@ PP_DEVINL void write_selection_row(int32_t* ids, float* gates, int j, int E, int
     }
 }
 
+// ---------------------------------------------------------------------------
+// The whole selection of one token by a CTA of 256 threads, written in both
+// forms: rank order for the caller (ids, counts, gates, logits: the token's
+// rows, each may be NULL but ids and gates only together) and per expert for
+// the FFN kernels (bits: E bits in 8 words; gexp: the gate weight, 0 where the
+// expert is not activated; NULL when no FFN follows).  `load(j)` returns logit
+// j.  The cumulative-mass rules below p = 1 take the three-barrier cut, the
+// others the counting selection.
+struct SelOut {
+    int32_t* ids;
+    int32_t* count;
+    float* gates;
+    float* logits;
+    uint32_t* bits;
+    float* gexp;
+};
+
+struct SelScratch {
+    CutShared cut;
+    __align__(16) WarpCand cand[256];
+    CtaSelScratch sel;
+    float gx[256];    // gate weight per expert
+    uint32_t bw[8];   // activated experts
+};
+
+template <typename Load>
+PP_DEVINL void select_token_cta(Load load, int E, float p, int rule, int gate, SelScratch& s, const SelOut& o,
+                                unsigned* status) {
+    const int j = threadIdx.x;
+    float g;
+    int k;
+    s.gx[j] = 0.0f;  // ordered before the selection's writes by its barriers
+    if (j < 8) s.bw[j] = 0u;
+    if ((rule == PP_SEL_MIN_PREFIX || rule == PP_SEL_PAPER) && p < 1.0f) {
+        g = j < E ? load(j) : -INFINITY;
+        k = cta_mass_cut(g, E, p, rule, s.cut, s.cand, status, [&](int r, int e, float ge) {
+            const float gv = gate == PP_GATE_NONE ? 1.0f : sigmoidf_(ge);
+            if (o.ids) {
+                o.ids[r] = e;
+                o.gates[r] = gv;
+            }
+            s.gx[e] = gv;
+            atomicOr(&s.bw[e >> 5], 1u << (e & 31));
+        }, [] {});  // its last barrier orders gx and bw before the reads below
+        if (o.ids)
+            for (int r = k + j; r < E; r += 256) {
+                o.ids[r] = -1;
+                o.gates[r] = 0.0f;
+            }
+    } else {
+        bool on;
+        int r;
+        k = cta_select_fn(load, E, p, rule, o.ids != nullptr, s.sel, status, &on, &r, &g);
+        const float gv = on ? (gate == PP_GATE_NONE ? 1.0f : sigmoidf_(g)) : 0.0f;
+        if (o.ids) write_selection_row(o.ids, o.gates, j, E, k, on, r, gv);
+        if (on) {
+            s.gx[j] = gv;
+            atomicOr(&s.bw[j >> 5], 1u << (j & 31));
+        }
+        __syncthreads();
+    }
+    if (o.bits) {
+        if (j < 8) o.bits[j] = s.bw[j];
+        if (j < E) o.gexp[j] = s.gx[j];
+    }
+    if (j < E && o.logits) o.logits[j] = g;
+    if (j == 0 && o.count) *o.count = k;
+}
+
 }  // namespace pp

@@ -1,4 +1,4 @@
-// Router logits for many tokens, stand-alone selection, sparsity statistics
+// Stand-alone selection, sparsity statistics
 // and the bounded-wait test kernel.
 #include "pp_common.cuh"
 #include "pp_kernels.h"
@@ -68,65 +68,6 @@ cudaError_t select_launch(const float* logits, int T, int E, float p, int rule, 
         case 4: select_kernel<4><<<grid, block, 0, st>>>(logits, T, E, p, rule, gate, ids, counts, gates, status); break;
         default: select_kernel<8><<<grid, block, 0, st>>>(logits, T, E, p, rule, gate, ids, counts, gates, status); break;
     }
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- router
-// logits[t][j] = sum_i W_r[j][i] * x[t][i] (Eq. routing_logits) for any T,
-// fp32 FMA on CUDA cores.  A CTA computes a 64-token x 32-expert tile,
-// staging 32-wide k slices of x and W_r in shared memory as fp32.
-constexpr int kRT = 64, kRE = 32, kRK = 32;
-
-template <typename TW>
-__global__ void __launch_bounds__(256) router_kernel(const TW* __restrict__ x, int T, int d,
-                                                     const TW* __restrict__ Wr, int E,
-                                                     float* __restrict__ logits) {
-    __shared__ float xs[kRK][kRT + 1];
-    __shared__ float ws[kRK][kRE + 1];
-    const int t0 = blockIdx.x * kRT, j0 = blockIdx.y * kRE;
-    const int tid = threadIdx.x;
-    const int tj = tid & 31;        // expert within tile
-    const int tt = (tid >> 5) * 8;  // 8 tokens per thread
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int k0 = 0; k0 < d; k0 += kRK) {
-        for (int i = tid; i < kRK * kRT; i += 256) {
-            const int kk = i % kRK, r = i / kRK;
-            const int t = t0 + r;
-            xs[kk][r] = (t < T && k0 + kk < d) ? (float)x[(size_t)t * d + k0 + kk] : 0.0f;
-        }
-        for (int i = tid; i < kRK * kRE; i += 256) {
-            const int kk = i % kRK, r = i / kRK;
-            const int j = j0 + r;
-            ws[kk][r] = (j < E && k0 + kk < d) ? (float)Wr[(size_t)j * d + k0 + kk] : 0.0f;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < kRK; kk++) {
-            const float w = ws[kk][tj];
-#pragma unroll
-            for (int q = 0; q < 8; q++) acc[q] = fmaf(w, xs[kk][tt + q], acc[q]);
-        }
-        __syncthreads();
-    }
-    const int j = j0 + tj;
-    if (j < E)
-        for (int q = 0; q < 8; q++) {
-            const int t = t0 + tt + q;
-            if (t < T) logits[(size_t)t * E + j] = acc[q];
-        }
-}
-
-cudaError_t router_launch(int dtype, const void* x, int T, int d, const void* Wr, int E,
-                          float* logits, cudaStream_t st) {
-    if (T == 0) return cudaSuccess;
-    const dim3 grid((T + kRT - 1) / kRT, (E + kRE - 1) / kRE), block(256);
-    if (dtype == PP_BF16)
-        router_kernel<__nv_bfloat16><<<grid, block, 0, st>>>(
-            reinterpret_cast<const __nv_bfloat16*>(x), T, d, reinterpret_cast<const __nv_bfloat16*>(Wr), E,
-            logits);
-    else
-        router_kernel<float><<<grid, block, 0, st>>>(reinterpret_cast<const float*>(x), T, d,
-                                                     reinterpret_cast<const float*>(Wr), E, logits);
     return cudaGetLastError();
 }
 

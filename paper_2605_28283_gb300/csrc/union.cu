@@ -198,23 +198,14 @@ PP_DEVINL void router_phase(const UnionArgs& a, UnionShared& sh, unsigned char* 
     if (tid == 32 * kHWarp) sh.bar_target = grid_bar_base(a.bar, gridDim.x);
 }
 
-// Selection of tokens b, b + G, ... from the summed partial logits, in rank
-// order for the caller (where wanted) and as bits / gexp for the FFN.
+// Selection of tokens b, b + G, ... from the summed partial logits.
 PP_DEVINL void select_phase(const UnionArgs& a, unsigned char* smem) {
-    const int j = threadIdx.x, E = a.E;
-    struct Scratch {
-        CutShared cut;
-        WarpCand cand[kThreads];
-        CtaSelScratch sel;
-        float gx[kThreads];
-        uint32_t bw[8];
-    };
-    Scratch& s = *reinterpret_cast<Scratch*>(smem);
-    const bool mass_cut = (a.rule == PP_SEL_MIN_PREFIX || a.rule == PP_SEL_PAPER) && a.p < 1.0f;
+    SelScratch& s = *reinterpret_cast<SelScratch*>(smem);
     for (int t = blockIdx.x; t < a.T; t += gridDim.x) {
+        const size_t row = (size_t)t * a.E;
         auto logit = [&](int e) {  // partials added in split order, eight loads in flight
-            const float* q = a.part + (size_t)t * E + e;
-            const size_t stride = (size_t)a.T * E;
+            const float* q = a.part + row + e;
+            const size_t stride = (size_t)a.T * a.E;
             float v = 0.0f;
             int i = 0;
             for (; i + 8 <= a.nsplit; i += 8) {
@@ -227,46 +218,9 @@ PP_DEVINL void select_phase(const UnionArgs& a, unsigned char* smem) {
             for (; i < a.nsplit; i++) v += __ldcg(q + (size_t)i * stride);
             return v;
         };
-        int32_t* idr = a.ids ? a.ids + (size_t)t * E : nullptr;
-        float* gtr = a.gates ? a.gates + (size_t)t * E : nullptr;
-        float g;
-        int k;
-        s.gx[j] = 0.0f;  // ordered before the selection's writes by its barriers
-        if (j < 8) s.bw[j] = 0u;
-        if (mass_cut) {
-            g = j < E ? logit(j) : -INFINITY;
-            k = cta_mass_cut(g, E, a.p, a.rule, s.cut, s.cand, a.status, [&](int r, int e, float ge) {
-                const float gv = a.gate == PP_GATE_NONE ? 1.0f : sigmoidf_(ge);
-                if (idr) {
-                    idr[r] = e;
-                    gtr[r] = gv;
-                }
-                s.gx[e] = gv;
-                atomicOr(&s.bw[e >> 5], 1u << (e & 31));
-            }, [] {});
-            if (idr)
-                for (int r = k + j; r < E; r += kThreads) {
-                    idr[r] = -1;
-                    gtr[r] = 0.0f;
-                }
-        } else {
-            bool on;
-            int r;
-            k = cta_select_fn(logit, E, a.p, a.rule, idr != nullptr, s.sel, a.status, &on, &r, &g);
-            const float gv = on ? (a.gate == PP_GATE_NONE ? 1.0f : sigmoidf_(g)) : 0.0f;
-            if (idr) write_selection_row(idr, gtr, j, E, k, on, r, gv);
-            if (on) {
-                s.gx[j] = gv;
-                atomicOr(&s.bw[j >> 5], 1u << (j & 31));
-            }
-            __syncthreads();
-        }
-        if (j < 8) a.bits[(size_t)t * 8 + j] = s.bw[j];
-        if (j < E) {
-            a.gexp[(size_t)t * E + j] = s.gx[j];
-            if (a.logits) a.logits[(size_t)t * E + j] = g;
-        }
-        if (j == 0 && a.counts) a.counts[t] = k;
+        const SelOut o{a.ids ? a.ids + row : nullptr, a.counts ? a.counts + t : nullptr, a.gates ? a.gates + row : nullptr,
+                       a.logits ? a.logits + row : nullptr, a.bits + (size_t)t * 8, a.gexp + row};
+        select_token_cta(logit, a.E, a.p, a.rule, a.gate, s, o, a.status);
         __syncthreads();  // the scratch is reused by the next token
     }
 }
