@@ -54,8 +54,7 @@ bool use_grouped(const pp_desc& d, int T) { return d.dtype == PP_BF16 && T >= kG
 struct Layout {
     size_t logits, ids, counts, gates, tlog, th, stats;
     // grouped path
-    size_t part, bits, gexp, invpos, wcnt, blkcnt, blkbase, offsets, n_items, items, perm_token, perm_gate, H, Y,
-        yacc, overflow, dpart;
+    size_t part, bits, gexp, slot_of, cnt, ltok, lgate, offsets, H, Y, yacc, overflow, dpart;
     // fp32 calls of more tokens than a fused decode launch takes (bits and gexp too)
     size_t h32;
     size_t total;
@@ -83,16 +82,11 @@ Layout layout(const pp_desc& d, int T) {
         L.part = take((size_t)g.nsplit * Tn * E * 4);
         L.bits = take(Tn * 8 * 4);
         L.gexp = take(Tn * E * 4);
-        L.invpos = take(Tn * E * 4);
-        const size_t nblk = (Tn + 255) / 256;
-        L.wcnt = take(nblk * 8 * E * 4);
-        L.blkcnt = take(nblk * E * 4);
-        L.blkbase = take(nblk * E * 4);
+        L.slot_of = take(Tn * E * 4);
+        L.cnt = take(E * 4);
+        L.ltok = take((size_t)g.nnz_max * 4);
+        L.lgate = take((size_t)g.nnz_max * 4);
         L.offsets = take((E + 1) * 4);
-        L.n_items = take(16);
-        L.items = take((size_t)g.max_items * 16);
-        L.perm_token = take((size_t)g.nnz_max * 4);
-        L.perm_gate = take((size_t)g.nnz_max * 4);
         L.H = take(((size_t)g.nnz_max + 128) * kDExpert * 2);
         L.Y = take((size_t)g.ycap * d.d_model * 2);
         L.yacc = take(Tn * (size_t)d.d_model * 4);
@@ -256,15 +250,11 @@ GroupedArgs grouped_args(const pp_desc& d, int T, void* ws, const void* x, const
     a.part = reinterpret_cast<float*>(b + L.part);
     a.bits = reinterpret_cast<uint32_t*>(b + L.bits);
     a.gexp = reinterpret_cast<float*>(b + L.gexp);
-    a.invpos = reinterpret_cast<int*>(b + L.invpos);
-    a.wcnt = reinterpret_cast<int*>(b + L.wcnt);
-    a.blkcnt = reinterpret_cast<int*>(b + L.blkcnt);
-    a.blkbase = reinterpret_cast<int*>(b + L.blkbase);
+    a.slot_of = reinterpret_cast<int*>(b + L.slot_of);
+    a.cnt = reinterpret_cast<int*>(b + L.cnt);
+    a.ltok = reinterpret_cast<int*>(b + L.ltok);
+    a.lgate = reinterpret_cast<float*>(b + L.lgate);
     a.offsets = reinterpret_cast<int*>(b + L.offsets);
-    a.n_items = reinterpret_cast<int*>(b + L.n_items);
-    a.items = b + L.items;
-    a.perm_token = reinterpret_cast<int*>(b + L.perm_token);
-    a.perm_gate = reinterpret_cast<float*>(b + L.perm_gate);
     a.H = reinterpret_cast<__nv_bfloat16*>(b + L.H);
     a.Y = reinterpret_cast<__nv_bfloat16*>(b + L.Y);
     a.yacc = reinterpret_cast<float*>(b + L.yacc);
@@ -527,13 +517,11 @@ pp_status pp_layer(const pp_desc* desc, const void* x, int T, const void* W_r, c
     const float kp = rule_kernel_param(desc->rule, p, desc->n_experts);
     if (use_grouped(*desc, T)) {
         GroupedArgs a = grouped_args(*desc, T, ws, x, W_r, W_gate, W_up, W_down, kp, s, y);
-        if (T <= kUnionMaxT) {
-            if (!sel_out) {  // nobody reads the rank order
-                a.ids = a.counts = nullptr;
-                a.gates = nullptr;
-            }
-            return cuda_status(union_layer(a, true, device_info().sms, st));
+        if (!sel_out) {  // nobody reads the rank order
+            a.ids = a.counts = nullptr;
+            a.gates = nullptr;
         }
+        if (T <= kUnionMaxT) return cuda_status(union_layer(a, true, device_info().sms, st));
         PP_TRY(cuda_status(grouped_route(a, st)));
         return cuda_status(grouped_ffn(a, device_info().sms, st));
     }

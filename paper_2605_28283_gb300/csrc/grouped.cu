@@ -1,28 +1,27 @@
-// Tensor-core (tcgen05) path for many tokens: batched decode and prefill.
+// Tensor-core (tcgen05) path for prompts and prefill (bf16, more than
+// kUnionMaxT tokens), and the stand-alone routing of the batched path.
 //
 //   router GEMM   logits = X W_r^T (Eq. routing_logits), split over K; the
 //                 selection kernel sums the K-split partials in fixed order
-//   dispatch      per-token expert bitmasks -> per-expert counts -> offsets
-//                 and 128-row work items -> a stable permutation (tokens in
-//                 ascending order within each expert) with each assignment's
-//                 gate weight
+//   selection     a warp per token; an activated (token, expert) pair takes
+//                 the next slot of the expert's token list
 //   grouped G/U   per work item (expert e, <= 128 of its tokens):
 //                 D[128 x (64|128)] = X_gathered * [W_gate_e ; W_up_e]^T on
 //                 tcgen05 (TMA gather4 for the token rows), then
 //                 h = act(gate, up) * gate weight (Eq. ffn, Eq. moe_output),
-//                 stored bf16 in permuted order
-//   grouped down  per work item and 256-wide slice j of d:
-//                 D[128 x 256] = H_item * W_down[j, e-block]^T (K = 64); each
-//                 row (one token-expert assignment) is stored bf16 in the
-//                 permuted order
+//                 stored bf16, one row per pair, experts in ascending order
+//   grouped down  per (work item, 128-row tile of W_down):
+//                 D[128 rows x tokens] = W_down[tile, e-block] * H_item^T
+//                 (K = 64); each pair's output row is stored bf16
 //   combine       y[t] = sum over t's experts, in ascending expert order, of
-//                 its assignment rows (fp32 accumulation, deterministic)
-//   Assignments past the row buffer's capacity (only near-dense selections)
-//   are added into an fp32 accumulator with vector reductions instead; the
-//   combine step reads and re-zeroes it.
+//                 its pairs' rows (fp32 accumulation, deterministic)
+//   Pairs past the row buffer's capacity (only near-dense selections) are
+//   added into an fp32 accumulator instead; the combine step reads and
+//   re-zeroes it.
 //
-// Every GEMM kernel: warp 0 = TMA producer, warp 1 = TMEM owner and UMMA
-// issuer (one thread), warps 2..5 = epilogue (TMEM lanes 32*(warp%4)..).
+// A slot is given out by an atomic, so the order of an expert's tokens varies
+// between calls; no result depends on it (a row of a GEMM tile does not depend
+// on its place, and the combine step goes by expert).
 // All waits are bounded (PP_ERR_TIMEOUT).
 #include "pp_common.cuh"
 #include "pp_kernels.h"
@@ -33,11 +32,12 @@
 namespace pp {
 
 constexpr int kTcThreads = 192;
+// Prompts above this many tokens run the down projection with tokens as the M
+// operand (333 tokens of the 7B shape: 34 us with weights as M against 45; 2048
+// of the 13B shape: 69 against 60; 8192: 199 against 124).
+constexpr int kDownRowsMinT = 1024;
 constexpr int kTileBytesA = 128 * 128;  // 128 rows x 64 bf16
 
-struct WorkItem {
-    int e, a0, cnt, pad;
-};
 
 // ====================================================================== router
 // Grid (m-tiles, splits).  CTA (m, s): D[128 tokens x NE] over K chunks
@@ -45,9 +45,14 @@ struct WorkItem {
 template <int NE>
 __global__ void __launch_bounds__(kTcThreads, 1)
     router_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_wr,
-                       int T, int E, int nk, int kpb, float* part, unsigned* status, uint64_t lim) {
+                       int T, int E, int nk, int kpb, float* part, int* cnt, int* overflow, unsigned* status,
+                       uint64_t lim) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
+    if (cnt && blockIdx.x == 0 && blockIdx.y == 0) {  // the selection fills the lists
+        for (int e = threadIdx.x; e < E; e += blockDim.x) cnt[e] = 0;
+        if (threadIdx.x == 0) *overflow = 0;
+    }
     constexpr int kStages = 4;
     constexpr int kTileB = NE * 128;
     constexpr int kStage = kTileBytesA + kTileB;
@@ -60,7 +65,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int k0 = split * kpb, k1 = min(nk, k0 + kpb);
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; i++) {
-            mbar_init(&full[i], 1);
+            mbar_init(&full[i], 2);
             mbar_init(&empty[i], 1);
         }
         mbar_init(&tfull, 1);
@@ -75,14 +80,18 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tc_fence_after();
     const uint32_t tmem = taddr_s;
 
-    if (warp == 0 && lane == 0) {
+    // the W_r and x tiles are issued by two warps (a TMA instruction costs its
+    // warp 24 ns plus 1.3 ns per row: 224 + 128 rows a stage by one took 450 ns)
+    if ((warp == 0 || warp == 2) && lane == 0) {
         for (int kc = k0, it = 0; kc < k1; kc++, it++) {
             const int s = it % kStages;
             if (it >= kStages) mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, status, lim);
             unsigned char* st = smem + (size_t)s * kStage;
-            mbar_arrive_expect_tx(&full[s], kStage);
-            tma_load_2d(st, &map_x, kc * 64, m0, &full[s]);
-            tma_load_2d(st + kTileBytesA, &map_wr, kc * 64, 0, &full[s]);
+            mbar_arrive_expect_tx(&full[s], warp == 0 ? kTileB : kTileBytesA);
+            if (warp == 0)
+                tma_load_2d(st + kTileBytesA, &map_wr, kc * 64, 0, &full[s]);
+            else
+                tma_load_2d(st, &map_x, kc * 64, m0, &full[s]);
         }
     } else if (warp == 1 && lane == 0) {
         constexpr uint32_t idesc = idesc_bf16_m128(NE);
@@ -95,28 +104,32 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             umma_commit(&empty[s]);
         }
         umma_commit(&tfull);
-    } else if (warp >= 2) {
-        // lane = row 32 q + lane of the tile; 32 x 32 blocks are transposed
-        // through shared memory (the pipeline stages are free once every MMA
-        // has completed) so that each store writes 32 consecutive logits of
-        // one row
-        const int q = warp & 3;
+    }
+    __syncwarp();
+    if (warp >= 2) {
+        // lane = token row 32 q + lane; a lane stores its row's 32 logits in
+        // 16-byte pieces where rows are 16-byte aligned
+        const int q = warp & 3, t = m0 + 32 * q + lane;
         mbar_wait(&tfull, 0, status, lim);
         tc_fence_after();
-        float* tr = reinterpret_cast<float*>(smem) + (size_t)(warp - 2) * 32 * 33;
+        float* row = part + ((size_t)split * T + t) * E;
 #pragma unroll 1
-        for (int c = 0; c < NE; c += 32) {
+        for (int c = 0; c < (m0 + 32 * q < T ? E : 0); c += 32) {
             uint32_t r[32];
             tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c, r);
             tmem_ld_wait();
+            if (t >= T) continue;
+            if ((E & 3) == 0) {
 #pragma unroll
-            for (int i = 0; i < 32; i++) tr[lane * 33 + i] = k1 > k0 ? __uint_as_float(r[i]) : 0.0f;
-            __syncwarp();
-            for (int i = 0; i < 32; i++) {
-                const int t = m0 + 32 * q + i;
-                if (t < T && c + lane < E) part[((size_t)split * T + t) * E + c + lane] = tr[i * 33 + lane];
+                for (int i = 0; i < 32; i += 4)
+                    if (c + i < E)
+                        *reinterpret_cast<uint4*>(row + c + i) =
+                            k1 > k0 ? make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]) : make_uint4(0u, 0u, 0u, 0u);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 32; i++)
+                    if (c + i < E) row[c + i] = k1 > k0 ? __uint_as_float(r[i]) : 0.0f;
             }
-            __syncwarp();
         }
     }
     tc_fence_before();
@@ -125,9 +138,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 }
 
 // ================================================================= selection
-// Selection from K-split partial logits (summed in split order).  The
-// cumulative-mass cut, and the other rules up to kCtaSelectMaxTokens tokens,
-// take one CTA per token; the others one warp per token (the warp sort).
+// Selection from K-split partial logits (summed in split order): one CTA per
+// token up to kCtaSelectMaxTokens tokens (latency), one warp per token beyond.
 constexpr int kCtaSelectMaxTokens = 256;
 
 // Logit = sum over s of part[s * stride + off], added in split order; the
@@ -146,70 +158,157 @@ PP_DEVINL float sum_partials(const float* __restrict__ part, int nsplit, size_t 
     return v;
 }
 
-// The selection is written in two forms: rank order (ids, counts, gates) for
-// the caller, and per expert for the FFN kernels -- bits[t] (E bits in 8
-// words) and gexp[t][e], the gate weight, 0 where e is not activated.  bits is
-// NULL when no FFN follows (pp_route).
+// Per-expert lists of the activated pairs: cnt[e] tokens ltok[e * T + slot]
+// with gate weights lgate[e * T + slot]; slot_of[t * E + e] = slot.
+struct Lists {
+    int* cnt;
+    int* ltok;
+    float* lgate;
+    int* slot_of;
+};
+
+PP_DEVINL void list_add(const Lists& l, int T, int E, int t, int e, float gv) {
+    const int s = atomicAdd(&l.cnt[e], 1);
+    l.ltok[(size_t)e * T + s] = t;
+    l.lgate[(size_t)e * T + s] = gv;
+    l.slot_of[(size_t)t * E + e] = s;
+}
+
+// Selection of one token by a warp, lane l holding logits l, l + 32, ...: the
+// experts are taken in descending order one by one (two warp reductions each)
+// until the rule stops, with the exact fixed-point masses of group_mass_cut, so
+// the decisions are the same.  An activated expert costs about 110 cycles and
+// nothing is sorted that is not activated: one CTA per token took 46 us for
+// 8192 tokens of 216 experts (7 activated each), this 12 us.  ids and gates
+// (together), counts, logits_out may be NULL; so may bits with the lists.
 template <int S>
-__global__ void __launch_bounds__(256) select_part_kernel(const float* __restrict__ part, int nsplit, int T, int E,
-                                                          float p, int rule, int gate, int32_t* ids, int32_t* counts,
-                                                          float* gates, float* logits_out, uint32_t* bits,
-                                                          float* gexp, unsigned* status) {
+__global__ void __launch_bounds__(256)
+    select_warp_kernel(const float* __restrict__ part, int nsplit, int T, int E, float p, int rule, int gate, int32_t* ids,
+                       int32_t* counts, float* gates, float* logits_out, uint32_t* bits, Lists lists, unsigned* status) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (t >= T) return;
-    auto load = [&](int j) { return sum_partials(part, nsplit, (size_t)T * E, (size_t)t * E + j); };
-    unsigned long long key[S];
-    bool finite = true;
-    const int k = warp_select<S>(load, E, p, rule, key, &finite);
-    if (!finite && lane == 0) record_status(status, PP_ERR_NONFINITE);
-    float* grow = gexp + (size_t)t * E;
-    if (bits) {
-        for (int e = lane; e < E; e += 32) grow[e] = 0.0f;
-        __syncwarp();  // before the activated experts' weights below
+    const size_t row = (size_t)t * E;
+    float g[S];
+    uint32_t D[S], U[S];
+    bool fin = true;
+    uint32_t dmin = 0xffffffffu;
+    const size_t stride = (size_t)T * E;
+#pragma unroll
+    for (int s = 0; s < S; s++) g[s] = 0.0f;
+#pragma unroll 4
+    for (int sp = 0; sp < nsplit; sp++) {  // partials added in split order, all slots' loads in flight
+        const float* q = part + sp * stride + row + lane;
+#pragma unroll
+        for (int s = 0; s < S; s++)
+            if (lane + 32 * s < E) g[s] += __ldg(q + 32 * s);
     }
-    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
     for (int s = 0; s < S; s++) {
-        const int r = lane * S + s;
-        if (r >= E) continue;
-        const bool on = finite && r < k;
-        const int e = on ? key_index(key[s]) : -1;
-        const float gv = on ? gate_of(gate, key[s]) : 0.0f;
-        ids[(size_t)t * E + r] = e;
-        gates[(size_t)t * E + r] = gv;
-        if (on && bits) {
-            grow[e] = gv;
-#pragma unroll
-            for (int i = 0; i < 8; i++) w[i] |= (e >> 5) == i ? 1u << (e & 31) : 0u;
+        const int j = lane + 32 * s;
+        D[s] = 0xffffffffu;  // no finite logit has this key
+        if (j < E) {
+            if (logits_out) logits_out[row + j] = g[s];
+            fin = fin && isfinite(g[s]);
+            D[s] = desc_key(g[s]);
+            dmin = min(dmin, D[s]);
         }
     }
+    fin = __all_sync(kFull, fin);
+    if (!fin && lane == 0) record_status(status, PP_ERR_NONFINITE);
+    const float m = desc_key_logit(__reduce_min_sync(kFull, dmin));
+    const bool mass_cut = (rule == PP_SEL_MIN_PREFIX || rule == PP_SEL_PAPER) && p < 1.0f;
+    unsigned long long z = 0ull;
+#pragma unroll
+    for (int s = 0; s < S; s++) {
+        U[s] = mass_cut && lane + 32 * s < E ? __float2uint_rn(expf(g[s] - m) * 2147483648.0f) : 0u;
+        z += U[s];
+    }
+    long long thr = -1;
+    if (mass_cut) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(kFull, z, o);
+        thr = prefix_threshold(p, z);
+    }
+    const int kmax = !fin ? 0 : rule == PP_SEL_TOPK ? min(E, (int)p) : E;
+    unsigned long long A = 0ull;  // mass ahead of rank r
+    int r = 0, my_e = 0;          // lane l keeps rank 32 i + l until it is written
+    float my_g = 0.0f;
+    auto flush = [&](int base, int n) {
+        if (lane < n) {
+            const float gv = gate == PP_GATE_NONE ? 1.0f : sigmoidf_(my_g);
+            if (ids) {
+                ids[row + base + lane] = my_e;
+                gates[row + base + lane] = gv;
+            }
+            if (bits) list_add(lists, T, E, t, my_e, gv);
+        }
+    };
+    while (r < kmax) {
+        uint32_t bd = 0xffffffffu, bu = 0u;
+        int bs = 0;
+        float bg = 0.0f;
+#pragma unroll
+        for (int s = 0; s < S; s++)
+            if (D[s] < bd) {  // the lowest index of equal keys
+                bd = D[s];
+                bs = s;
+                bu = U[s];
+                bg = g[s];
+            }
+        const uint32_t wd = __reduce_min_sync(kFull, bd);
+        const unsigned wj = __reduce_min_sync(kFull, bd == wd ? (unsigned)(bs * 32 + lane) : 0xffffffffu);
+        const int owner = (int)(wj & 31u);
+        const uint32_t u = __shfl_sync(kFull, bu, owner);
+        const float gv = __shfl_sync(kFull, bg, owner);
+        if (mass_cut) {
+            const unsigned long long mass = rule == PP_SEL_PAPER ? A + u : A;
+            if (!(A == 0ull || (thr >= 0 && mass <= (unsigned long long)thr))) break;
+            A += u;
+        } else if (rule == PP_SEL_LTE && !(gv >= p)) {
+            break;
+        }
+        if (lane == (r & 31)) {
+            my_e = (int)wj;
+            my_g = gv;
+        }
+#pragma unroll
+        for (int s = 0; s < S; s++)
+            if (lane == owner && s == bs) D[s] = 0xffffffffu;
+        r++;
+        if ((r & 31) == 0) flush(r - 32, 32);
+    }
+    flush(r & ~31, r & 31);
+    if (ids)
+        for (int i = r + lane; i < E; i += 32) {
+            ids[row + i] = -1;
+            gates[row + i] = 0.0f;
+        }
+    if (counts && lane == 0) counts[t] = r;
     if (bits) {
 #pragma unroll
-        for (int i = 0; i < 8; i++) {
-            const uint32_t v = __reduce_or_sync(kFull, w[i]);
-            if (lane == i) bits[(size_t)t * 8 + i] = v;
+        for (int s = 0; s < 8; s++) {  // expert lane + 32 s is bit `lane` of word s
+            bool on = false;
+            if (s < S) on = fin && lane + 32 * s < E && D[s < S ? s : 0] == 0xffffffffu;
+            const unsigned v = __ballot_sync(kFull, on);
+            if (lane == s) bits[(size_t)t * 8 + s] = v;
         }
     }
-    if (lane == 0) counts[t] = k;
-    if (logits_out)
-        for (int j = lane; j < E; j += 32) logits_out[(size_t)t * E + j] = load(j);
 }
 
 // One CTA per token.
 __global__ void __launch_bounds__(256) select_part_cta_kernel(const float* __restrict__ part, int nsplit, int T,
                                                               int E, float p, int rule, int gate, int32_t* ids,
                                                               int32_t* counts, float* gates, float* logits_out,
-                                                              uint32_t* bits, float* gexp, unsigned* status) {
+                                                              unsigned* status) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
     __shared__ __align__(16) SelScratch sc;
     const int t = blockIdx.x;
     const size_t row = (size_t)t * E;
-    const SelOut o{ids + row, counts + t, gates + row, logits_out ? logits_out + row : nullptr,
-                   bits ? bits + (size_t)t * 8 : nullptr, gexp + row};
+    const SelOut o{ids + row, counts + t, gates + row, logits_out ? logits_out + row : nullptr, nullptr, nullptr};
     select_token_cta([&](int j) { return sum_partials(part, nsplit, (size_t)T * E, row + j); }, E, p, rule, gate, sc, o,
                      status);
 }
@@ -222,9 +321,14 @@ __global__ void __launch_bounds__(256) select_part_cta_kernel(const float* __res
 __global__ void __launch_bounds__(256) dispatch_bits_kernel(const int32_t* __restrict__ ids,
                                                             const int32_t* __restrict__ counts,
                                                             const float* __restrict__ gates, int T, int E,
-                                                            uint32_t* bits, float* gexp, unsigned* status) {
+                                                            uint32_t* bits, float* gexp, int* cnt, int* overflow,
+                                                            unsigned* status) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
+    if (cnt && blockIdx.x == 0) {  // lengths of the lists that dispatch_list_kernel fills
+        for (int e = threadIdx.x; e < E; e += blockDim.x) cnt[e] = 0;
+        if (threadIdx.x == 0) *overflow = 0;
+    }
     // one warp per token: coalesced row writes
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -265,244 +369,209 @@ __global__ void __launch_bounds__(256) dispatch_bits_kernel(const int32_t* __res
     }
 }
 
-// Token block b (256 tokens, one per thread): per-warp counts of every
-// expert via ballots; block totals blkcnt[b][e].
-constexpr int kDispBlock = 256;
-
-__global__ void __launch_bounds__(kDispBlock) dispatch_count_kernel(const uint32_t* __restrict__ bits, int T, int E,
-                                                                    int* wcnt, int* blkcnt) {
+// The lists from bits and gexp (a selection given by the caller): a warp per
+// token, lane l the experts l, l + 32, ...
+__global__ void __launch_bounds__(256) dispatch_list_kernel(const uint32_t* __restrict__ bits,
+                                                            const float* __restrict__ gexp, int T, int E, Lists lists) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
-    const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t = b * kDispBlock + threadIdx.x;
-    uint32_t w[8];
+    const int lane = threadIdx.x & 31, t = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (t >= T) return;
+    for (int e = lane; e < E; e += 32)
+        if ((bits[(size_t)t * 8 + (e >> 5)] >> (e & 31)) & 1u) list_add(lists, T, E, t, e, gexp[(size_t)t * E + e]);
+}
+
+// Work items of a call, formed by each CTA from the list lengths: expert e's
+// tokens are cut into items of 128; off = first row of the expert in H and Y.
+struct Item {
+    int e, m0, cnt, a0;  // expert, first slot, tokens (<= 128), first row
+};
+
+struct ItemTable {
+    int off[kMaxExperts + 1], ib[kMaxExperts + 1];
+    int longest;  // tokens of the longest item
+
+    // Warp 0 of the CTA builds the table (8 experts per lane); a barrier follows.
+    PP_DEVINL void build(const int* __restrict__ cnt, int E) {
+        if (threadIdx.x >= 32) return;
+        const int lane = threadIdx.x;
+        int c[8], cs = 0, ms = 0, cm = 0;
 #pragma unroll
-    for (int i = 0; i < 8; i++) w[i] = t < T ? bits[(size_t)t * 8 + i] : 0u;
-    __shared__ int sc[8][kMaxExperts];
-    for (int e = 0; e < E; e++) {
-        const unsigned bal = __ballot_sync(kFull, (w[e >> 5] >> (e & 31)) & 1u);
-        if (lane == 0) sc[warp][e] = __popc(bal);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < E; e += kDispBlock) {
-        int s = 0;
-        for (int v = 0; v < 8; v++) {
-            wcnt[((size_t)b * 8 + v) * E + e] = s;  // exclusive prefix over the block's warps
-            s += sc[v][e];
+        for (int q = 0; q < 8; q++) {
+            const int e = lane * 8 + q;
+            c[q] = e < E ? cnt[e] : 0;
+            cm = max(cm, min(c[q], 128));
+            cs += c[q];
+            ms += (c[q] + 127) / 128;
         }
-        blkcnt[(size_t)b * E + e] = s;
-    }
-}
-
-// One block, thread e: hist, offsets (exclusive scan over experts), the
-// per-token-block bases and the expert's 128-row work items; clears the
-// overflow flag of the down projection.
-__global__ void __launch_bounds__(kMaxExperts) dispatch_scan_kernel(const int* __restrict__ blkcnt, int nblk, int E,
-                                                                    int* offsets, int* blkbase, WorkItem* items,
-                                                                    int* n_items, int* overflow) {
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    const int e = threadIdx.x;
-    if (e == 0) *overflow = 0;  // the down projection's overflow flag starts clear
-    __shared__ int sh[kMaxExperts], si[kMaxExperts];
-    int h = 0;
-    if (e < E)
-        for (int b = 0; b < nblk; b++) h += blkcnt[(size_t)b * E + e];
-    sh[e] = e < E ? h : 0;
-    si[e] = e < E ? (h + 127) / 128 : 0;
-    __syncthreads();
-    if (e == 0) {  // exclusive scans of counts and item counts (E <= 256)
-        int a = 0, n = 0;
-        for (int i = 0; i < E; i++) {
-            const int c = sh[i], m = si[i];
-            sh[i] = a;
-            si[i] = n;
-            a += c;
-            n += m;
-        }
-        offsets[E] = a;
-        *n_items = n;
-    }
-    __syncthreads();
-    if (e >= E) return;
-    const int off = sh[e];
-    offsets[e] = off;
-    int base = off;
-    for (int b = 0; b < nblk; b++) {
-        blkbase[(size_t)b * E + e] = base;
-        base += blkcnt[(size_t)b * E + e];
-    }
-    int n = si[e];
-    for (int m = 0; m < h; m += 128) items[n++] = WorkItem{e, off + m, min(128, h - m), 0};
-}
-
-// Token block b again: each token writes itself (and its gate weight) at
-// base + (earlier warps) + (earlier lanes) for every activated expert, so
-// tokens stay in ascending order within each expert; invpos[t][e] records
-// where (t, e) landed.
-__global__ void __launch_bounds__(kDispBlock) dispatch_scatter_kernel(const uint32_t* __restrict__ bits,
-                                                                      const float* __restrict__ gexp, int T, int E,
-                                                                      const int* __restrict__ wcnt,
-                                                                      const int* __restrict__ blkbase,
-                                                                      int* perm_token, float* perm_gate,
-                                                                      int* invpos) {
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t = b * kDispBlock + threadIdx.x;
-    const bool live = t < T;
-    // experts [e0, e1) of this block (blockIdx.y splits the expert loop)
-    const int e0 = blockIdx.y * E / gridDim.y, e1 = (blockIdx.y + 1) * E / gridDim.y;
-    // this block's bases, per warp: blkbase[b][e] + wcnt[b][warp][e]
-    __shared__ int base_s[8][kMaxExperts];
-    for (int i = threadIdx.x; i < 8 * (e1 - e0); i += kDispBlock) {
-        const int v = i / (e1 - e0), e = e0 + i - v * (e1 - e0);
-        base_s[v][e] = blkbase[(size_t)b * E + e] + wcnt[((size_t)b * 8 + v) * E + e];
-    }
-    __syncthreads();
-    uint32_t w[8];
+        int ci = cs, mi = ms;
 #pragma unroll
-    for (int i = 0; i < 8; i++) w[i] = live ? bits[(size_t)t * 8 + i] : 0u;
-    const unsigned lt = (1u << lane) - 1u;
-    for (int e = e0; e < e1; e++) {
-        const bool on = (w[e >> 5] >> (e & 31)) & 1u;
-        const unsigned bal = __ballot_sync(kFull, on);
-        if (on) {
-            const int pos = base_s[warp][e] + __popc(bal & lt);
-            perm_token[pos] = t;
-            perm_gate[pos] = gexp[(size_t)t * E + e];
-            invpos[(size_t)t * E + e] = pos;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int cv = __shfl_up_sync(kFull, ci, o), mv = __shfl_up_sync(kFull, mi, o);
+            if (lane >= o) {
+                ci += cv;
+                mi += mv;
+            }
+        }
+        int co = ci - cs, mo = mi - ms;
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            off[lane * 8 + q] = co;
+            ib[lane * 8 + q] = mo;
+            co += c[q];
+            mo += (c[q] + 127) / 128;
+        }
+        cm = __reduce_max_sync(kFull, cm);
+        if (lane == 31) {
+            longest = cm;
+            off[kMaxExperts] = co;
+            ib[kMaxExperts] = mo;
         }
     }
-}
+    PP_DEVINL int n_items() const { return ib[kMaxExperts]; }
+    PP_DEVINL Item item(int wi) const {
+        int lo = 0, hi = kMaxExperts;  // ib[lo] <= wi < ib[hi]
+#pragma unroll 1
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (ib[mid] <= wi) lo = mid; else hi = mid;
+        }
+        const int m0 = (wi - ib[lo]) * 128;
+        return Item{lo, m0, min(128, off[lo + 1] - off[lo] - m0), off[lo] + m0};
+    }
+};
 
 // =============================================================== grouped G/U
-// Persistent over work items.  NB = 128 (SwiGLU: gate rows then up rows) or
-// 64 (non-gated: up rows).  Two TMEM accumulators let the epilogue of one
-// item overlap the MMAs of the next.
+// Persistent over tasks: a work item, or half of its neurons where whole items
+// would leave the last round nearly empty.  A = the item's token rows (TMA
+// gather4, live rows only), B = the expert's gate and up rows, K-chunks of 64.
 //
-// Warp roles: warp 0 streams the expert's weight tiles with 2-D TMA, warp 1
-// issues the MMAs, warps 2-5 run the epilogue, and warps 6-9 gather the
-// item's token rows: thread r copies row r of the A tile (128 bytes per
-// K chunk) with eight 16-byte cp.async into the 128-byte-swizzled layout the
-// TMA would write.  (A TMA gather4 moves 512 bytes per instruction and its
-// rate, about 14 GB/s per SM, bounded this kernel; cp.async keeps the L2
-// streaming.)  A gather thread keeps kGatherLag stages of copies in flight;
-// once a stage's copies are complete it fences them into the async proxy
-// and arrives on the stage's full barrier (129 arrivals: the weight TMA's
-// expect-tx arrival and the 128 gather threads).
-constexpr int kGuThreads = 320;
-constexpr int kGatherLag = 3;
+// What bounds it: the SM's TMA and L2 path, about 1 ns per 128-byte row (256
+// rows of a full chunk), if enough warps issue and enough stages are in flight
+// (a stage's round trip is about 1.4 us: the ring holds as many stages as the
+// longest item's rows leave room for, 16 at most; six fixed stages took 330 ns
+// per chunk of a 12-token item's half): a gather4 costs its warp about
+// 30 ns, so eight producer warps take 4 of a chunk's 32 gathers each (one
+// gather thread per row with cp.async, three stages in flight, took 400-580 ns
+// per chunk).  An MMA thread needs 55-64 cycles per MMA and about 300 for a
+// stage's wait and commit, so two MMA warps take the stages in turn, each with
+// its own accumulators (added in the epilogue); the ring is even, so that a
+// slot is always the same MMA warp's.  Two accumulator sets let the epilogue
+// of one task overlap the MMAs of the next.  An MMA reads 128 token rows; those
+// past the item's are whatever the ring holds, and so are their sums, which are
+// never stored.
+constexpr int kGuProd = 8, kGuMma = 2, kGuEpi = 4;  // warps
+constexpr int kGuThreads = (kGuProd + kGuMma + kGuEpi) * 32;
+constexpr int kGuStages = 16;  // at most
+constexpr size_t kGuRing = 206 * 1024, kGuSlack = kTileBytesA;  // ring, and the rows that the last MMA reads past it
+constexpr int kGuBox = 32;  // weight rows of a TMA box
 
-template <int NB>
 __global__ void __launch_bounds__(kGuThreads, 1)
-    gu_gemm_kernel(const __nv_bfloat16* __restrict__ x, int d, const __grid_constant__ CUtensorMap map_wg,
-                   const __grid_constant__ CUtensorMap map_wu, const WorkItem* __restrict__ items,
-                   const int* __restrict__ n_items_p, const int* __restrict__ perm_token,
-                   const float* __restrict__ perm_gate, int nk, int act, __nv_bfloat16* H, unsigned* status,
-                   uint64_t lim) {
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    constexpr int kStages = NB == 128 ? 6 : 8;
-    static_assert(kGatherLag < kStages, "a gather thread must release a stage before it waits for it again");
-    constexpr int kTileB = NB * 128;
-    constexpr int kStage = kTileBytesA + kTileB;
-    constexpr uint32_t kCols = 2 * NB;  // two accumulators
+    gu_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_wg,
+                   const __grid_constant__ CUtensorMap map_wu, const int* __restrict__ cnt, const int* __restrict__ ltok,
+                   const float* __restrict__ lgate, int* offsets, int T, int E, int nk, int act, __nv_bfloat16* H,
+                   unsigned* status, uint64_t lim) {
+    const bool gated = act == PP_ACT_SWIGLU;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t full[kStages], empty[kStages], tfull[2], tempty[2];
+    __shared__ uint64_t full[kGuStages], empty[kGuStages], tfull[2], tempty[2];
     __shared__ uint32_t taddr_s;
+    __shared__ ItemTable tab;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_items = *n_items_p;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; i++) {
-            mbar_init(&full[i], 1 + 128);
+        for (int i = 0; i < kGuStages; i++) {
+            mbar_init(&full[i], kGuProd);
             mbar_init(&empty[i], 1);
         }
         for (int i = 0; i < 2; i++) {
-            mbar_init(&tfull[i], 1);
-            mbar_init(&tempty[i], 4);
+            mbar_init(&tfull[i], kGuMma);
+            mbar_init(&tempty[i], kGuEpi);
         }
         fence_mbar_init();
     }
-    if (warp == 1) {
-        tmem_alloc(&taddr_s, kCols < 32 ? 32 : kCols);
+    if (warp == kGuProd) {
+        tmem_alloc(&taddr_s, 512);  // 2 sets x 2 MMA warps x 128 columns
         tmem_relinquish();
     }
+    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
+    pdl_launch_dependents();
+    tab.build(cnt, E);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = taddr_s;
+    if (blockIdx.x == 0)
+        for (int e = threadIdx.x; e <= E; e += kGuThreads) offsets[e] = tab.off[e];
+    // whole items, or halves where they shorten the longest CTA (a half costs
+    // about 0.6 of an item: its tokens are gathered again)
+    const int n_items = tab.n_items(), G = gridDim.x;
+    const int split = ((2 * n_items + G - 1) / G) * 6 < ((n_items + G - 1) / G) * 10 ? 2 : 1;
+    const int nb = 64 / split, n_tasks = n_items * split;  // neurons of a task
+    const int brows = gated ? 2 * nb : nb;
+    const int bbytes = brows * 128, stage = bbytes + ((tab.longest + 7) & ~7) * 128;
+    const int nst = min(kGuStages, (int)kGuRing / stage) & ~1;
 
-    if (warp == 0) {
-        if (lane == 0) {
-            int it = 0;
-            for (int wi = blockIdx.x; wi < n_items; wi += gridDim.x) {
-                const WorkItem w = items[wi];
-                for (int kc = 0; kc < nk; kc++, it++) {
-                    const int s = it % kStages;
-                    unsigned char* st = smem + (size_t)s * kStage;
-                    if (it >= kStages) mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, status, lim);
-                    mbar_arrive_expect_tx(&full[s], (uint32_t)kTileB);
-                    if (NB == 128) {
-                        tma_load_2d(st + kTileBytesA, &map_wg, kc * 64, w.e * 64, &full[s]);
-                        tma_load_2d(st + kTileBytesA + 64 * 128, &map_wu, kc * 64, w.e * 64, &full[s]);
-                    } else {
-                        tma_load_2d(st + kTileBytesA, &map_wu, kc * 64, w.e * 64, &full[s]);
-                    }
-                }
-            }
-        }
-        __syncwarp();
-    } else if (warp >= 6) {
-        // token-row gather; rows past the item's count are not copied (their
-        // accumulator rows are never stored)
-        const int row = (warp - 6) * 32 + lane;
-        const uint32_t swz = (uint32_t)(row & 7);
-        int it = 0;
-        for (int wi = blockIdx.x; wi < n_items; wi += gridDim.x) {
-            const WorkItem w = items[wi];
-            const bool live = row < w.cnt;
-            const __nv_bfloat16* src = x + (size_t)(live ? perm_token[w.a0 + row] : 0) * d;
-            for (int kc = 0; kc < nk; kc++, it++) {
-                const int s = it % kStages;
-                if (lane == 0 && it >= kStages) mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, status, lim);
-                __syncwarp();
-                unsigned char* dst = smem + (size_t)s * kStage + row * 128;
-                const int c0 = kc * 64;
-                if (live) {
+    if (warp < kGuProd) {
+        int it_s = 0;
+        uint32_t it_ph = 0;
+        bool primed = false;
+        for (int v = blockIdx.x; v < n_tasks; v += G) {
+            const Item w = tab.item(v / split);
+            const int n0 = (v % split) * nb;
+            // lane l < 4: rows 4 (warp + 8 l) .. + 3 (past the count: the last row)
+            const int grp = warp + kGuProd * lane, ng = (w.cnt + 3) >> 2;
+            const bool gather = lane < 4 && grp < ng;
+            int r[4] = {0, 0, 0, 0};
+            if (gather)
 #pragma unroll
-                    for (int c = 0; c < 8; c++) {
-                        const bool in = c0 + c * 8 < d;  // d is a multiple of 8: chunks are whole
-                        cp_async_16(dst + (((uint32_t)c ^ swz) << 4), in ? src + c0 + c * 8 : src, in ? 16u : 0u);
-                    }
+                for (int i = 0; i < 4; i++) r[i] = ltok[(size_t)w.e * T + w.m0 + min(4 * grp + i, w.cnt - 1)];
+            // box `warp` of the weight rows goes out from lane 4
+            const bool box = lane == 4 && warp * kGuBox < brows;
+            const bool up = !gated || warp * kGuBox >= nb;
+            const int brow = w.e * 64 + n0 + (up && gated ? warp * kGuBox - nb : warp * kGuBox);
+            const uint32_t bytes =
+                (uint32_t)(__popc(__ballot_sync(kFull, gather)) * 512 + (warp * kGuBox < brows ? kGuBox * 128 : 0));
+            for (int kc = 0; kc < nk; kc++) {
+                if (lane == 0) {
+                    if (primed) mbar_wait(&empty[it_s], it_ph ^ 1u, status, lim);
+                    mbar_arrive_expect_tx(&full[it_s], bytes);
                 }
-                cp_async_commit();
-                if (it >= kGatherLag) {
-                    cp_async_wait<kGatherLag>();
-                    fence_proxy_async_smem();
-                    mbar_arrive(&full[(it - kGatherLag) % kStages]);
+                __syncwarp();
+                unsigned char* st = smem + (size_t)it_s * stage;
+                if (gather) tma_gather4(st + bbytes + grp * 512, &map_x, kc * 64, r[0], r[1], r[2], r[3], &full[it_s]);
+                if (box)
+                    tma_load_2d(st + warp * kGuBox * 128, up ? &map_wu : &map_wg, kc * 64, brow, &full[it_s]);
+                if (++it_s == nst) {
+                    it_s = 0;
+                    it_ph ^= 1u;
+                    primed = true;
                 }
             }
         }
-        cp_async_wait<0>();
-        fence_proxy_async_smem();
-        for (int j = it > kGatherLag ? it - kGatherLag : 0; j < it; j++) mbar_arrive(&full[j % kStages]);
-    } else if (warp == 1) {
+    } else if (warp < kGuProd + kGuMma) {
         if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16_m128(NB);
-            int it = 0, acc = 0;
-            for (int wi = blockIdx.x; wi < n_items; wi += gridDim.x, acc++) {
+            const int m = warp - kGuProd;
+            const uint32_t idesc = idesc_bf16_m128(brows);
+            int it = 0, s = 0, acc = 0;
+            uint32_t ph = 0;
+            for (int v = blockIdx.x; v < n_tasks; v += G, acc++) {
                 const int a = acc & 1;
                 if (acc >= 2) mbar_wait(&tempty[a], (uint32_t)((acc >> 1) - 1) & 1u, status, lim);
                 tc_fence_after();
+                bool fresh = true;
                 for (int kc = 0; kc < nk; kc++, it++) {
-                    const int s = it % kStages;
-                    mbar_wait(&full[s], (uint32_t)(it / kStages) & 1u, status, lim);
-                    tc_fence_after();
-                    unsigned char* st = smem + (size_t)s * kStage;
-                    umma_k64(tmem + (uint32_t)(a * NB), st, st + kTileBytesA, idesc, kc > 0);
-                    umma_commit(&empty[s]);
+                    if ((it & 1) == m) {
+                        mbar_wait(&full[s], ph, status, lim);
+                        tc_fence_after();
+                        unsigned char* st = smem + (size_t)s * stage;
+                        umma_k64(tmem + (uint32_t)(a * 256 + m * 128), st + bbytes, st, idesc, !fresh);
+                        umma_commit(&empty[s]);
+                        fresh = false;
+                    }
+                    if (++s == nst) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
                 umma_commit(&tfull[a]);
             }
@@ -511,37 +580,52 @@ __global__ void __launch_bounds__(kGuThreads, 1)
     } else {
         const int q = warp & 3;
         const int row = 32 * q + lane;
-        int acc = 0;
-        for (int wi = blockIdx.x; wi < n_items; wi += gridDim.x, acc++) {
-            const WorkItem w = items[wi];
+        int acc = 0, it = 0;
+        for (int v = blockIdx.x; v < n_tasks; v += G, acc++, it += nk) {
+            const Item w = tab.item(v / split);
+            const int n0 = (v % split) * nb;
             const int a = acc & 1;
+            const bool live = row < w.cnt;
+            const float gw = live ? lgate[(size_t)w.e * T + w.m0 + row] : 0.0f;
             mbar_wait(&tfull[a], (uint32_t)(acc >> 1) & 1u, status, lim);
             tc_fence_after();
-            const bool live = row < w.cnt;
-            const float gw = live ? perm_gate[w.a0 + row] : 0.0f;
-            const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(a * NB);
-#pragma unroll 1
-            for (int c = 0; c < 64; c += 32) {
-                uint32_t u[32];
-                tmem_ld32(base + (uint32_t)(NB == 128 ? 64 + c : c), u);
-                float h[32];
-                if (NB == 128) {
-                    uint32_t g[32];
-                    tmem_ld32(base + (uint32_t)c, g);
-                    tmem_ld_wait();
+            if (32 * q < w.cnt) {
+                // a single chunk is in the accumulator of the MMA warp that took it
+                const uint32_t b0 = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(a * 256);
+                const bool both = nk > 1;
+                const uint32_t base = both ? b0 : b0 + (uint32_t)((it & 1) * 128);
+                auto sums = [&](int c, uint32_t (&r)[16]) {
+                    tmem_ld16(base + (uint32_t)c, r);
+                    if (both) {
+                        uint32_t o[16];
+                        tmem_ld16(b0 + (uint32_t)(128 + c), o);
+                        tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 32; i++) h[i] = act_h(PP_ACT_SWIGLU, __uint_as_float(u[i]), __uint_as_float(g[i])) * gw;
-                } else {
-                    tmem_ld_wait();
+                        for (int i = 0; i < 16; i++) r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(o[i]));
+                    } else {
+                        tmem_ld_wait();
+                    }
+                };
+                for (int c = 0; c < nb; c += 16) {
+                    uint32_t u[16];
+                    float h[16];
+                    sums(gated ? nb + c : c, u);
+                    if (gated) {
+                        uint32_t g[16];
+                        sums(c, g);
 #pragma unroll
-                    for (int i = 0; i < 32; i++) h[i] = act_h(act, __uint_as_float(u[i]), 0.0f) * gw;
-                }
-                if (live) {
-                    uint4* dst = reinterpret_cast<uint4*>(H + (size_t)(w.a0 + row) * 64 + c);
+                        for (int i = 0; i < 16; i++) h[i] = act_h(PP_ACT_SWIGLU, __uint_as_float(u[i]), __uint_as_float(g[i])) * gw;
+                    } else {
 #pragma unroll
-                    for (int v = 0; v < 4; v++)
-                        dst[v] = make_uint4(pack_bf16x2(h[8 * v], h[8 * v + 1]), pack_bf16x2(h[8 * v + 2], h[8 * v + 3]),
-                                            pack_bf16x2(h[8 * v + 4], h[8 * v + 5]), pack_bf16x2(h[8 * v + 6], h[8 * v + 7]));
+                        for (int i = 0; i < 16; i++) h[i] = act_h(act, __uint_as_float(u[i]), 0.0f) * gw;
+                    }
+                    if (live) {
+                        uint4* dst = reinterpret_cast<uint4*>(H + (size_t)(w.a0 + row) * 64 + n0 + c);
+#pragma unroll
+                        for (int k = 0; k < 2; k++)
+                            dst[k] = make_uint4(pack_bf16x2(h[8 * k], h[8 * k + 1]), pack_bf16x2(h[8 * k + 2], h[8 * k + 3]),
+                                                pack_bf16x2(h[8 * k + 4], h[8 * k + 5]), pack_bf16x2(h[8 * k + 6], h[8 * k + 7]));
+                    }
                 }
             }
             tc_fence_before();
@@ -551,23 +635,228 @@ __global__ void __launch_bounds__(kGuThreads, 1)
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, kCols < 32 ? 32 : kCols);
+    if (warp == kGuProd) tmem_dealloc(tmem, 512);
 }
 
-PP_DEVINL bool jt_first_overflow(const WorkItem& w, long long ycap) { return (long long)w.a0 + w.cnt > ycap; }
-
 // ============================================================== grouped down
-// Persistent over work items: an item's H tile is loaded once and the njt
+// (128-row tile of W_down, work item) pairs, tile by tile, dealt to the CTAs in
+// equal consecutive runs: D[128 rows x N] = W_down[tile, expert] * H_item^T,
+// N = the item's tokens padded to 16.  Weights are the M operand, so a tile's
+// epilogue costs by the tokens that there are and every warp has rows to store;
+// with tokens as M, one warp held all 12 tokens of a short prompt's item (45 us
+// at 333 tokens of the 7B shape for 90 MB of weights).  Tile by tile, a CTA
+// reads the 128-byte column blocks of consecutive experts, neighbours in a row
+// of W_down, and an expert's items share its block in L2.  Bound: HBM (W_down
+// and the rows of Y).  A pair's round trip (MMA, commit, TMEM load) is about
+// 1 us: four accumulators, released as soon as they are in registers.  The
+// 32-token groups of a pair are transposed through shared memory and leave as
+// one 256-byte bulk copy per token (4-byte stores, 64 bytes to a row, took
+// 1.6-2.2 us per pair: 94 us at 2048 tokens of the 13B shape).
+constexpr int kDnEpi = 8;  // epilogue warps: two sets of four (TMEM lane quarters), on alternating 32 tokens
+constexpr int kDnThreads = (2 + kDnEpi) * 32;
+constexpr int kDnStages = 12, kDnAcc = 4;
+constexpr int kDnBox = 32;               // H rows of a TMA box
+constexpr int kDnPitch = 128 * 2 + 16;   // staged token row
+constexpr int kDnStageOut = 32 * kDnPitch;
+constexpr size_t kDnRing = 172 * 1024;   // followed by 2 staging areas per set of epilogue warps
+
+// Position in the pairs of a call: item `it` of tile rt is work item `sub` of
+// expert e.
+struct DownPos {
+    const ItemTable& tab;
+    int rt, it, e, sub;
+    PP_DEVINL DownPos(const ItemTable& t, long long p) : tab(t) {
+        const int n = t.n_items();
+        rt = (int)(p / n);
+        it = (int)(p - (long long)rt * n);
+        const Item w = t.item(it);
+        e = w.e;
+        sub = w.m0 / 128;
+    }
+    PP_DEVINL int a0() const { return tab.off[e] + 128 * sub; }
+    PP_DEVINL int count() const { return min(128, tab.off[e + 1] - a0()); }
+    PP_DEVINL void next() {
+        if (++it == tab.n_items()) {
+            it = 0;
+            rt++;
+            e = 0;
+            sub = 0;
+        } else if (++sub < tab.ib[e + 1] - tab.ib[e]) {
+            return;
+        } else {
+            e++;
+            sub = 0;
+        }
+        while (tab.ib[e + 1] == tab.ib[e]) e++;  // (n_items > 0)
+    }
+};
+
+__global__ void __launch_bounds__(kDnThreads, 1)
+    down_gemm_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
+                     const int* __restrict__ cnt, const int* __restrict__ ltok, int T, int E, int d, int nrt,
+                     __nv_bfloat16* Y, long long ycap, float* yacc, int* overflow, unsigned* status, uint64_t lim) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    __shared__ uint64_t full[kDnStages], empty[kDnStages], tfull[kDnAcc], tempty[kDnAcc];
+    __shared__ uint32_t taddr_s;
+    __shared__ ItemTable tab;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kDnStages; i++) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < kDnAcc; i++) {
+            mbar_init(&tfull[i], 1);
+            mbar_init(&tempty[i], kDnEpi);
+        }
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(&taddr_s, kDnAcc * 128);
+        tmem_relinquish();
+    }
+    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
+    pdl_launch_dependents();
+    tab.build(cnt, E);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = taddr_s;
+    const long long P = (long long)tab.n_items() * nrt;
+    const long long p0 = P * blockIdx.x / gridDim.x;
+    const int n = (int)(P * (blockIdx.x + 1) / gridDim.x - p0);
+    // H tiles in boxes of kDnBox rows, as many as the longest item needs
+    const int nbox = (tab.longest + kDnBox - 1) / kDnBox, stage = kTileBytesA + nbox * kDnBox * 128;
+    const int nst = min(kDnStages, (int)kDnRing / stage);
+
+    if (n > 0 && warp == 0) {
+        if (lane == 0) {
+            DownPos w(tab, p0);
+            int s = 0;
+            uint32_t ph = 0;
+            for (int i = 0; i < n; i++) {
+                if (i >= nst) mbar_wait(&empty[s], ph ^ 1u, status, lim);
+                mbar_arrive_expect_tx(&full[s], (uint32_t)stage);
+                unsigned char* st = smem + (size_t)s * stage;
+                tma_load_2d(st, &map_wd, w.e * 64, w.rt * 128, &full[s]);
+                for (int b = 0; b < nbox; b++)
+                    tma_load_2d(st + kTileBytesA + b * kDnBox * 128, &map_h, 0, w.a0() + b * kDnBox, &full[s]);
+                if (++s == nst) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+                if (i + 1 < n) w.next();
+            }
+        }
+        __syncwarp();
+    } else if (n > 0 && warp == 1) {
+        if (lane == 0) {
+            DownPos w(tab, p0);
+            int s = 0, a = 0;
+            uint32_t ph = 0, aph = 0;
+            for (int i = 0; i < n; i++) {
+                if (i >= kDnAcc) mbar_wait(&tempty[a], aph ^ 1u, status, lim);
+                mbar_wait(&full[s], ph, status, lim);
+                tc_fence_after();
+                unsigned char* st = smem + (size_t)s * stage;
+                umma_k64(tmem + (uint32_t)(a * 128), st, st + kTileBytesA, idesc_bf16_m128((w.count() + 15) & ~15), false);
+                umma_commit(&empty[s]);
+                umma_commit(&tfull[a]);
+                if (++s == nst) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+                if (++a == kDnAcc) {
+                    a = 0;
+                    aph ^= 1u;
+                }
+                if (i + 1 < n) w.next();
+            }
+        }
+        __syncwarp();
+    } else if (n > 0) {
+        const int q = warp & 3, set = (warp - 2) >> 2;
+        unsigned char* out_s = smem + kDnRing + (size_t)set * 2 * kDnStageOut;
+        DownPos w(tab, p0);
+        int a = 0, buf = 0;
+        uint32_t aph = 0;
+        for (int i = 0; i < n; i++) {
+            const int m = w.count(), a0 = w.a0();
+            const bool spill = (long long)a0 + m > ycap;  // some of the item's rows go to yacc
+            mbar_wait(&tfull[a], aph, status, lim);
+            tc_fence_after();
+            const int row = w.rt * 128 + 32 * q + lane;  // output element
+            const uint32_t rbytes = (uint32_t)min(128, d - w.rt * 128) * 2u;
+            if (32 * set >= m) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tempty[a]);
+            }
+            for (int c = 32 * set; c < m; c += 64) {
+                uint32_t v[32];
+                tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(a * 128 + c), v);
+                tmem_ld_wait();
+                if (c + 64 >= m) {  // the accumulator is in registers
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tempty[a]);
+                }
+                if (!spill) {
+                    // this thread's copies out of the buffer, two groups ago, have been read
+                    bulk_wait_read<1>();
+                    named_bar_sync(1 + set, 128);
+                    unsigned char* sb = out_s + buf * kDnStageOut;
+                    __nv_bfloat16* col = reinterpret_cast<__nv_bfloat16*>(sb) + 32 * q + lane;
+#pragma unroll
+                    for (int k = 0; k < 32; k++) {
+                        if ((k & 7) == 0 && c + k >= m) break;
+                        col[(size_t)k * (kDnPitch / 2)] = __float2bfloat16_rn(__uint_as_float(v[k]));
+                    }
+                    fence_proxy_async_smem();
+                    named_bar_sync(1 + set, 128);
+                    // warp q sends tokens q, q + 4, ... of the group
+                    const int t = 4 * lane + q;
+                    if (lane < 8 && c + t < m)
+                        bulk_s2g(Y + (size_t)(a0 + c + t) * d + w.rt * 128, sb + t * kDnPitch, rbytes);
+                    bulk_commit();
+                    buf ^= 1;
+                } else if (row < d) {
+#pragma unroll
+                    for (int k = 0; k < 32; k++) {
+                        const int t = c + k;
+                        if (t >= m) break;
+                        const float val = __uint_as_float(v[k]);
+                        if ((long long)a0 + t < ycap)
+                            Y[(size_t)(a0 + t) * d + row] = __float2bfloat16_rn(val);
+                        else
+                            atomicAdd(&yacc[(size_t)ltok[(size_t)w.e * T + 128 * w.sub + t] * d + row], val);
+                    }
+                    if (lane == 0) *overflow = 1;
+                }
+            }
+            if (++a == kDnAcc) {
+                a = 0;
+                aph ^= 1u;
+            }
+            if (i + 1 < n) w.next();
+        }
+        bulk_wait_all();  // the stores are done before the CTA's shared memory goes away
+        __syncwarp();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem, kDnAcc * 128);
+}
+
+// Down projection of many tokens per expert (more than kDownRowsMinT tokens),
+// tokens as the M operand.  Persistent over work items: an item's H tile is loaded once and the njt
 // 256-wide slices of d stream through the B ring.  Two 256-column TMEM
 // accumulators overlap the reduction epilogue with the next slice's MMAs.
 __global__ void __launch_bounds__(kTcThreads, 1)
-    down_gemm_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
-                     const __grid_constant__ CUtensorMap map_y, const WorkItem* __restrict__ items,
-                     const int* __restrict__ n_items_p,
-                     const int* __restrict__ perm_token, int d, int njt, __nv_bfloat16* Y, long long ycap,
+    down_rows_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
+                     const __grid_constant__ CUtensorMap map_y, const int* __restrict__ cnt,
+                     const int* __restrict__ ltok, int T, int E, int d, int njt, __nv_bfloat16* Y, long long ycap,
                      float* yacc, int* overflow, unsigned* status, uint64_t lim) {
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
     constexpr int kStages = 4;
     constexpr int kTileB = 256 * 128;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -577,7 +866,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __shared__ uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], afull, aempty;
     __shared__ uint32_t taddr_s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_items = *n_items_p;
+    __shared__ ItemTable tab;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; i++) {
             mbar_init(&full[i], 1);
@@ -595,16 +884,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tmem_alloc(&taddr_s, 512);
         tmem_relinquish();
     }
+    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
+    pdl_launch_dependents();
+    tab.build(cnt, E);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = taddr_s;
+    const int n_items = tab.n_items();
 
     if (warp == 0) {
         if (lane == 0) {
             int it = 0, ii = 0;
             for (int v = blockIdx.x; v < n_items; v += gridDim.x, ii++) {
-                const WorkItem w = items[v];
+                const Item w = tab.item(v);
                 if (ii >= 1) mbar_wait(&aempty, (uint32_t)(ii - 1) & 1u, status, lim);
                 mbar_arrive_expect_tx(&afull, kTileBytesA);
                 tma_load_2d(tileA, &map_h, 0, w.a0, &afull);
@@ -645,16 +938,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         unsigned char* stage = smem + kTileBytesA + (size_t)kStages * kTileB + (size_t)q * 16384;
         int acc = 0;
         for (int v = blockIdx.x; v < n_items; v += gridDim.x) {
-            const WorkItem w = items[v];
+            const Item w = tab.item(v);
             const bool live = row < w.cnt;
             const bool group_live = 32 * q < w.cnt;  // any live row in this warp's 32 rows
             // all 32 rows live and inside Y: the group's rows go out as 2-D bulk stores
             const bool group_full = 32 * q + 32 <= w.cnt && (long long)w.a0 + 32 * q + 32 <= ycap;
             const long long arow = (long long)w.a0 + row;
             const bool in_buf = live && arow < ycap;
-            const int tok = live && !in_buf ? perm_token[arow] : -1;
+            const int tok = live && !in_buf ? ltok[(size_t)w.e * T + w.m0 + row] : -1;
             float* yrow = tok >= 0 ? yacc + (size_t)tok * d : nullptr;
-            if (tok >= 0 && jt_first_overflow(w, ycap)) *overflow = 1;
+            if (tok >= 0) *overflow = 1;
             __nv_bfloat16* Yrow = in_buf ? Y + (size_t)arow * d : nullptr;
             for (int jt = 0; jt < njt; jt++, acc++) {
                 const int a = acc & 1;
@@ -737,7 +1030,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // cleared again).  Grid (T, ceil(d / 1024)): 128 threads of 8 columns each.
 // The expert list is built in parallel: 128 experts per round, compacted in
 // ascending order with ballots.
-__global__ void __launch_bounds__(128) combine_kernel(const uint32_t* __restrict__ bits, const int* __restrict__ invpos,
+__global__ void __launch_bounds__(128) combine_kernel(const uint32_t* __restrict__ bits, const int* __restrict__ slot_of,
+                                                      const int* __restrict__ offsets,
                                                       const __nv_bfloat16* __restrict__ Y, long long ycap,
                                                       float* yacc, const int* __restrict__ overflow, int T, int E,
                                                       int d, __nv_bfloat16* y) {
@@ -750,7 +1044,7 @@ __global__ void __launch_bounds__(128) combine_kernel(const uint32_t* __restrict
     for (int e0 = 0; e0 < E; e0 += 128) {
         const int e = e0 + tid;
         bool on = e < E && ((bits[(size_t)t * 8 + (e >> 5)] >> (e & 31)) & 1u);
-        const int pos = on ? invpos[(size_t)t * E + e] : 0;
+        const int pos = on ? offsets[e] + slot_of[(size_t)t * E + e] : 0;
         on = on && pos < ycap;
         const unsigned bal = __ballot_sync(kFull, on);
         if (lane == 0) wn_s[warp] = __popc(bal);
@@ -796,12 +1090,12 @@ namespace {
 
 template <int NE>
 cudaError_t launch_router(const CUtensorMap& mx, const CUtensorMap& mwr, int T, int E, int nk, int kpb, int nsplit,
-                          float* part, unsigned* status, uint64_t lim, cudaStream_t st) {
+                          float* part, int* cnt, int* overflow, unsigned* status, uint64_t lim, cudaStream_t st) {
     const size_t smem = 4 * (size_t)(kTileBytesA + NE * 128) + 1024;
     cudaError_t e = set_smem(router_gemm_kernel<NE>, smem);
     if (e != cudaSuccess) return e;
     PP_LAUNCH(router_gemm_kernel<NE>, dim3((T + 127) / 128, nsplit), dim3(kTcThreads), smem, st, mx, mwr, T, E, nk,
-        kpb, part, status, lim);
+        kpb, part, cnt, overflow, status, lim);
     return cudaGetLastError();
 }
 
@@ -815,7 +1109,6 @@ GroupedPlan grouped_plan(int T, int d, int E, int sms) {
     const int ns = std::max(1, std::min(sms / mt, std::min(g.nk / 4, 64)));
     g.kpb = (g.nk + ns - 1) / ns;
     g.nsplit = (g.nk + g.kpb - 1) / g.kpb;
-    g.max_items = (int)std::min<long long>((long long)T * E / 128 + E + 1, (long long)T * E);  // 128-row items
     g.nnz_max = (long long)T * E;
     g.ycap = (long long)T * std::min(E, 64);  // assignment rows kept for the combine
     return g;
@@ -825,41 +1118,46 @@ cudaError_t grouped_route(const GroupedArgs& a, cudaStream_t st) {
     const GroupedPlan& g = a.plan;
     CUtensorMap mx, mwr;
     const int NE = router_ne(a.E);
+    int* cnt = a.bits ? a.cnt : nullptr;  // the FFN's lists
     if (!encode_2d(&mx, a.x, a.d, a.T, 64, 128) || !encode_2d(&mwr, a.Wr, a.d, a.E, 64, NE)) return cudaErrorInvalidValue;
     cudaError_t e;
     switch (NE) {
-        case 32: e = launch_router<32>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, a.status, a.timeout_ns, st); break;
-        case 64: e = launch_router<64>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, a.status, a.timeout_ns, st); break;
-        case 128: e = launch_router<128>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, a.status, a.timeout_ns, st); break;
-        case 160: e = launch_router<160>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, a.status, a.timeout_ns, st); break;
-        case 192: e = launch_router<192>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, a.status, a.timeout_ns, st); break;
-        case 224: e = launch_router<224>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, a.status, a.timeout_ns, st); break;
-        default: e = launch_router<256>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, a.status, a.timeout_ns, st); break;
+        case 32: e = launch_router<32>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
+        case 64: e = launch_router<64>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
+        case 128: e = launch_router<128>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
+        case 160: e = launch_router<160>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
+        case 192: e = launch_router<192>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
+        case 224: e = launch_router<224>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
+        default: e = launch_router<256>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
     }
     if (e != cudaSuccess) return e;
-    const bool mass_cut = (a.rule == PP_SEL_MIN_PREFIX || a.rule == PP_SEL_PAPER) && a.p < 1.0f;
-    if (mass_cut || a.T <= kCtaSelectMaxTokens) {
-        PP_LAUNCH(select_part_cta_kernel, dim3(a.T), dim3(256), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-            a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status);
+    if (a.T <= kCtaSelectMaxTokens) {  // pp_route: the union kernel makes its own selection
+        PP_LAUNCH(select_part_cta_kernel, dim3(a.T), dim3(256), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule, a.gate,
+                  a.ids, a.counts, a.gates, a.logits_out, a.status);
         return cudaGetLastError();
     }
     const dim3 grid((a.T + 7) / 8), block(256);
+    const Lists lists{a.cnt, a.ltok, a.lgate, a.slot_of};
+#define PP_SELECT(S)                                                                                                   \
+    PP_LAUNCH(select_warp_kernel<S>, grid, block, 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule, a.gate, a.ids, a.counts, \
+              a.gates, a.logits_out, a.bits, lists, a.status)
     switch (sel_slots_for(a.E)) {
-        case 1: PP_LAUNCH(select_part_kernel<1>, dim3(grid), dim3(block), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status); break;
-        case 2: PP_LAUNCH(select_part_kernel<2>, dim3(grid), dim3(block), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status); break;
-        case 4: PP_LAUNCH(select_part_kernel<4>, dim3(grid), dim3(block), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status); break;
-        default: PP_LAUNCH(select_part_kernel<8>, dim3(grid), dim3(block), 0, st, a.part, g.nsplit, a.T, a.E, a.p, a.rule,
-                a.gate, a.ids, a.counts, a.gates, a.logits_out, a.bits, a.gexp, a.status); break;
+        case 1: PP_SELECT(1); break;
+        case 2: PP_SELECT(2); break;
+        case 4: PP_SELECT(4); break;
+        default: PP_SELECT(8); break;
     }
+#undef PP_SELECT
     return cudaGetLastError();
 }
 
 cudaError_t grouped_load_selection(const GroupedArgs& a, cudaStream_t st) {
+    const bool lists = a.cnt != nullptr && a.T > kUnionMaxT;
     PP_LAUNCH(dispatch_bits_kernel, dim3((a.T + 7) / 8), dim3(256), 0, st, a.ids, a.counts, a.gates, a.T, a.E, a.bits,
-              a.gexp, a.status);
+              a.gexp, lists ? a.cnt : nullptr, a.overflow, a.status);
+    if (lists)
+        PP_LAUNCH(dispatch_list_kernel, dim3((a.T + 7) / 8), dim3(256), 0, st, a.bits, a.gexp, a.T, a.E,
+                  Lists{a.cnt, a.ltok, a.lgate, a.slot_of});
     return cudaGetLastError();
 }
 
@@ -867,48 +1165,36 @@ cudaError_t grouped_ffn(const GroupedArgs& a, int sms, cudaStream_t st) {
     if (a.T <= kUnionMaxT) return union_layer(a, false, sms, st);
     const GroupedPlan& g = a.plan;
     const bool gated = a.act == PP_ACT_SWIGLU;
-    cudaError_t e;
-    // dispatch
-    const int nblk = (a.T + kDispBlock - 1) / kDispBlock;
-    PP_LAUNCH(dispatch_count_kernel, dim3(nblk), dim3(kDispBlock), 0, st, a.bits, a.T, a.E, a.wcnt, a.blkcnt);
-    PP_LAUNCH(dispatch_scan_kernel, dim3(1), dim3(kMaxExperts), 0, st, a.blkcnt, nblk, a.E, a.offsets, a.blkbase,
-              reinterpret_cast<WorkItem*>(a.items), a.n_items, a.overflow);
-    PP_LAUNCH(dispatch_scatter_kernel, dim3(nblk, std::min(8, a.E)), dim3(kDispBlock), 0, st, a.bits, a.gexp, a.T,
-              a.E, a.wcnt, a.blkbase, a.perm_token, a.perm_gate, a.invpos);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // grouped gate/up
-    CUtensorMap mwg, mwu, mh, mwd;
-    if (!encode_2d(&mwu, a.Wu, a.d, (uint64_t)a.E * 64, 64, 64) ||
-        !encode_2d(&mwg, gated ? a.Wg : a.Wu, a.d, (uint64_t)a.E * 64, 64, 64) ||
-        !encode_2d(&mh, a.H, 64, (uint64_t)g.nnz_max + 128, 64, 128) ||
-        !encode_2d(&mwd, a.Wd, (uint64_t)a.E * 64, a.d, 64, 256, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
+    const uint64_t rows = (uint64_t)a.E * 64;
+    CUtensorMap mx, mwg, mwu, mh, mwd;
+    if (!encode_2d(&mx, a.x, a.d, a.T, 64, 1) || !encode_2d(&mwu, a.Wu, a.d, rows, 64, kGuBox) ||
+        !encode_2d(&mwg, gated ? a.Wg : a.Wu, a.d, rows, 64, kGuBox) ||
+        !encode_2d(&mh, a.H, 64, (uint64_t)g.nnz_max + 128, 64, kDnBox) ||
+        !encode_2d(&mwd, a.Wd, rows, a.d, 64, 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
         return cudaErrorInvalidValue;
-    const int grid = std::max(1, std::min(sms, g.max_items));
-    const WorkItem* items = reinterpret_cast<const WorkItem*>(a.items);
-    if (gated) {
-        const size_t smem = 6 * (size_t)(kTileBytesA + 128 * 128) + 1024;
-        if ((e = set_smem(gu_gemm_kernel<128>, smem)) != cudaSuccess) return e;
-        PP_LAUNCH(gu_gemm_kernel<128>, dim3(grid), dim3(kGuThreads), smem, st,
-            reinterpret_cast<const __nv_bfloat16*>(a.x), a.d, mwg, mwu, items, a.n_items, a.perm_token, a.perm_gate,
-            g.nk, a.act, a.H, a.status, a.timeout_ns);
+    const size_t gu_smem = kGuRing + kGuSlack + 1024, dn_smem = kDnRing + 4 * kDnStageOut + 1024;
+    cudaError_t e;
+    if ((e = set_smem(gu_gemm_kernel, gu_smem)) != cudaSuccess || (e = set_smem(down_gemm_kernel, dn_smem)) != cudaSuccess)
+        return e;
+    PP_LAUNCH(gu_gemm_kernel, dim3(sms), dim3(kGuThreads), gu_smem, st, mx, mwg, mwu, a.cnt, a.ltok, a.lgate, a.offsets, a.T,
+              a.E, g.nk, a.act, a.H, a.status, a.timeout_ns);
+    if (a.T <= kDownRowsMinT) {
+        PP_LAUNCH(down_gemm_kernel, dim3(sms), dim3(kDnThreads), dn_smem, st, mh, mwd, a.cnt, a.ltok, a.T, a.E, a.d,
+                  (a.d + 127) / 128, a.Y, g.ycap, a.yacc, a.overflow, a.status, a.timeout_ns);
     } else {
-        const size_t smem = 8 * (size_t)(kTileBytesA + 64 * 128) + 1024;
-        if ((e = set_smem(gu_gemm_kernel<64>, smem)) != cudaSuccess) return e;
-        PP_LAUNCH(gu_gemm_kernel<64>, dim3(grid), dim3(kGuThreads), smem, st,
-            reinterpret_cast<const __nv_bfloat16*>(a.x), a.d, mwg, mwu, items, a.n_items, a.perm_token, a.perm_gate,
-            g.nk, a.act, a.H, a.status, a.timeout_ns);
+        // A tile, the 4-stage W_down ring, 4 x 16 KB store staging
+        const size_t smem = (size_t)kTileBytesA + 4 * (size_t)256 * 128 + 4 * (size_t)16384 + 1024;
+        CUtensorMap mh128, mwd256, my;
+        if (!encode_2d(&mh128, a.H, 64, (uint64_t)g.nnz_max + 128, 64, 128) ||
+            !encode_2d(&mwd256, a.Wd, rows, a.d, 64, 256, CU_TENSOR_MAP_L2_PROMOTION_L2_128B) ||
+            !encode_2d(&my, a.Y, a.d, (uint64_t)g.ycap, 64, 32))
+            return cudaErrorInvalidValue;
+        if ((e = set_smem(down_rows_kernel, smem)) != cudaSuccess) return e;
+        PP_LAUNCH(down_rows_kernel, dim3(sms), dim3(kTcThreads), smem, st, mh128, mwd256, my, a.cnt, a.ltok, a.T, a.E, a.d,
+                  (a.d + 255) / 256, a.Y, g.ycap, a.yacc, a.overflow, a.status, a.timeout_ns);
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // grouped down: A tile, the 4-stage W_down ring, 4 x 16 KB store staging
-    const size_t smem = (size_t)kTileBytesA + 4 * (size_t)256 * 128 + 4 * (size_t)16384 + 1024;
-    CUtensorMap my;
-    if (!encode_2d(&my, a.Y, a.d, (uint64_t)g.ycap, 64, 32)) return cudaErrorInvalidValue;
-    if ((e = set_smem(down_gemm_kernel, smem)) != cudaSuccess) return e;
-    PP_LAUNCH(down_gemm_kernel, dim3(grid), dim3(kTcThreads), smem, st, mh, mwd, my, items, a.n_items, a.perm_token, a.d,
-              (a.d + 255) / 256, a.Y, g.ycap, a.yacc, a.overflow, a.status, a.timeout_ns);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    PP_LAUNCH(combine_kernel, dim3(a.T, (a.d + 1023) / 1024), dim3(128), 0, st, a.bits, a.invpos, a.Y, g.ycap,
-        a.yacc, a.overflow, a.T, a.E, a.d, reinterpret_cast<__nv_bfloat16*>(a.y));
+    PP_LAUNCH(combine_kernel, dim3(a.T, (a.d + 1023) / 1024), dim3(128), 0, st, a.bits, a.slot_of, a.offsets, a.Y, g.ycap,
+              a.yacc, a.overflow, a.T, a.E, a.d, reinterpret_cast<__nv_bfloat16*>(a.y));
     return cudaGetLastError();
 }
 

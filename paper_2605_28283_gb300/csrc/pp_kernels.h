@@ -151,7 +151,6 @@ struct GroupedPlan {
     int nk;          // 64-wide K chunks of d
     int kpb;         // router K chunks per split
     int nsplit;      // router K splits
-    int max_items;   // upper bound on 128-row work items
     long long nnz_max;  // upper bound on (token, expert) assignments
     long long ycap;     // rows of the bf16 assignment-output buffer
 };
@@ -173,15 +172,11 @@ struct GroupedArgs {
     float* part;        // [nsplit][T][E] router partials
     uint32_t* bits;     // [T][8]
     float* gexp;        // [T][E] gate weight per (token, expert)
-    int* invpos;        // [T][E] permuted row of (token, expert)
-    int* wcnt;          // [T/256][8][E] per-warp exclusive counts
-    int* blkcnt;        // [T/256][E]
-    int* blkbase;       // [T/256][E]
-    int* offsets;       // [E + 1]
-    void* items;        // [max_items] work items
-    int* n_items;
-    int* perm_token;    // [nnz_max]
-    float* perm_gate;   // [nnz_max]
+    int* slot_of;       // [T][E] slot of the token in the expert's list
+    int* cnt;           // [E] list lengths (more than kUnionMaxT tokens)
+    int* ltok;          // [E][T] tokens of each expert
+    float* lgate;       // [E][T] their gate weights
+    int* offsets;       // [E + 1] first row of each expert in H and Y
     __nv_bfloat16* H;   // [nnz_max + 128][64]
     __nv_bfloat16* Y;   // [ycap][d] assignment outputs
     float* yacc;        // [T][d] overflow accumulator, zero at rest

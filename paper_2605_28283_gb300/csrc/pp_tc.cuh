@@ -1,6 +1,5 @@
 // 5th-generation tensor core (tcgen05) helpers: TMEM allocation, UMMA
-// issue/commit, TMEM loads, shared-memory matrix descriptors, TMA gather4 and
-// vector reductions.  Inline PTX for sm_100-family (built for sm_103a).
+// issue/commit, TMEM loads, shared-memory matrix descriptors, TMA gather4.  Inline PTX for sm_100-family (built for sm_103a).
 //
 // Conventions used by the GEMM kernels:
 //  * D[128 x N] (fp32, TMEM lanes 0..127 = rows, columns 0..N-1) +=
@@ -120,21 +119,6 @@ PP_DEVINL void tma_prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
-// 16-byte cp.async global -> shared through L2 (not L1); src_bytes = 0
-// writes 16 zero bytes instead of reading.  Completion: cp_async_commit
-// closes a group, cp_async_wait<N> waits until at most N groups are pending.
-PP_DEVINL void cp_async_16(void* dst, const void* src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
-                 : "memory");
-}
-
-PP_DEVINL void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-
-template <int N>
-PP_DEVINL void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // 2-D tiled store shared -> global of one box (c0, c1 >= 0; the part of the
 // box past the tensor's extent is not written), tracked as a bulk group of
 // the issuing thread.
@@ -145,6 +129,18 @@ PP_DEVINL void tma_store_2d(const CUtensorMap* map, const void* src, int c0, int
                  : "memory");
 }
 
+// y[0..3] += v (fp32, one 16-byte vector reduction in L2)
+PP_DEVINL void red_add_v4(float* addr, float a, float b, float c, float d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
+}
+
+// 1-D bulk copy shared -> global (16-byte aligned, a multiple of 16 bytes),
+// tracked as a bulk group of the issuing thread.
+PP_DEVINL void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
+                 : "memory");
+}
 PP_DEVINL void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // the shared-memory sources of all but the N most recent committed bulk
 // groups have been read
@@ -154,12 +150,6 @@ PP_DEVINL void bulk_wait_read() {
 }
 // all committed bulk groups are complete (their global writes done)
 PP_DEVINL void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
-// y[0..3] += v (fp32, one 16-byte vector reduction in L2)
-PP_DEVINL void red_add_v4(float* addr, float a, float b, float c, float d) {
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
-                 : "memory");
-}
 
 PP_DEVINL uint32_t pack_bf16x2(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
