@@ -167,8 +167,9 @@ pp_status pp_layer(const pp_desc *desc, const void *x, int T, const void *W_r, c
    and then y = pp_layer(x).  x_prev, y_prev, x, y are [T][d]; gamma is [d];
    y_prev may be NULL (no residual term: the first layer) and gamma NULL
    (unit weights).  The sum and the mean square are fp32; x is stored in the
-   desc dtype and the layer reads exactly that x.  For up to 4 bf16 / 8 fp32
-   tokens the fused decode kernel forms x in its prologue (one launch);
+   desc dtype and the layer reads exactly that x.  Where the fused decode
+   kernel runs the layer (up to 4 bf16 / 8 fp32 tokens, but not 2 to 4 tokens
+   of a wide layer with a large p) it forms x in its prologue (one launch);
    otherwise one more kernel runs first.  x and y must not overlap x_prev,
    y_prev or each other (PP_ERR_INVALID_ARG); eps >= 0. */
 pp_status pp_layer_chained(const pp_desc *desc, const void *x_prev, const void *y_prev, const void *gamma,

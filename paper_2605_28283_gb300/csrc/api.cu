@@ -50,6 +50,31 @@ constexpr int kGroupedMinT = 5;
 
 bool use_grouped(const pp_desc& d, int T) { return d.dtype == PP_BF16 && T >= kGroupedMinT; }
 
+// Whole bf16 layers of 2 to 4 tokens that read enough weights for the union
+// kernel: it streams them at 5-6 TB/s behind about 26 us of phases, the fused
+// decode kernel at 1.9 TB/s (fp32 products of every token) behind 10.  How many
+// experts a call selects is known only on the device; the lines lie where the
+// two measured the same on the 7B, 8B and 13B shapes (270-425 MB of expert
+// weights, router logits with a spread of 2 to 4), in us, fused / union:
+//   8B, 4 tokens: p = 0.5 30/32, 0.7 44/37, 0.9 80/51, 1 146/77; top-4 31/33, top-12 48/39
+//   8B, 3 tokens: p = 0.7 32/34, 0.8 41/37, 0.9 58/45
+//   8B, 2 tokens: p = 0.9 38/41, 0.95 48/46, 1 94/77; top-12 26/34
+//   7B, 3 tokens: p = 0.8 36/36;  13B, 3 tokens: p = 0.8 37/36;  13B, 2 tokens: p = 0.95 43/45
+//   4 tokens, LTE at 0.95: 69/47; 3 tokens 50/43; 2 tokens 34/39
+// GPT-2-medium (17 MB) is faster fused up to p = 0.9 (4 tokens 18/23), slower
+// for every expert (33/24).
+constexpr size_t kUnionMinBytes = (size_t)128 << 20;
+
+bool use_union_small(const pp_desc& d, int T, float p) {
+    if (d.dtype != PP_BF16 || T < 2 || T >= kGroupedMinT) return false;
+    const size_t bytes = (size_t)(d.act == PP_ACT_SWIGLU ? 3 : 2) * d.d_ff * d.d_model * 2;
+    const bool mass = d.rule == PP_SEL_MIN_PREFIX || d.rule == PP_SEL_PAPER;
+    if (bytes < kUnionMinBytes) return mass && p >= 1.0f && T >= 3 && bytes >= ((size_t)16 << 20);
+    if (mass) return p >= (T == 4 ? 0.65f : T == 3 ? 0.8f : 0.97f);
+    if (d.rule == PP_SEL_TOPK) return T >= 3 && T * p >= 32.0f;
+    return T >= 3;  // LTE
+}
+
 // Workspace layout for calls with up to T tokens.
 struct Layout {
     size_t logits, ids, counts, gates, tlog, th, stats;
@@ -77,7 +102,7 @@ Layout layout(const pp_desc& d, int T) {
     L.tlog = take(8 * E * 8);
     L.th = take(E * 8 * kDExpert * 8);
     L.stats = take((size_t)router_stats_blocks((int)Tn) * (E + 2) * 8);
-    if (use_grouped(d, T)) {
+    if (d.dtype == PP_BF16 && T >= 2) {
         const GroupedPlan g = grouped_plan(T, d.d_model, d.n_experts, 152);
         L.part = take((size_t)g.nsplit * Tn * E * 4);
         L.bits = take(Tn * 8 * 4);
@@ -87,7 +112,7 @@ Layout layout(const pp_desc& d, int T) {
         L.ltok = take((size_t)g.nnz_max * 4);
         L.lgate = take((size_t)g.nnz_max * 4);
         L.offsets = take((E + 1) * 4);
-        L.H = take(((size_t)g.nnz_max + 128) * kDExpert * 2);
+        L.H = take(std::max((size_t)g.nnz_max + 128, 15 * E) * kDExpert * 2);  // three terms of up to 5 tokens
         L.Y = take((size_t)g.ycap * d.d_model * 2);
         L.yacc = take(Tn * (size_t)d.d_model * 4);
         L.overflow = take(16);
@@ -515,7 +540,7 @@ pp_status pp_layer(const pp_desc* desc, const void* x, int T, const void* W_r, c
     const Ws w = ws_views(*desc, T, ws);
     pp_selection s = sel_out ? *sel_out : pp_selection{w.ids, w.counts, w.gates, nullptr};
     const float kp = rule_kernel_param(desc->rule, p, desc->n_experts);
-    if (use_grouped(*desc, T)) {
+    if (use_grouped(*desc, T) || use_union_small(*desc, T, p)) {
         GroupedArgs a = grouped_args(*desc, T, ws, x, W_r, W_gate, W_up, W_down, kp, s, y);
         if (!sel_out) {  // nobody reads the rank order
             a.ids = a.counts = nullptr;
@@ -573,7 +598,7 @@ pp_status pp_layer_chained(const pp_desc* desc, const void* x_prev, const void* 
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Ws w = ws_views(*desc, T, ws);
     // fused: the decode kernel forms x in its prologue
-    if (!use_grouped(*desc, T)) {
+    if (!use_grouped(*desc, T) && !use_union_small(*desc, T, p)) {
         const int ts = decode_ts_limit(*desc);
         DecodePlan plan;
         int TS = 1;

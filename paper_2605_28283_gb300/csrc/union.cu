@@ -1,5 +1,5 @@
 // Batched path for a few to a few hundred tokens (bf16, up to kUnionMaxT
-// tokens): one cooperative launch, one CTA per SM, for the whole layer, with
+// tokens; below 5 where use_union in api.cu says so): one cooperative launch, one CTA per SM, for the whole layer, with
 // the FFN evaluated over the union of the batch's selected experts.
 //
 // At these sizes the weights are the traffic (a 64-token Llama-3-8B call reads
@@ -21,6 +21,10 @@
 //            in equal consecutive runs; a CTA accumulates a tile's experts in
 //            TMEM (fp32) and writes one partial tile per run
 //   reduce   y = the tile's partials in CTA order (deterministic)
+//
+// Up to 5 tokens the activations go through the down projection as three bf16
+// terms each (all 24 bits of the fp32 value), in columns that the MMA's 16 have
+// to spare; beyond, rounded to bf16.
 //
 // A grid barrier separates the phases (about 1.5 us, against 4-5 us for a
 // launch boundary with 200 KB CTAs, which cannot overlap their predecessors),
@@ -83,14 +87,14 @@ struct UnionArgs {
     CUtensorMap map_rx, map_wr;        // router: x in 128-row boxes, W_r in rn-row boxes
     CUtensorMap map_x, map_wg, map_wu; // gate/up
     CUtensorMap map_h, map_wd;         // down
-    int T, E, d, N, rn, nk, kpb, nsplit, mt, ntile, slots, act, gate, rule, do_route;
+    int T, E, d, N, terms, rn, nk, kpb, nsplit, mt, ntile, slots, act, gate, rule, do_route;
     float p;
     float* part;            // router partials [nsplit][T][E]
     int32_t *ids, *counts;  // selection outputs (NULL: not wanted)
     float *gates, *logits;
     uint32_t* bits;
     float* gexp;
-    __nv_bfloat16* H;       // [T][E * 64]: activations at union position * 64 + neuron
+    __nv_bfloat16* H;       // [terms * T][E * 64]: activations at union position * 64 + neuron
     float* dpart;
     const __nv_bfloat16* Wd;
     __nv_bfloat16* y;
@@ -266,6 +270,18 @@ PP_DEVINL void wd_prologue(const UnionArgs& a, UnionShared& sh, unsigned char* s
     __syncwarp();
 }
 
+// An activation in bf16, or as three bf16 terms (24 bits: the fp32 value) whose
+// rows are `next` elements apart.
+PP_DEVINL void store_h(__nv_bfloat16* p, float h, int terms, size_t next) {
+    const __nv_bfloat16 hi = __float2bfloat16_rn(h);
+    *p = hi;
+    if (terms == 1) return;
+    const float r = isfinite(h) ? h - __bfloat162float(hi) : 0.0f;
+    const __nv_bfloat16 mid = __float2bfloat16_rn(r);
+    p[next] = mid;
+    p[2 * next] = __float2bfloat16_rn(r - __bfloat162float(mid));
+}
+
 // Out of line: the epilogue runs once per launch and is bound by instruction
 // fetch (unrolled inline, 16 copies of the tanh form took 4.4 us at 16 tokens).
 static __device__ __noinline__ float union_act(int act, float u, float g) { return act_h(act, u, g); }
@@ -316,7 +332,7 @@ PP_DEVINL void gu_epilogue(const UnionArgs& a, UnionShared& sh, uint32_t tmem, i
                         const float o = __shfl_xor_sync(kFull, up ? e0 : e1, 8);
                         if (w != 0.0f) h = union_act(PP_ACT_SWIGLU, up ? e1 : o, up ? o : e0) * w;
                     }
-                    if (live && t < T) Hn[(size_t)t * ldh] = __float2bfloat16_rn(h);
+                    if (live && t < T) store_h(Hn + (size_t)t * ldh, h, a.terms, T * ldh);
                 }
             } else {
 #pragma unroll
@@ -324,7 +340,7 @@ PP_DEVINL void gu_epilogue(const UnionArgs& a, UnionShared& sh, uint32_t tmem, i
                     const int t = c + k;
                     const float w = live && t < T ? gt[t] : 0.0f;
                     const float h = w != 0.0f ? union_act(a.act, __uint_as_float(v[k]), 0.0f) * w : 0.0f;
-                    if (live && t < T) Hn[(size_t)t * ldh] = __float2bfloat16_rn(h);
+                    if (live && t < T) store_h(Hn + (size_t)t * ldh, h, a.terms, T * ldh);
                 }
             }
         }
@@ -462,8 +478,9 @@ static __device__ __noinline__ float own_experts_only(const UnionArgs& a, const 
         const int e = ul[u];
         if (__ldcg(a.gexp + (size_t)t * a.E + e) == 0.0f) continue;
         for (int k = 0; k < kDExpert; k++)
-            s = fmaf(__bfloat162float(a.H[(size_t)t * ld + u * kDExpert + k]),
-                     __bfloat162float(a.Wd[(size_t)row * ld + e * kDExpert + k]), s);
+            for (int m = a.terms - 1; m >= 0; m--)
+                s = fmaf(__bfloat162float(a.H[(size_t)(m * a.T + t) * ld + u * kDExpert + k]),
+                         __bfloat162float(a.Wd[(size_t)row * ld + e * kDExpert + k]), s);
     }
     return s;
 }
@@ -477,7 +494,7 @@ static __device__ __noinline__ float own_experts_only(const UnionArgs& a, const 
 // Only the H producer waits for the other CTAs' activations.
 PP_DEVINL void down_phase(const UnionArgs& a, UnionShared& sh, unsigned char* smem, uint32_t tmem, int nU) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int T = a.T, N = a.N, G = gridDim.x;
+    const int T = a.T, TT = a.terms * T, N = a.N, G = gridDim.x;  // TT columns are used
     const DownRun d(a, nU);
     const int mm = down_mma(N);
     const int L = a.ntile * nU, R = d.R, n = d.n, tile0 = d.tile0, first = d.first, stage = d.stage, nst = d.nst;
@@ -490,7 +507,7 @@ PP_DEVINL void down_phase(const UnionArgs& a, UnionShared& sh, unsigned char* sm
             const int acc = sg & 1;
             mbar_wait(&sh.dt[acc], (uint32_t)(sg >> 1) & 1u, a.status, a.lim);
             tc_fence_after();
-            float* out = a.dpart + ((size_t)blockIdx.x * a.slots + sg) * T * 128 + 32 * warp + lane;
+            float* out = a.dpart + ((size_t)blockIdx.x * a.slots + sg) * TT * 128 + 32 * warp + lane;
             const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(acc * mm * N);
             // pairs [s0, s1) of the run; a single pair is in the accumulator of its own MMA warp
             const int s0 = max(0, sg * nU - first), s1 = min(n, (sg + 1) * nU - first);
@@ -510,7 +527,7 @@ PP_DEVINL void down_phase(const UnionArgs& a, UnionShared& sh, unsigned char* sm
                 }
 #pragma unroll
                 for (int k = 0; k < 16; k++)
-                    if (c + k < T) out[(size_t)(c + k) * 128] = __uint_as_float(v[k]);
+                    if (c + k < TT) out[(size_t)(c + k) * 128] = __uint_as_float(v[k]);
             }
             tc_fence_before();
             __syncwarp();
@@ -588,22 +605,24 @@ PP_DEVINL void down_phase(const UnionArgs& a, UnionShared& sh, unsigned char* sm
             // the first run may have begun in an earlier tile; every other run
             // of the tile begins inside it (slot 0)
             const int slot0 = tile - run_begin(L, b0, R) / nU;
-            const float* base = a.dpart + (size_t)t * 128 + lane * 4;
-            for (int b = b0; b <= b1; b += 8) {
-                float4 v[8];
+            for (int m = a.terms - 1; m >= 0; m--) {  // the smallest term first
+                const float* base = a.dpart + (size_t)(m * T + t) * 128 + lane * 4;
+                for (int b = b0; b <= b1; b += 8) {
+                    float4 v[8];
 #pragma unroll
-                for (int k = 0; k < 8; k++)
-                    if (b + k <= b1)
-                        v[k] = __ldcg(reinterpret_cast<const float4*>(
-                            base + ((size_t)(b + k) * a.slots + (b + k == b0 ? slot0 : 0)) * T * 128));
+                    for (int k = 0; k < 8; k++)
+                        if (b + k <= b1)
+                            v[k] = __ldcg(reinterpret_cast<const float4*>(
+                                base + ((size_t)(b + k) * a.slots + (b + k == b0 ? slot0 : 0)) * TT * 128));
 #pragma unroll
-                for (int k = 0; k < 8; k++)
-                    if (b + k <= b1) {
-                        s[0] += v[k].x;
-                        s[1] += v[k].y;
-                        s[2] += v[k].z;
-                        s[3] += v[k].w;
-                    }
+                    for (int k = 0; k < 8; k++)
+                        if (b + k <= b1) {
+                            s[0] += v[k].x;
+                            s[1] += v[k].y;
+                            s[2] += v[k].z;
+                            s[3] += v[k].w;
+                        }
+                }
             }
 #pragma unroll
             for (int k = 0; k < 4; k++)
@@ -692,7 +711,7 @@ int pad16(int T) { return (T + 15) / 16 * 16; }
 size_t union_part_floats(int T, int d) {
     // [CTAs][slots][T][128] for any grid of up to kUnionMaxGrid CTAs (slots below)
     const size_t ntile = (size_t)(d + 127) / 128, rows = 3 * (size_t)kUnionMaxGrid + ntile;
-    return rows * 128 * (size_t)std::min(T, kUnionMaxT);
+    return rows * 128 * (size_t)std::min(std::max(T, 16), kUnionMaxT);
 }
 
 cudaError_t union_layer(const GroupedArgs& g, bool do_route, int sms, cudaStream_t st) {
@@ -705,6 +724,7 @@ cudaError_t union_layer(const GroupedArgs& g, bool do_route, int sms, cudaStream
     a.E = g.E;
     a.d = g.d;
     a.N = pad16(g.T);
+    a.terms = 3 * g.T <= 16 ? 3 : 1;  // the terms fit the MMA's 16 columns
     a.nk = g.plan.nk;
     a.mt = (g.T + 127) / 128;
     a.kpb = g.plan.kpb;
@@ -737,7 +757,7 @@ cudaError_t union_layer(const GroupedArgs& g, bool do_route, int sms, cudaStream
     const uint32_t box = gated ? 8 : 16;
     if ((do_route && (!encode_2d(&a.map_rx, g.x, g.d, g.T, 64, 128) || !encode_2d(&a.map_wr, g.Wr, g.d, g.E, 64, a.rn))) ||
         !encode_2d(&a.map_x, g.x, g.d, g.T, 64, a.N) || !encode_2d(&a.map_wu, g.Wu, g.d, rows, 64, box) ||
-        !encode_2d(&a.map_wg, gated ? g.Wg : g.Wu, g.d, rows, 64, box) || !encode_2d(&a.map_h, g.H, rows, g.T, 64, a.N) ||
+        !encode_2d(&a.map_wg, gated ? g.Wg : g.Wu, g.d, rows, 64, box) || !encode_2d(&a.map_h, g.H, rows, (uint64_t)a.terms * g.T, 64, a.N) ||
         !encode_2d(&a.map_wd, g.Wd, rows, g.d, 64, 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
         return cudaErrorInvalidValue;
     cudaError_t e = set_smem(union_layer_kernel, kUnionSmem);

@@ -100,3 +100,28 @@ def test_union_non_finite_weight_stays_with_its_expert(pp):
     assert not np.isfinite(b[uses[:, e]]).any()
     assert np.isfinite(b[~uses[:, e]]).all()
     assert rel_err_per_token(b[~uses[:, e]], a[~uses[:, e]]).max() <= Y_TOL["bf16"]
+
+
+@pytest.mark.parametrize("T,rule,p", [(2, "min_prefix", 1.0), (3, "min_prefix", 0.9), (4, "paper", 0.9), (4, "topk", 9.0),
+                                      (3, "lte", 0.95)])
+def test_union_small_batches_of_wide_layers(pp, T, rule, p):
+    """2 to 4 tokens that the union kernel runs instead of the fused decode
+    kernel: parity, and no less exact than the fused kernel (pp_layer_noalloc
+    always takes it).  Both sides' error is the rounding of y to bf16; 3 % is
+    four standard deviations of the ratio of two such errors over the 8192 or
+    more elements."""
+    import torch
+    layer_parity(pp, "llama3_8b_batched", T, p, rule)
+    w, L, (x, Wr, Wg, Wu, Wd) = _device_layer("llama3_8b_batched", T, 4096, 224)
+    desc = pp.make_desc(w.d_model, w.n_experts, w.dtype, w.act, "sigmoid", rule)
+    ws = pp.alloc_workspace(desc, T)
+    sels = [pp.Selection.empty(T, w.n_experts, "cuda") for _ in range(2)]
+    ys = [torch.empty_like(x) for _ in range(2)]
+    pp.pp_layer(desc, x, T, Wr, Wg, Wu, Wd, f32(p), sels[0], ys[0], ws)
+    pp.pp_layer_noalloc(desc, x, T, Wr, Wg, Wu, Wd, f32(p), sels[1], ys[1])
+    torch.cuda.synchronize()
+    counts, ids = to_host(sels[0].counts), to_host(sels[0].ids)
+    assert np.array_equal(counts, to_host(sels[1].counts)) and np.array_equal(ids, to_host(sels[1].ids))
+    ref = oracle.sparse_ffn(L.x, L.Wg, L.Wu, L.Wd, counts, ids, oracle.logits(L.x, L.Wr), w.n_experts, w.act, "sigmoid")
+    e = [np.linalg.norm(to_host(y).astype(np.float64) - ref) / np.linalg.norm(ref) for y in ys]
+    assert e[0] <= 1.03 * e[1], e
