@@ -2,6 +2,7 @@
 // and the bounded-wait test kernel.
 #include "pp_common.cuh"
 #include "pp_kernels.h"
+#include "pp_launch.h"
 #include "pp_select.cuh"
 
 namespace pp {
@@ -73,71 +74,88 @@ cudaError_t select_launch(const float* logits, int T, int E, float p, int rule, 
 
 // ------------------------------------------------------------ statistics
 // acc[0] += sum_t counts[t]; acc[1 + c] += #{t : counts[t] == c}  (s_FFN, Sec. 4.1)
-__global__ void stats_kernel(const int32_t* __restrict__ counts, int T, int E, unsigned long long* acc) {
-    __shared__ unsigned long long hist[kMaxExperts + 2];
-    for (int i = threadIdx.x; i < E + 2; i += blockDim.x) hist[i] = 0ull;
+// Bound: launch and L2 latency.  The sum is reduced over the warp and the
+// histogram kept in 32 bits (a thread's 64-bit shared atomics on the one sum
+// serialised the block: 16 us for 2048 tokens, 5 now, cold under ncu).
+__global__ void __launch_bounds__(256) stats_kernel(const int32_t* __restrict__ counts, int T, int E,
+                                                    unsigned long long* acc) {
+    __shared__ unsigned hist[kMaxExperts + 1];
+    pdl_wait();
+    pdl_launch_dependents();
+    for (int i = threadIdx.x; i <= E; i += blockDim.x) hist[i] = 0u;
     __syncthreads();
+    unsigned long long sum = 0ull;  // of this thread's tokens
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x) {
         int c = counts[t];
         c = c < 0 ? 0 : (c > E ? E : c);
-        atomicAdd(&hist[0], (unsigned long long)c);
-        atomicAdd(&hist[1 + c], 1ull);
+        sum += (unsigned)c;
+        atomicAdd(&hist[c], 1u);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&acc[0], sum);
     __syncthreads();
-    for (int i = threadIdx.x; i < E + 2; i += blockDim.x)
-        if (hist[i]) atomicAdd(&acc[i], hist[i]);
+    for (int i = threadIdx.x; i <= E; i += blockDim.x)
+        if (hist[i]) atomicAdd(&acc[1 + i], (unsigned long long)hist[i]);
 }
 
 cudaError_t stats_launch(const int32_t* counts, int T, int E, uint64_t* acc, cudaStream_t st) {
     if (T == 0) return cudaSuccess;
     const int blocks = std::min(152, (T + 255) / 256);
-    stats_kernel<<<blocks, 256, 0, st>>>(counts, T, E, reinterpret_cast<unsigned long long*>(acc));
-    return cudaGetLastError();
+    PP_LAUNCH(stats_kernel, dim3(blocks), dim3(256), 0, st, counts, T, E, reinterpret_cast<unsigned long long*>(acc));
+    return cudaSuccess;
 }
 
 // ------------------------------------------------------ router statistics
 // Forward values of the router terms of the training objective (Sec. 3.2,
 // Eq. entropy_loss and Eq. load_balance_loss; L_gate of Sec. 4.2.3) over a
 // batch of logits [T][E].  Pass 1: CTA b takes tokens [64 b, 64 b + 64),
-// warp w eight of them, lane l the experts l + 32 s.  Per token the softmax
+// warp w two of them (eight warps with eight each took 24 us for 2048 tokens,
+// a chain of eight tokens), lane l the experts l + 32 s.  Per token the softmax
 // is max-shifted in fp32.  part[b] = (column sums of p [E], sum of
 // p log(p + eps), sum of sigmoid(g)) over the CTA's tokens, fp32, reduced over
 // the warps in a fixed order.  Pass 2 (one CTA of 1024 threads) adds the
 // parts pairwise in a fixed tree order and combines the totals in fp64: the
 // result is deterministic.  (This GPU's fp64 pipe is narrow, so fp64 is kept
 // to the final scalars.)
-constexpr int kStatTok = 64;
+constexpr int kStatTok = 64, kStatWarps = 32;
 constexpr int kStatFinal = 1024;
 
-__global__ void __launch_bounds__(256) router_stats_part_kernel(const float* __restrict__ logits, int T, int E,
-                                                                float eps, float* __restrict__ part,
-                                                                unsigned* status) {
-    __shared__ float colw[8][kMaxExperts];
-    __shared__ float entw[8], gatew[8];
+__global__ void __launch_bounds__(kStatWarps * 32)
+    router_stats_part_kernel(const float* __restrict__ logits, int T, int E, float eps, float* __restrict__ part,
+                             unsigned* status) {
+    __shared__ float colw[kStatWarps][kMaxExperts];
+    __shared__ float entw[kStatWarps], gatew[kStatWarps];
+    pdl_wait();
+    pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = (E + 31) / 32;
+    constexpr int kPer = kStatTok / kStatWarps;
+    const int t0 = blockIdx.x * kStatTok + warp * kPer;
+    float g[kPer][8];  // the warp's tokens, all loads in flight
+#pragma unroll
+    for (int i = 0; i < kPer; i++)
+#pragma unroll
+        for (int s = 0; s < 8; s++)
+            g[i][s] = t0 + i < T && lane + 32 * s < E ? logits[(size_t)(t0 + i) * E + lane + 32 * s] : -INFINITY;
     float col[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     float ent = 0.0f, gsum = 0.0f;
-    const int per = kStatTok / 8;
-    const int tbeg = blockIdx.x * kStatTok + warp * per, tend = min(T, tbeg + per);
-    for (int t = tbeg; t < tend; t++) {
-        const float* row = logits + (size_t)t * E;
-        float g[8];
+#pragma unroll
+    for (int i = 0; i < kPer; i++) {
+        if (t0 + i >= T) break;
         bool fin = true;
         float m = -INFINITY;
 #pragma unroll
         for (int s = 0; s < 8; s++) {
-            const int j = lane + 32 * s;
-            g[s] = (s < S && j < E) ? row[j] : -INFINITY;
-            if (s < S && j < E) fin = fin && isfinite(g[s]);
-            m = fmaxf(m, g[s]);
+            if (lane + 32 * s < E) fin = fin && isfinite(g[i][s]);
+            m = fmaxf(m, g[i][s]);
         }
         fin = __all_sync(kFull, fin);
         m = warp_max(m);
         float e[8], z = 0.0f;
 #pragma unroll
         for (int s = 0; s < 8; s++) {
-            e[s] = (s < S && lane + 32 * s < E) ? expf(g[s] - m) : 0.0f;
+            e[s] = (s < S && lane + 32 * s < E) ? expf(g[i][s] - m) : 0.0f;
             z += e[s];
         }
         z = warp_sum(z);
@@ -148,7 +166,7 @@ __global__ void __launch_bounds__(256) router_stats_part_kernel(const float* __r
                 const float pj = e[s] / z;
                 col[s] += pj;
                 te += pj * logf(pj + eps);
-                tg += sigmoidf_(g[s]);
+                tg += sigmoidf_(g[i][s]);
             }
         }
         if (!fin) {
@@ -168,22 +186,22 @@ __global__ void __launch_bounds__(256) router_stats_part_kernel(const float* __r
         gatew[warp] = gsum;
     }
     __syncthreads();
+    // four threads per expert sum eight warps each, then pairwise
     float* out = part + (size_t)blockIdx.x * (E + 2);
-    for (int j = threadIdx.x; j < E; j += blockDim.x) {
-        float c = 0.0f;
+    const int j = threadIdx.x >> 2, q = threadIdx.x & 3;
+    float c = 0.0f;
+    if (j < E)
 #pragma unroll
-        for (int w = 0; w < 8; w++) c += colw[w][j];
-        out[j] = c;
-    }
-    if (threadIdx.x == 0) {
-        float a = 0.0f, b = 0.0f;
-#pragma unroll
-        for (int w = 0; w < 8; w++) {
-            a += entw[w];
-            b += gatew[w];
+        for (int w = 0; w < 8; w++) c += colw[q * 8 + w][j];
+    c += __shfl_xor_sync(kFull, c, 1);
+    c += __shfl_xor_sync(kFull, c, 2);
+    if (j < E && q == 0) out[j] = c;
+    if (warp == 0) {
+        const float a = warp_sum(entw[lane]), b = warp_sum(gatew[lane]);
+        if (lane == 0) {
+            out[E] = a;
+            out[E + 1] = b;
         }
-        out[E] = a;
-        out[E + 1] = b;
     }
 }
 
@@ -204,6 +222,8 @@ __global__ void __launch_bounds__(kStatFinal) router_stats_final_kernel(const fl
                                                                         int T, int E, double* __restrict__ out) {
     __shared__ float csum[4][kMaxExperts];
     __shared__ float red[kStatFinal / 32];
+    pdl_wait();
+    pdl_launch_dependents();
     // column sums: four threads per expert, each over a contiguous quarter of
     // the parts, eight loads in flight and a pairwise sum of each eight
     {
@@ -249,9 +269,9 @@ int router_stats_blocks(int T) { return (T + kStatTok - 1) / kStatTok; }
 cudaError_t router_stats_launch(const float* logits, int T, int E, float eps, float* part, double* out,
                                 unsigned* status, cudaStream_t st) {
     const int nblk = router_stats_blocks(T);
-    router_stats_part_kernel<<<nblk, 256, 0, st>>>(logits, T, E, eps, part, status);
-    router_stats_final_kernel<<<1, kStatFinal, 0, st>>>(part, nblk, T, E, out);
-    return cudaGetLastError();
+    PP_LAUNCH(router_stats_part_kernel, dim3(nblk), dim3(kStatWarps * 32), 0, st, logits, T, E, eps, part, status);
+    PP_LAUNCH(router_stats_final_kernel, dim3(1), dim3(kStatFinal), 0, st, part, nblk, T, E, out);
+    return cudaSuccess;
 }
 
 // ------------------------------------------------------- chained step
