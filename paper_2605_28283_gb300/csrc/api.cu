@@ -61,16 +61,18 @@ bool use_grouped(const pp_desc& d, int T) { return d.dtype == PP_BF16 && T >= kG
 //   8B, 2 tokens: p = 0.9 38/41, 0.95 48/46, 1 94/77; top-12 26/34
 //   7B, 3 tokens: p = 0.8 36/36;  13B, 3 tokens: p = 0.8 37/36;  13B, 2 tokens: p = 0.95 43/45
 //   4 tokens, LTE at 0.95: 69/47; 3 tokens 50/43; 2 tokens 34/39
-// GPT-2-medium (17 MB) is faster fused up to p = 0.9 (4 tokens 18/23), slower
-// for every expert (33/24).
+// GPT-2-medium (17 MB) is faster fused up to p = 0.95 (4 tokens at 0.9: 18/23).
 constexpr size_t kUnionMinBytes = (size_t)128 << 20;
 
+// Shapes and token counts of which some call may take the union kernel.
+bool union_small_shape(const pp_desc& d, int T) {
+    return d.dtype == PP_BF16 && T >= 2 && T < kGroupedMinT &&
+           (size_t)(d.act == PP_ACT_SWIGLU ? 3 : 2) * d.d_ff * d.d_model * 2 >= kUnionMinBytes;
+}
+
 bool use_union_small(const pp_desc& d, int T, float p) {
-    if (d.dtype != PP_BF16 || T < 2 || T >= kGroupedMinT) return false;
-    const size_t bytes = (size_t)(d.act == PP_ACT_SWIGLU ? 3 : 2) * d.d_ff * d.d_model * 2;
-    const bool mass = d.rule == PP_SEL_MIN_PREFIX || d.rule == PP_SEL_PAPER;
-    if (bytes < kUnionMinBytes) return mass && p >= 1.0f && T >= 3 && bytes >= ((size_t)16 << 20);
-    if (mass) return p >= (T == 4 ? 0.65f : T == 3 ? 0.8f : 0.97f);
+    if (!union_small_shape(d, T)) return false;
+    if (d.rule == PP_SEL_MIN_PREFIX || d.rule == PP_SEL_PAPER) return p >= (T == 4 ? 0.65f : T == 3 ? 0.8f : 0.97f);
     if (d.rule == PP_SEL_TOPK) return T >= 3 && T * p >= 32.0f;
     return T >= 3;  // LTE
 }
@@ -102,7 +104,7 @@ Layout layout(const pp_desc& d, int T) {
     L.tlog = take(8 * E * 8);
     L.th = take(E * 8 * kDExpert * 8);
     L.stats = take((size_t)router_stats_blocks((int)Tn) * (E + 2) * 8);
-    if (d.dtype == PP_BF16 && T >= 2) {
+    if (use_grouped(d, T) || union_small_shape(d, T)) {
         const GroupedPlan g = grouped_plan(T, d.d_model, d.n_experts, 152);
         L.part = take((size_t)g.nsplit * Tn * E * 4);
         L.bits = take(Tn * 8 * 4);

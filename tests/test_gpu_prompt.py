@@ -38,6 +38,37 @@ def test_prompt_large_lists(pp):
     layer_parity(pp, "llama3_8b_batched", 600, 0.95, d=320, E=12)
 
 
+@pytest.mark.parametrize("d,E,T,p", [(64, 1, 1025, 0.5), (64, 40, 1100, 0.8), (200, 12, 1300, 0.95), (1000, 70, 1030, 0.7),
+                                     (2312, 9, 1041, 0.9), (264, 100, 1027, 1.0)])
+@pytest.mark.parametrize("name", ["llama3_8b_batched", "gpt2m_gelu_bf16"])
+def test_prompt_down_projection_by_token_rows(pp, name, d, E, T, p):
+    """Above 1024 tokens the down projection has tokens as the M operand: full
+    and partial groups of 32 rows, partial column slices, and with p = 1 pairs
+    past the row buffer's capacity."""
+    layer_parity(pp, name, T, p, d=d, E=E)
+
+
+def test_prompt_repeated_calls(pp):
+    """Back to back on one workspace, alternating lengths (and so kernels): every
+    call gives the same bits."""
+    import torch
+    Ts, p = (1500, 300, 1100), f32(0.8)
+    w, L = layer_inputs("llama3_8b_batched", max(Ts), d=1304, E=30)
+    desc = pp.make_desc(w.d_model, w.n_experts, w.dtype, w.act)
+    ws = pp.alloc_workspace(desc, max(Ts))
+    x, Wr, Wg, Wu, Wd = (dev(a) for a in (L.x, L.Wr, L.Wg, L.Wu, L.Wd))
+    ref = {}
+    for rep in range(8):
+        for T in Ts:
+            y = torch.empty_like(x[:T])
+            pp.pp_layer(desc, x, T, Wr, Wg, Wu, Wd, p, None, y, ws)
+            ref.setdefault(T, []).append(y)
+    torch.cuda.synchronize()
+    assert pp.pp_get_device_status(ws) == pp.PP_OK
+    for T in Ts:
+        assert all(torch.equal(y, ref[T][0]) for y in ref[T]), T
+
+
 @pytest.mark.parametrize("E", [20, 50, 120, 250])
 @pytest.mark.parametrize("rule,p", [("min_prefix", 0.7), ("min_prefix", 1.0), ("paper", 0.9), ("topk", 6.0), ("lte", 0.9)])
 def test_prompt_route_matches_select(pp, E, rule, p):
