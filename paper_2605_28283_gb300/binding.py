@@ -102,19 +102,34 @@ def _check(s, what):
         raise PPError(s, what)
 
 
+# Arguments go to ctypes as plain integers (argtypes convert them): a c_void_p
+# object per pointer and a torch Stream object per call cost a small eager call
+# about as much host time as its launches.
 def _ptr(t):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_torch = None
+
+
+def _current_stream() -> int:
+    """cudaStream_t of torch's current stream on the current device."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    if not _torch.cuda.is_initialized():
+        return _torch.cuda.current_stream().cuda_stream
+    raw = getattr(_torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return _torch.cuda.current_stream().cuda_stream
+    return raw(_torch._C._cuda_getDevice())
 
 
 def _stream(stream):
     if stream is None:
-        import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return _current_stream()
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 def make_desc(d_model, n_experts, dtype="bf16", act="swiglu", gate="sigmoid", rule="min_prefix",
