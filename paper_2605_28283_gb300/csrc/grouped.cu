@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(kGuThreads, 1)
 // 32-token groups of a pair are transposed through shared memory and leave as
 // one 256-byte bulk copy per token (4-byte stores, 64 bytes to a row, took
 // 1.6-2.2 us per pair: 94 us at 2048 tokens of the 13B shape).
-constexpr int kDnEpi = 8;  // epilogue warps: two sets of four (TMEM lane quarters), on alternating 32 tokens
+constexpr int kDnEpi = 8;  // epilogue warps: two sets of four (TMEM lane quarters), on alternating 32 tokens or pairs
 constexpr int kDnThreads = (2 + kDnEpi) * 32;
 constexpr int kDnStages = 12, kDnAcc = 4;
 constexpr int kDnBox = 32;               // H rows of a TMA box
@@ -788,11 +788,13 @@ __global__ void __launch_bounds__(kDnThreads, 1)
             tc_fence_after();
             const int row = w.rt * 128 + 32 * q + lane;  // output element
             const uint32_t rbytes = (uint32_t)min(128, d - w.rt * 128) * 2u;
-            if (32 * set >= m) {
+            // items of one group: the sets take the pairs in turn
+            const int c0 = m > 32 ? 32 * set : set == (i & 1) ? 0 : m;
+            if (c0 >= m) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&tempty[a]);
             }
-            for (int c = 32 * set; c < m; c += 64) {
+            for (int c = c0; c < m; c += 64) {
                 uint32_t v[32];
                 tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(a * 128 + c), v);
                 tmem_ld_wait();
