@@ -179,7 +179,7 @@ PP_DEVINL void list_add(const Lists& l, int T, int E, int t, int e, float gv) {
 // until the rule stops, with the exact fixed-point masses of group_mass_cut, so
 // the decisions are the same.  An activated expert costs about 110 cycles and
 // nothing is sorted that is not activated: one CTA per token took 46 us for
-// 8192 tokens of 216 experts (7 activated each), this 12 us.  ids and gates
+// 8192 tokens of 216 experts (7 activated each), this 20 us (under ncu).  ids and gates
 // (together), counts, logits_out may be NULL; so may bits with the lists.
 template <int S>
 __global__ void __launch_bounds__(256)
@@ -450,7 +450,8 @@ struct ItemTable {
 // rows of a full chunk), if enough warps issue and enough stages are in flight
 // (a stage's round trip is about 1.4 us: the ring holds as many stages as the
 // longest item's rows leave room for, 16 at most; six fixed stages took 330 ns
-// per chunk of a 12-token item's half): a gather4 costs its warp about
+// per chunk of a 12-token item's half).  Under ncu: 8192 tokens of the 13B shape
+// 170 -> 100 us, 2048 tokens 93 -> 76, 333 tokens of the 7B shape 61 -> 57: a gather4 costs its warp about
 // 30 ns, so eight producer warps take 4 of a chunk's 32 gathers each (one
 // gather thread per row with cp.async, three stages in flight, took 400-580 ns
 // per chunk).  An MMA thread needs 55-64 cycles per MMA and about 300 for a
@@ -651,7 +652,8 @@ __global__ void __launch_bounds__(kGuThreads, 1)
 // 1 us: four accumulators, released as soon as they are in registers.  The
 // 32-token groups of a pair are transposed through shared memory and leave as
 // one 256-byte bulk copy per token (4-byte stores, 64 bytes to a row, took
-// 1.6-2.2 us per pair: 94 us at 2048 tokens of the 13B shape).
+// 1.6-2.2 us per pair: 94 us at 2048 tokens of the 13B shape).  333 tokens of
+// the 7B shape: 45 -> 31 us.
 constexpr int kDnEpi = 8;  // epilogue warps: two sets of four (TMEM lane quarters), on alternating 32 tokens or pairs
 constexpr int kDnThreads = (2 + kDnEpi) * 32;
 constexpr int kDnStages = 12, kDnAcc = 4;

@@ -145,11 +145,6 @@ PP_DEVINL void named_bar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// Arrive on a named barrier without waiting for it.
-PP_DEVINL void named_bar_arrive(int id, int nthreads) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
 // ---------------------------------------------------------- tagged words
 PP_DEVINL unsigned ld_acquire_gpu(const unsigned* p) {
     unsigned v;

@@ -188,6 +188,8 @@ struct GroupedArgs {
 };
 
 // -------------------------------------- union path (up to kUnionMaxT tokens)
+// 256 is the most columns an MMA has for the tokens (256 tokens of the 8B shape:
+// 125 us per layer against 140 by token lists).
 constexpr int kUnionMaxT = 256;
 constexpr int kUnionMaxGrid = 152;
 size_t union_part_floats(int T, int d);  // of GroupedArgs.dpart

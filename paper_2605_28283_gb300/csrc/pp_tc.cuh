@@ -1,5 +1,6 @@
 // 5th-generation tensor core (tcgen05) helpers: TMEM allocation, UMMA
-// issue/commit, TMEM loads, shared-memory matrix descriptors, TMA gather4.  Inline PTX for sm_100-family (built for sm_103a).
+// issue/commit, TMEM loads, shared-memory matrix descriptors, TMA gather4,
+// bulk stores.  Inline PTX for sm_100-family (built for sm_103a).
 //
 // Conventions used by the GEMM kernels:
 //  * D[128 x N] (fp32, TMEM lanes 0..127 = rows, columns 0..N-1) +=
@@ -112,11 +113,6 @@ PP_DEVINL void tma_gather4(void* dst, const CUtensorMap* map, int col, int r0, i
         "{%2, %3, %4, %5, %6}], [%7];" ::"r"(smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(col), "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(smem_u32(bar))
         : "memory");
-}
-
-// Fetch a tensor map (a kernel parameter) ahead of its first use.
-PP_DEVINL void tma_prefetch_map(const CUtensorMap* map) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
 // 2-D tiled store shared -> global of one box (c0, c1 >= 0; the part of the

@@ -76,7 +76,7 @@ cudaError_t select_launch(const float* logits, int T, int E, float p, int rule, 
 // acc[0] += sum_t counts[t]; acc[1 + c] += #{t : counts[t] == c}  (s_FFN, Sec. 4.1)
 // Bound: launch and L2 latency.  The sum is reduced over the warp and the
 // histogram kept in 32 bits (a thread's 64-bit shared atomics on the one sum
-// serialised the block: 16 us for 2048 tokens, 5 now, cold under ncu).
+// serialised the block: 16 us for 2048 tokens).
 __global__ void __launch_bounds__(256) stats_kernel(const int32_t* __restrict__ counts, int T, int E,
                                                     unsigned long long* acc) {
     __shared__ unsigned hist[kMaxExperts + 1];

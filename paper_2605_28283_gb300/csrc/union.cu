@@ -30,6 +30,9 @@
 // launch boundary with 200 KB CTAs, which cannot overlap their predecessors),
 // and the first W_down tiles of a CTA are in flight while it waits for the
 // others' activations.
+// Per layer of the 8B shape, against six kernels over 16-row items of whole
+// experts: 8 tokens 52 -> 39 us, 64 tokens 88 -> 75; GPT-2-medium, 16 tokens,
+// 28 -> 25.
 //
 // Warps: 0-3 producers of the gate/up ring and epilogues (TMEM lanes
 // 32 * warp ..), 4-5 MMA issue, 6 W_down producer, 7 H producer.
@@ -283,7 +286,7 @@ PP_DEVINL void store_h(__nv_bfloat16* p, float h, int terms, size_t next) {
 }
 
 // Out of line: the epilogue runs once per launch and is bound by instruction
-// fetch (unrolled inline, 16 copies of the tanh form took 4.4 us at 16 tokens).
+// fetch (unrolled inline, 16 copies of the tanh form took 4.4 us at 16 tokens, 3.6 now).
 static __device__ __noinline__ float union_act(int act, float u, float g) { return act_h(act, u, g); }
 
 // h = act(gate, up) * gate weight of the pass's units [base, base + nun), bf16,
@@ -292,6 +295,11 @@ static __device__ __noinline__ float union_act(int act, float u, float g) { retu
 // the expert (most do not: 5 % of the pairs at 64 tokens of the 8B shape) costs
 // a store of zero and no activation.  `halves`: the sums are those of two
 // accumulators.
+// UN: how far the loops over the tokens are unrolled.  A column block of 16 that
+// is run once is bound by instruction fetch, so it is rolled (8 tokens of the 8B
+// shape: 321 -> 313 us for 8 layers); the four blocks of 64 tokens reuse the
+// unrolled code (604 against 612 us).
+template <int UN>
 PP_DEVINL void gu_epilogue(const UnionArgs& a, UnionShared& sh, uint32_t tmem, int base, int nun, int upe, bool halves) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3;
     const int T = a.T, N = a.N, p0 = base / upe;
@@ -322,7 +330,7 @@ PP_DEVINL void gu_epilogue(const UnionArgs& a, UnionShared& sh, uint32_t tmem, i
             if (gated) {
                 // gate lanes finish the even tokens, up lanes the odd ones
                 const bool up = (lane & 8) != 0;
-#pragma unroll
+#pragma unroll UN
                 for (int k = 0; k < 8; k++) {
                     const int t = c + 2 * k + (up ? 1 : 0);
                     const float w = live && t < T ? gt[t] : 0.0f;
@@ -335,7 +343,7 @@ PP_DEVINL void gu_epilogue(const UnionArgs& a, UnionShared& sh, uint32_t tmem, i
                     if (live && t < T) store_h(Hn + (size_t)t * ldh, h, a.terms, T * ldh);
                 }
             } else {
-#pragma unroll
+#pragma unroll UN
                 for (int k = 0; k < 16; k++) {
                     const int t = c + k;
                     const float w = live && t < T ? gt[t] : 0.0f;
@@ -460,7 +468,10 @@ PP_DEVINL void gu_phase(const UnionArgs& a, UnionShared& sh, unsigned char* smem
         // the ring is free: the first W_down tiles may go out
         if (warp == kWdWarp && base + kPassUnits >= u1) wd_prologue(a, sh, smem, nU);
         tc_fence_after();
-        gu_epilogue(a, sh, tmem, base, nun, upe, !two && nks > 1);
+        if (N == 16)
+            gu_epilogue<1>(a, sh, tmem, base, nun, upe, !two && nks > 1);
+        else
+            gu_epilogue<16>(a, sh, tmem, base, nun, upe, !two && nks > 1);
         if (base + kPassUnits < u1) {  // the accumulators and gw are free for the next pass
             __syncthreads();
             tc_fence_after();
