@@ -110,39 +110,45 @@ cudaError_t stats_launch(const int32_t* counts, int T, int E, uint64_t* acc, cud
 // Forward values of the router terms of the training objective (Sec. 3.2,
 // Eq. entropy_loss and Eq. load_balance_loss; L_gate of Sec. 4.2.3) over a
 // batch of logits [T][E].  Pass 1: CTA b takes tokens [64 b, 64 b + 64),
-// warp w two of them (eight warps with eight each took 24 us for 2048 tokens,
-// a chain of eight tokens), lane l the experts l + 32 s.  Per token the softmax
-// is max-shifted in fp32.  part[b] = (column sums of p [E], sum of
-// p log(p + eps), sum of sigmoid(g)) over the CTA's tokens, fp32, reduced over
-// the warps in a fixed order.  Pass 2 (one CTA of 1024 threads) adds the
-// parts pairwise in a fixed tree order and combines the totals in fp64: the
-// result is deterministic.  (This GPU's fp64 pipe is narrow, so fp64 is kept
-// to the final scalars.)
-constexpr int kStatTok = 64, kStatWarps = 32;
+// warp w two of them, lane l the experts l + 32 s.  Per token the softmax is
+// max-shifted in fp32.  part[b] = (column sums of p [E], sum of p log(p + eps),
+// sum of sigmoid(g)) over the CTA's tokens, fp32.  Pass 2 (one CTA of 1024
+// threads) adds the parts pairwise in a fixed tree order and combines the
+// totals in fp64: the result is deterministic.  (This GPU's fp64 pipe is
+// narrow, so fp64 is kept to the final scalars.)
+//
+// The order of the sums is part of the result, down to the last bit: eight
+// consecutive tokens are added one after the other (per lane for the entropy
+// and gate terms, whose lanes are added last), then the eight groups of eight.
+// What a token costs is its loads, exponentials and logarithms, and these run
+// for all 64 tokens at once; only the additions go in turn, the four warps of a
+// group handing their running sums on through shared memory (eight warps with
+// eight tokens each, one after the other, took 24 us for 2048 tokens).
+constexpr int kStatTok = 64, kStatWarps = 32, kStatGroups = 8;
 constexpr int kStatFinal = 1024;
 
 __global__ void __launch_bounds__(kStatWarps * 32)
     router_stats_part_kernel(const float* __restrict__ logits, int T, int E, float eps, float* __restrict__ part,
                              unsigned* status) {
-    __shared__ float colw[kStatWarps][kMaxExperts];
-    __shared__ float entw[kStatWarps], gatew[kStatWarps];
+    __shared__ float colw[kStatGroups][kMaxExperts];
+    __shared__ float entl[kStatGroups][32], gatel[kStatGroups][32];
     pdl_wait();
     pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = (E + 31) / 32;
-    constexpr int kPer = kStatTok / kStatWarps;
+    constexpr int kPer = kStatTok / kStatWarps, kTurns = kStatWarps / kStatGroups;
     const int t0 = blockIdx.x * kStatTok + warp * kPer;
-    float g[kPer][8];  // the warp's tokens, all loads in flight
+    float g[kPer][8];  // the warp's tokens, all loads in flight; then their probabilities
 #pragma unroll
     for (int i = 0; i < kPer; i++)
 #pragma unroll
         for (int s = 0; s < 8; s++)
             g[i][s] = t0 + i < T && lane + 32 * s < E ? logits[(size_t)(t0 + i) * E + lane + 32 * s] : -INFINITY;
-    float col[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    float ent = 0.0f, gsum = 0.0f;
+    float ent[kPer], gsum[kPer];
 #pragma unroll
     for (int i = 0; i < kPer; i++) {
-        if (t0 + i >= T) break;
+        ent[i] = gsum[i] = 0.0f;
+        if (t0 + i >= T) continue;  // (the whole warp)
         bool fin = true;
         float m = -INFINITY;
 #pragma unroll
@@ -164,40 +170,57 @@ __global__ void __launch_bounds__(kStatWarps * 32)
         for (int s = 0; s < 8; s++) {
             if (s < S && lane + 32 * s < E) {
                 const float pj = e[s] / z;
-                col[s] += pj;
                 te += pj * logf(pj + eps);
                 tg += sigmoidf_(g[i][s]);
+                g[i][s] = pj;
             }
         }
         if (!fin) {
             te = __int_as_float(0x7fc00000);  // NaN: the statistics of a batch with a non-finite logit
             if (lane == 0) record_status(status, PP_ERR_NONFINITE);
         }
-        ent += te;
-        gsum += tg;
+        ent[i] = te;
+        gsum[i] = tg;
     }
+    // warp w is the (w % 4)-th of group w / 4: the groups' warps add in turn
+    const int grp = warp / kTurns;
+    for (int turn = 0; turn < kTurns; turn++) {
+        if (warp % kTurns == turn) {
+            float a = turn ? entl[grp][lane] : 0.0f, b = turn ? gatel[grp][lane] : 0.0f;
 #pragma unroll
-    for (int s = 0; s < 8; s++)
-        if (s < S && lane + 32 * s < E) colw[warp][lane + 32 * s] = col[s];
-    ent = warp_sum(ent);
-    gsum = warp_sum(gsum);
-    if (lane == 0) {
-        entw[warp] = ent;
-        gatew[warp] = gsum;
+            for (int i = 0; i < kPer; i++)
+                if (t0 + i < T) {
+                    a += ent[i];
+                    b += gsum[i];
+                }
+            entl[grp][lane] = a;
+            gatel[grp][lane] = b;
+#pragma unroll
+            for (int s = 0; s < 8; s++) {
+                if (s >= S || lane + 32 * s >= E) continue;
+                float c = turn ? colw[grp][lane + 32 * s] : 0.0f;
+#pragma unroll
+                for (int i = 0; i < kPer; i++)
+                    if (t0 + i < T) c += g[i][s];
+                colw[grp][lane + 32 * s] = c;
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    // four threads per expert sum eight warps each, then pairwise
     float* out = part + (size_t)blockIdx.x * (E + 2);
-    const int j = threadIdx.x >> 2, q = threadIdx.x & 3;
-    float c = 0.0f;
-    if (j < E)
+    if (threadIdx.x < E) {
+        float c = 0.0f;
 #pragma unroll
-        for (int w = 0; w < 8; w++) c += colw[q * 8 + w][j];
-    c += __shfl_xor_sync(kFull, c, 1);
-    c += __shfl_xor_sync(kFull, c, 2);
-    if (j < E && q == 0) out[j] = c;
-    if (warp == 0) {
-        const float a = warp_sum(entw[lane]), b = warp_sum(gatew[lane]);
+        for (int w = 0; w < kStatGroups; w++) c += colw[w][threadIdx.x];
+        out[threadIdx.x] = c;
+    }
+    if (warp == kStatWarps - 1) {  // (its threads have no column)
+        float a = 0.0f, b = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kStatGroups; w++) {
+            a += warp_sum(entl[w][lane]);
+            b += warp_sum(gatel[w][lane]);
+        }
         if (lane == 0) {
             out[E] = a;
             out[E + 1] = b;
