@@ -141,7 +141,9 @@ PP_DEVINL void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dep
 // later async-proxy (TMA) accesses of the same memory.
 PP_DEVINL void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// (`bar` is an aligned instruction: the lanes of a warp arrive together)
 PP_DEVINL void named_bar_sync(int id, int nthreads) {
+    __syncwarp();
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 

@@ -448,8 +448,9 @@ PP_DEVINL float desc_key_logit(uint32_t D) {
 
 // Barriers of a group of nt threads (whole warps) with barrier id `id`
 // (id 0 with the whole CTA is __syncthreads).
-PP_DEVINL void group_bar(int id, int nt) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nt) : "memory"); }
+PP_DEVINL void group_bar(int id, int nt) { named_bar_sync(id, nt); }
 PP_DEVINL bool group_bar_or(int id, int nt, bool v) {
+    __syncwarp();
     unsigned r;
     asm volatile(
         "{\n\t.reg .pred pi, po;\n\t"
@@ -462,6 +463,7 @@ PP_DEVINL bool group_bar_or(int id, int nt, bool v) {
     return r != 0u;
 }
 PP_DEVINL int group_bar_count(int id, int nt, bool v) {
+    __syncwarp();
     unsigned r;
     asm volatile(
         "{\n\t.reg .pred pi;\n\t"

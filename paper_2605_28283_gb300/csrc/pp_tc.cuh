@@ -16,15 +16,21 @@
 namespace pp {
 
 // ------------------------------------------------------------------- TMEM
+// The `.aligned` instructions below are for the whole warp at once: undefined
+// when its lanes have come apart (a per-lane `continue`, call or wait before
+// them), so each helper brings the lanes together first.
 PP_DEVINL void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {  // whole warp
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
                  "r"(ncols)
                  : "memory");
 }
 PP_DEVINL void tmem_relinquish() {  // whole warp
+    __syncwarp();
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 PP_DEVINL void tmem_dealloc(uint32_t taddr, uint32_t ncols) {  // whole warp
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 PP_DEVINL void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -82,6 +88,7 @@ PP_DEVINL void umma_k64(uint32_t d_tmem, const void* a_tile, const void* b_tile,
 // Warp-collective: lane i receives row (lane base + i), 32 consecutive
 // fp32 columns starting at the address's column.
 PP_DEVINL void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
         "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
@@ -93,6 +100,7 @@ PP_DEVINL void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 // Same with 16 columns.
 PP_DEVINL void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
         "%14, %15}, [%16];"
@@ -100,7 +108,10 @@ PP_DEVINL void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
 }
-PP_DEVINL void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+PP_DEVINL void tmem_ld_wait() {
+    __syncwarp();
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
 
 // --------------------------------------------------------------- TMA extra
 // Four rows (row0..row3) of a 2-D tensor, one box of {64 x 1} each, landing
