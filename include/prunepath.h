@@ -126,7 +126,7 @@ typedef struct pp_selection {
 /* Bytes of workspace needed for calls with up to T tokens. */
 size_t pp_workspace_size(const pp_desc *desc, int T);
 
-/* Zero the whole workspace (status word, launch counts, accumulators) on
+/* Zero the whole workspace (status word, launch counts, barrier counter) on
    `stream`.  Call once after allocating a workspace, and again to clear a
    sticky device error. */
 pp_status pp_workspace_init(void *ws, size_t ws_bytes, void *stream);

@@ -81,7 +81,7 @@ bool use_union_small(const pp_desc& d, int T, float p) {
 struct Layout {
     size_t logits, ids, counts, gates, tlog, th, stats;
     // grouped path
-    size_t part, bits, gexp, slot_of, cnt, ltok, lgate, offsets, H, Y, yacc, overflow, dpart;
+    size_t part, bits, gexp, slot_of, cnt, ltok, lgate, offsets, H, Y, yacc, dpart;
     // fp32 calls of more tokens than a fused decode launch takes (bits and gexp too)
     size_t h32;
     size_t total;
@@ -117,7 +117,6 @@ Layout layout(const pp_desc& d, int T) {
         L.H = take(std::max((size_t)g.nnz_max + 128, 15 * E) * kDExpert * 2);  // three terms of up to 5 tokens
         L.Y = take((size_t)g.ycap * d.d_model * 2);
         L.yacc = take(Tn * (size_t)d.d_model * 4);
-        L.overflow = take(16);
         L.dpart = take(union_part_floats((int)Tn, d.d_model) * 4);
     }
     if (d.dtype == PP_F32) {
@@ -285,7 +284,6 @@ GroupedArgs grouped_args(const pp_desc& d, int T, void* ws, const void* x, const
     a.H = reinterpret_cast<__nv_bfloat16*>(b + L.H);
     a.Y = reinterpret_cast<__nv_bfloat16*>(b + L.Y);
     a.yacc = reinterpret_cast<float*>(b + L.yacc);
-    a.overflow = reinterpret_cast<int*>(b + L.overflow);
     a.dpart = reinterpret_cast<float*>(b + L.dpart);
     a.bar = &reinterpret_cast<Control*>(b)->bar;
     a.status = &reinterpret_cast<Control*>(b)->status;

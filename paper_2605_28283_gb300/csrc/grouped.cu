@@ -16,8 +16,10 @@
 //   combine       y[t] = sum over t's experts, in ascending expert order, of
 //                 its pairs' rows (fp32 accumulation, deterministic)
 //   Pairs past the row buffer's capacity (only near-dense selections) are
-//   added into an fp32 accumulator instead; the combine step reads and
-//   re-zeroes it.
+//   added into an fp32 accumulator instead, which the gate/up kernel clears
+//   when the call's pairs exceed the capacity and the combine step adds.
+//   (Nothing is expected of it before the call: its place depends on the
+//   call's token count, so calls of other lengths write over it.)
 //
 // A slot is given out by an atomic, so the order of an expert's tokens varies
 // between calls; no result depends on it (a row of a GEMM tile does not depend
@@ -45,14 +47,12 @@ constexpr int kTileBytesA = 128 * 128;  // 128 rows x 64 bf16
 template <int NE>
 __global__ void __launch_bounds__(kTcThreads, 1)
     router_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_wr,
-                       int T, int E, int nk, int kpb, float* part, int* cnt, int* overflow, unsigned* status,
+                       int T, int E, int nk, int kpb, float* part, int* cnt, unsigned* status,
                        uint64_t lim) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
-    if (cnt && blockIdx.x == 0 && blockIdx.y == 0) {  // the selection fills the lists
+    if (cnt && blockIdx.x == 0 && blockIdx.y == 0)  // the selection fills the lists
         for (int e = threadIdx.x; e < E; e += blockDim.x) cnt[e] = 0;
-        if (threadIdx.x == 0) *overflow = 0;
-    }
     constexpr int kStages = 4;
     constexpr int kTileB = NE * 128;
     constexpr int kStage = kTileBytesA + kTileB;
@@ -321,14 +321,12 @@ __global__ void __launch_bounds__(256) select_part_cta_kernel(const float* __res
 __global__ void __launch_bounds__(256) dispatch_bits_kernel(const int32_t* __restrict__ ids,
                                                             const int32_t* __restrict__ counts,
                                                             const float* __restrict__ gates, int T, int E,
-                                                            uint32_t* bits, float* gexp, int* cnt, int* overflow,
+                                                            uint32_t* bits, float* gexp, int* cnt,
                                                             unsigned* status) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
-    if (cnt && blockIdx.x == 0) {  // lengths of the lists that dispatch_list_kernel fills
+    if (cnt && blockIdx.x == 0)  // lengths of the lists that dispatch_list_kernel fills
         for (int e = threadIdx.x; e < E; e += blockDim.x) cnt[e] = 0;
-        if (threadIdx.x == 0) *overflow = 0;
-    }
     // one warp per token: coalesced row writes
     const int lane = threadIdx.x & 31;
     const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -429,6 +427,7 @@ struct ItemTable {
         }
     }
     PP_DEVINL int n_items() const { return ib[kMaxExperts]; }
+    PP_DEVINL int n_pairs() const { return off[kMaxExperts]; }
     PP_DEVINL Item item(int wi) const {
         int lo = 0, hi = kMaxExperts;  // ib[lo] <= wi < ib[hi]
 #pragma unroll 1
@@ -470,8 +469,8 @@ constexpr int kGuBox = 32;  // weight rows of a TMA box
 __global__ void __launch_bounds__(kGuThreads, 1)
     gu_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_wg,
                    const __grid_constant__ CUtensorMap map_wu, const int* __restrict__ cnt, const int* __restrict__ ltok,
-                   const float* __restrict__ lgate, int* offsets, int T, int E, int nk, int act, __nv_bfloat16* H,
-                   unsigned* status, uint64_t lim) {
+                   const float* __restrict__ lgate, int* offsets, int T, int E, int d, int nk, int act, __nv_bfloat16* H,
+                   long long ycap, float* yacc, unsigned* status, uint64_t lim) {
     const bool gated = act == PP_ACT_SWIGLU;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -581,6 +580,13 @@ __global__ void __launch_bounds__(kGuThreads, 1)
     } else {
         const int q = warp & 3;
         const int row = 32 * q + lane;
+        // some pairs go past the row buffer: their accumulator starts at zero
+        // (before the first sums are there; d is a multiple of 8)
+        if (tab.n_pairs() > ycap) {
+            float4* z = reinterpret_cast<float4*>(yacc);
+            const size_t n = (size_t)T * d / 4, step = (size_t)G * kGuEpi * 32;
+            for (size_t i = (size_t)blockIdx.x * kGuEpi * 32 + row; i < n; i += step) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
         int acc = 0, it = 0;
         for (int v = blockIdx.x; v < n_tasks; v += G, acc++, it += nk) {
             const Item w = tab.item(v / split);
@@ -696,7 +702,7 @@ struct DownPos {
 __global__ void __launch_bounds__(kDnThreads, 1)
     down_gemm_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
                      const int* __restrict__ cnt, const int* __restrict__ ltok, int T, int E, int d, int nrt,
-                     __nv_bfloat16* Y, long long ycap, float* yacc, int* overflow, unsigned* status, uint64_t lim) {
+                     __nv_bfloat16* Y, long long ycap, float* yacc, unsigned* status, uint64_t lim) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t full[kDnStages], empty[kDnStages], tfull[kDnAcc], tempty[kDnAcc];
@@ -835,7 +841,6 @@ __global__ void __launch_bounds__(kDnThreads, 1)
                         else
                             atomicAdd(&yacc[(size_t)ltok[(size_t)w.e * T + 128 * w.sub + t] * d + row], val);
                     }
-                    if (lane == 0) *overflow = 1;
                 }
             }
             if (++a == kDnAcc) {
@@ -860,7 +865,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     down_rows_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
                      const __grid_constant__ CUtensorMap map_y, const int* __restrict__ cnt,
                      const int* __restrict__ ltok, int T, int E, int d, int njt, __nv_bfloat16* Y, long long ycap,
-                     float* yacc, int* overflow, unsigned* status, uint64_t lim) {
+                     float* yacc, unsigned* status, uint64_t lim) {
     constexpr int kStages = 4;
     constexpr int kTileB = 256 * 128;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -951,7 +956,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const bool in_buf = live && arow < ycap;
             const int tok = live && !in_buf ? ltok[(size_t)w.e * T + w.m0 + row] : -1;
             float* yrow = tok >= 0 ? yacc + (size_t)tok * d : nullptr;
-            if (tok >= 0) *overflow = 1;
             __nv_bfloat16* Yrow = in_buf ? Y + (size_t)arow * d : nullptr;
             for (int jt = 0; jt < njt; jt++, acc++) {
                 const int a = acc & 1;
@@ -1030,15 +1034,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
 // =================================================================== combine
 // y[t] = the sum of token t's assignment rows Y[pos] in ascending expert
-// order, plus yacc[t] when the down projection overflowed (yacc is then
-// cleared again).  Grid (T, ceil(d / 1024)): 128 threads of 8 columns each.
+// order, plus yacc[t] when the call's pairs exceed the row buffer.  Grid (T, ceil(d / 1024)): 128 threads of 8 columns each.
 // The expert list is built in parallel: 128 experts per round, compacted in
 // ascending order with ballots.
 __global__ void __launch_bounds__(128) combine_kernel(const uint32_t* __restrict__ bits, const int* __restrict__ slot_of,
                                                       const int* __restrict__ offsets,
                                                       const __nv_bfloat16* __restrict__ Y, long long ycap,
-                                                      float* yacc, const int* __restrict__ overflow, int T, int E,
-                                                      int d, __nv_bfloat16* y) {
+                                                      const float* __restrict__ yacc, int T, int E, int d,
+                                                      __nv_bfloat16* y) {
     pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
     pdl_launch_dependents();
     const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1062,13 +1065,11 @@ __global__ void __launch_bounds__(128) combine_kernel(const uint32_t* __restrict
     const int c = blockIdx.y * 1024 + tid * 8;
     if (c >= d) return;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (*overflow != 0) {
-        float4* ya = reinterpret_cast<float4*>(yacc + (size_t)t * d + c);
+    if (offsets[E] > ycap) {
+        const float4* ya = reinterpret_cast<const float4*>(yacc + (size_t)t * d + c);
         const float4 a0 = ya[0], a1 = ya[1];
         acc[0] = a0.x; acc[1] = a0.y; acc[2] = a0.z; acc[3] = a0.w;
         acc[4] = a1.x; acc[5] = a1.y; acc[6] = a1.z; acc[7] = a1.w;
-        ya[0] = make_float4(0.f, 0.f, 0.f, 0.f);  // keep the accumulator zero at rest
-        ya[1] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     // rows added in ascending expert order; their loads go out 4 at a time
     for (int i0 = 0; i0 < n; i0 += 4) {
@@ -1094,12 +1095,12 @@ namespace {
 
 template <int NE>
 cudaError_t launch_router(const CUtensorMap& mx, const CUtensorMap& mwr, int T, int E, int nk, int kpb, int nsplit,
-                          float* part, int* cnt, int* overflow, unsigned* status, uint64_t lim, cudaStream_t st) {
+                          float* part, int* cnt, unsigned* status, uint64_t lim, cudaStream_t st) {
     const size_t smem = 4 * (size_t)(kTileBytesA + NE * 128) + 1024;
     cudaError_t e = set_smem(router_gemm_kernel<NE>, smem);
     if (e != cudaSuccess) return e;
     PP_LAUNCH(router_gemm_kernel<NE>, dim3((T + 127) / 128, nsplit), dim3(kTcThreads), smem, st, mx, mwr, T, E, nk,
-        kpb, part, cnt, overflow, status, lim);
+        kpb, part, cnt, status, lim);
     return cudaGetLastError();
 }
 
@@ -1126,13 +1127,13 @@ cudaError_t grouped_route(const GroupedArgs& a, cudaStream_t st) {
     if (!encode_2d(&mx, a.x, a.d, a.T, 64, 128) || !encode_2d(&mwr, a.Wr, a.d, a.E, 64, NE)) return cudaErrorInvalidValue;
     cudaError_t e;
     switch (NE) {
-        case 32: e = launch_router<32>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
-        case 64: e = launch_router<64>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
-        case 128: e = launch_router<128>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
-        case 160: e = launch_router<160>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
-        case 192: e = launch_router<192>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
-        case 224: e = launch_router<224>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
-        default: e = launch_router<256>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.overflow, a.status, a.timeout_ns, st); break;
+        case 32: e = launch_router<32>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.status, a.timeout_ns, st); break;
+        case 64: e = launch_router<64>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.status, a.timeout_ns, st); break;
+        case 128: e = launch_router<128>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.status, a.timeout_ns, st); break;
+        case 160: e = launch_router<160>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.status, a.timeout_ns, st); break;
+        case 192: e = launch_router<192>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.status, a.timeout_ns, st); break;
+        case 224: e = launch_router<224>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.status, a.timeout_ns, st); break;
+        default: e = launch_router<256>(mx, mwr, a.T, a.E, g.nk, g.kpb, g.nsplit, a.part, cnt, a.status, a.timeout_ns, st); break;
     }
     if (e != cudaSuccess) return e;
     if (a.T <= kCtaSelectMaxTokens) {  // pp_route: the union kernel makes its own selection
@@ -1158,7 +1159,7 @@ cudaError_t grouped_route(const GroupedArgs& a, cudaStream_t st) {
 cudaError_t grouped_load_selection(const GroupedArgs& a, cudaStream_t st) {
     const bool lists = a.cnt != nullptr && a.T > kUnionMaxT;
     PP_LAUNCH(dispatch_bits_kernel, dim3((a.T + 7) / 8), dim3(256), 0, st, a.ids, a.counts, a.gates, a.T, a.E, a.bits,
-              a.gexp, lists ? a.cnt : nullptr, a.overflow, a.status);
+              a.gexp, lists ? a.cnt : nullptr, a.status);
     if (lists)
         PP_LAUNCH(dispatch_list_kernel, dim3((a.T + 7) / 8), dim3(256), 0, st, a.bits, a.gexp, a.T, a.E,
                   Lists{a.cnt, a.ltok, a.lgate, a.slot_of});
@@ -1181,10 +1182,10 @@ cudaError_t grouped_ffn(const GroupedArgs& a, int sms, cudaStream_t st) {
     if ((e = set_smem(gu_gemm_kernel, gu_smem)) != cudaSuccess || (e = set_smem(down_gemm_kernel, dn_smem)) != cudaSuccess)
         return e;
     PP_LAUNCH(gu_gemm_kernel, dim3(sms), dim3(kGuThreads), gu_smem, st, mx, mwg, mwu, a.cnt, a.ltok, a.lgate, a.offsets, a.T,
-              a.E, g.nk, a.act, a.H, a.status, a.timeout_ns);
+              a.E, a.d, g.nk, a.act, a.H, g.ycap, a.yacc, a.status, a.timeout_ns);
     if (a.T <= kDownRowsMinT) {
         PP_LAUNCH(down_gemm_kernel, dim3(sms), dim3(kDnThreads), dn_smem, st, mh, mwd, a.cnt, a.ltok, a.T, a.E, a.d,
-                  (a.d + 127) / 128, a.Y, g.ycap, a.yacc, a.overflow, a.status, a.timeout_ns);
+                  (a.d + 127) / 128, a.Y, g.ycap, a.yacc, a.status, a.timeout_ns);
     } else {
         // A tile, the 4-stage W_down ring, 4 x 16 KB store staging
         const size_t smem = (size_t)kTileBytesA + 4 * (size_t)256 * 128 + 4 * (size_t)16384 + 1024;
@@ -1195,10 +1196,10 @@ cudaError_t grouped_ffn(const GroupedArgs& a, int sms, cudaStream_t st) {
             return cudaErrorInvalidValue;
         if ((e = set_smem(down_rows_kernel, smem)) != cudaSuccess) return e;
         PP_LAUNCH(down_rows_kernel, dim3(sms), dim3(kTcThreads), smem, st, mh128, mwd256, my, a.cnt, a.ltok, a.T, a.E, a.d,
-                  (a.d + 255) / 256, a.Y, g.ycap, a.yacc, a.overflow, a.status, a.timeout_ns);
+                  (a.d + 255) / 256, a.Y, g.ycap, a.yacc, a.status, a.timeout_ns);
     }
     PP_LAUNCH(combine_kernel, dim3(a.T, (a.d + 1023) / 1024), dim3(128), 0, st, a.bits, a.slot_of, a.offsets, a.Y, g.ycap,
-              a.yacc, a.overflow, a.T, a.E, a.d, reinterpret_cast<__nv_bfloat16*>(a.y));
+              a.yacc, a.T, a.E, a.d, reinterpret_cast<__nv_bfloat16*>(a.y));
     return cudaGetLastError();
 }
 

@@ -179,9 +179,8 @@ struct GroupedArgs {
     int* offsets;       // [E + 1] first row of each expert in H and Y
     __nv_bfloat16* H;   // [nnz_max + 128][64]
     __nv_bfloat16* Y;   // [ycap][d] assignment outputs
-    float* yacc;        // [T][d] overflow accumulator, zero at rest
+    float* yacc;        // [T][d] sums of the pairs past ycap
     float* dpart;       // partial down-projection tiles (union path)
-    int* overflow;      // set when any assignment went to yacc
     unsigned long long* bar;  // grid barrier counter (union path)
     unsigned* status;
     uint64_t timeout_ns;
