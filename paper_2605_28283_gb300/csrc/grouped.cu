@@ -15,15 +15,19 @@
 //                 (K = 64); each pair's output row is stored bf16
 //   combine       y[t] = sum over t's experts, in ascending expert order, of
 //                 its pairs' rows (fp32 accumulation, deterministic)
-//   Pairs past the row buffer's capacity (only near-dense selections) are
-//   added into an fp32 accumulator instead, which the gate/up kernel clears
-//   when the call's pairs exceed the capacity and the combine step adds.
+//   An expert whose rows do not all fit the row buffer (only near-dense
+//   selections have one) adds them into an fp32 accumulator instead, which the
+//   gate/up kernel clears when the call's pairs exceed the capacity and the
+//   combine step adds.
 //   (Nothing is expected of it before the call: its place depends on the
 //   call's token count, so calls of other lengths write over it.)
 //
 // A slot is given out by an atomic, so the order of an expert's tokens varies
-// between calls; no result depends on it (a row of a GEMM tile does not depend
-// on its place, and the combine step goes by expert).
+// between calls; no pair's value depends on it (a row of a GEMM tile does not
+// depend on its place, the combine step goes by expert, and all of an expert's
+// pairs are rounded alike: to bf16 in the row buffer, or not at all in the
+// accumulator).  What is free is the order of the fp32 additions into that
+// accumulator, so a token with several such experts may differ in the last bit.
 // All waits are bounded (PP_ERR_TIMEOUT).
 #include "pp_common.cuh"
 #include "pp_kernels.h"
@@ -428,6 +432,8 @@ struct ItemTable {
     }
     PP_DEVINL int n_items() const { return ib[kMaxExperts]; }
     PP_DEVINL int n_pairs() const { return off[kMaxExperts]; }
+    // whether expert e's rows end past the row buffer
+    PP_DEVINL bool spills(int e, long long ycap) const { return off[e + 1] > ycap; }
     PP_DEVINL Item item(int wi) const {
         int lo = 0, hi = kMaxExperts;  // ib[lo] <= wi < ib[hi]
 #pragma unroll 1
@@ -791,7 +797,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
         uint32_t aph = 0;
         for (int i = 0; i < n; i++) {
             const int m = w.count(), a0 = w.a0();
-            const bool spill = (long long)a0 + m > ycap;  // some of the item's rows go to yacc
+            const bool spill = tab.spills(w.e, ycap);  // the expert's rows go to yacc
             mbar_wait(&tfull[a], aph, status, lim);
             tc_fence_after();
             const int row = w.rt * 128 + 32 * q + lane;  // output element
@@ -835,11 +841,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
                     for (int k = 0; k < 32; k++) {
                         const int t = c + k;
                         if (t >= m) break;
-                        const float val = __uint_as_float(v[k]);
-                        if ((long long)a0 + t < ycap)
-                            Y[(size_t)(a0 + t) * d + row] = __float2bfloat16_rn(val);
-                        else
-                            atomicAdd(&yacc[(size_t)ltok[(size_t)w.e * T + 128 * w.sub + t] * d + row], val);
+                        atomicAdd(&yacc[(size_t)ltok[(size_t)w.e * T + 128 * w.sub + t] * d + row], __uint_as_float(v[k]));
                     }
                 }
             }
@@ -950,10 +952,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const Item w = tab.item(v);
             const bool live = row < w.cnt;
             const bool group_live = 32 * q < w.cnt;  // any live row in this warp's 32 rows
-            // all 32 rows live and inside Y: the group's rows go out as 2-D bulk stores
-            const bool group_full = 32 * q + 32 <= w.cnt && (long long)w.a0 + 32 * q + 32 <= ycap;
+            const bool spill = tab.spills(w.e, ycap);  // the expert's rows go to yacc
+            // all 32 rows live: the group's rows go out as 2-D bulk stores
+            const bool group_full = 32 * q + 32 <= w.cnt && !spill;
             const long long arow = (long long)w.a0 + row;
-            const bool in_buf = live && arow < ycap;
+            const bool in_buf = live && !spill;
             const int tok = live && !in_buf ? ltok[(size_t)w.e * T + w.m0 + row] : -1;
             float* yrow = tok >= 0 ? yacc + (size_t)tok * d : nullptr;
             __nv_bfloat16* Yrow = in_buf ? Y + (size_t)arow * d : nullptr;
@@ -1052,7 +1055,7 @@ __global__ void __launch_bounds__(128) combine_kernel(const uint32_t* __restrict
         const int e = e0 + tid;
         bool on = e < E && ((bits[(size_t)t * 8 + (e >> 5)] >> (e & 31)) & 1u);
         const int pos = on ? offsets[e] + slot_of[(size_t)t * E + e] : 0;
-        on = on && pos < ycap;
+        on = on && offsets[e + 1] <= ycap;
         const unsigned bal = __ballot_sync(kFull, on);
         if (lane == 0) wn_s[warp] = __popc(bal);
         __syncthreads();

@@ -33,3 +33,29 @@ def test_spilling_prompts_of_several_lengths_share_a_workspace(pp, lengths):
             assert pp.pp_get_device_status(ws) == pp.PP_OK
     for T, y, ref in zip(lengths, ys, alone):
         assert rel_err_per_token(to_host(y), to_host(ref)).max() <= Y_TOL["bf16"] / 2, T
+
+
+@pytest.mark.parametrize("T", [300, 1100])
+def test_spilling_does_not_depend_on_the_order_of_the_lists(pp, T):
+    """One expert's rows straddle the end of the row buffer (64 rows a token).
+    Its tokens stand in its list in any order, but all of its pairs are summed
+    in fp32, and as each token has one such pair at most nothing else is free:
+    repeated calls give the same bits."""
+    import torch
+    E, skip = 66, 100
+    w, (x, Wr, Wg, Wu, Wd) = _layer("llama3_8b_batched", T, 264, E)
+    ids = np.tile(np.arange(E, dtype=np.int32), (T, 1))
+    ids[:skip, 0] = 64  # `skip` tokens leave out expert 0: 64 T - skip pairs come before expert 64's T
+    ids[:skip, 64] = -1
+    ids[:, 65] = -1
+    counts = np.where(np.arange(T) < skip, 64, 65).astype(np.int32)
+    gates = np.where(ids >= 0, np.float32(0.7), np.float32(0))
+    desc = pp.make_desc(w.d_model, E, w.dtype, w.act)
+    ws = pp.alloc_workspace(desc, T)
+    sel = pp.Selection(dev(ids), dev(counts), dev(gates))
+    ys = [torch.empty_like(x) for _ in range(20)]
+    for y in ys:
+        pp.pp_sparse_ffn(desc, x, T, Wg, Wu, Wd, sel, y, ws)
+    torch.cuda.synchronize()
+    assert pp.pp_get_device_status(ws) == pp.PP_OK
+    assert all(torch.equal(y, ys[0]) for y in ys)
