@@ -77,7 +77,8 @@ bool use_union_small(const pp_desc& d, int T, float p) {
     return T >= 3;  // LTE
 }
 
-// Workspace layout for calls with up to T tokens.
+// Workspace layout of calls with T tokens.  Its size never falls as T grows: a
+// workspace for up to T tokens serves every shorter call.
 struct Layout {
     size_t logits, ids, counts, gates, tlog, th, stats;
     // grouped path
@@ -106,7 +107,7 @@ Layout layout(const pp_desc& d, int T) {
     L.stats = take((size_t)router_stats_blocks((int)Tn) * (E + 2) * 8);
     if (use_grouped(d, T) || union_small_shape(d, T)) {
         const GroupedPlan g = grouped_plan(T, d.d_model, d.n_experts, 152);
-        L.part = take((size_t)g.nsplit * Tn * E * 4);
+        L.part = take(router_part_rows(T, d.d_model, 152) * E * 4);
         L.bits = take(Tn * 8 * 4);
         L.gexp = take(Tn * E * 4);
         L.slot_of = take(Tn * E * 4);

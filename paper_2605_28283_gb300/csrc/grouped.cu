@@ -1122,6 +1122,15 @@ GroupedPlan grouped_plan(int T, int d, int E, int sms) {
     return g;
 }
 
+// nsplit(t) is at most the K chunks' limit and at most sms / ceil(t / 128), or 1:
+// it falls as t crosses a multiple of 128, so nsplit(t) * t does too, and the
+// bound is the largest of either limit's products.
+size_t router_part_rows(int T, int d, int sms) {
+    const size_t t = (size_t)std::max(T, 1);
+    const size_t most = (size_t)std::max(1, std::min((d + 63) / 64 / 4, 64));
+    return std::max(t, std::min(t * most, (size_t)sms * 128));
+}
+
 cudaError_t grouped_route(const GroupedArgs& a, cudaStream_t st) {
     const GroupedPlan& g = a.plan;
     CUtensorMap mx, mwr;

@@ -194,6 +194,9 @@ constexpr int kUnionMaxGrid = 152;
 size_t union_part_floats(int T, int d);  // of GroupedArgs.dpart
 
 GroupedPlan grouped_plan(int T, int d, int E, int sms);
+// Rows of GroupedArgs.part that calls with up to T tokens need: at least
+// nsplit(t) * t for every t <= T.
+size_t router_part_rows(int T, int d, int sms);
 cudaError_t grouped_route(const GroupedArgs& a, cudaStream_t st);
 // The FFN over a.bits / a.gexp (the selection as the FFN kernels read it,
 // written by grouped_route, or by grouped_load_selection from a.ids, a.counts
