@@ -110,15 +110,21 @@ Layout layout(const pp_desc& d, int T) {
         L.part = take(router_part_rows(T, d.d_model, 152) * E * 4);
         L.bits = take(Tn * 8 * 4);
         L.gexp = take(Tn * E * 4);
-        L.slot_of = take(Tn * E * 4);
-        L.cnt = take(E * 4);
-        L.ltok = take((size_t)g.nnz_max * 4);
-        L.lgate = take((size_t)g.nnz_max * 4);
-        L.offsets = take((E + 1) * 4);
         L.H = take(std::max((size_t)g.nnz_max + 128, 15 * E) * kDExpert * 2);  // three terms of up to 5 tokens
-        L.Y = take((size_t)g.ycap * d.d_model * 2);
-        L.yacc = take(Tn * (size_t)d.d_model * 4);
-        L.dpart = take(union_part_floats((int)Tn, d.d_model) * 4);
+        // the union kernel's partial tiles, or the prompt path's lists and rows
+        const size_t dpart = union_part_floats((int)Tn, d.d_model) * 4;
+        if (T <= kUnionMaxT) {
+            L.dpart = take(dpart);
+        } else {
+            L.slot_of = take(Tn * E * 4);
+            L.cnt = take(E * 4);
+            L.ltok = take((size_t)g.nnz_max * 4);
+            L.lgate = take((size_t)g.nnz_max * 4);
+            L.offsets = take((E + 1) * 4);
+            const size_t y = align256((size_t)g.ycap * d.d_model * 2);
+            L.Y = take(std::max(dpart, y + Tn * (size_t)d.d_model * 4));
+            L.yacc = L.Y + y;
+        }
     }
     if (d.dtype == PP_F32) {
         L.bits = take(Tn * 8 * 4);
