@@ -38,10 +38,6 @@
 namespace pp {
 
 constexpr int kTcThreads = 192;
-// Prompts above this many tokens run the down projection with tokens as the M
-// operand (333 tokens of the 7B shape: 34 us with weights as M against 45; 2048
-// of the 13B shape: 69 against 60; 8192: 199 against 124).
-constexpr int kDownRowsMinT = 1024;
 constexpr int kTileBytesA = 128 * 128;  // 128 rows x 64 bf16
 
 
@@ -673,6 +669,7 @@ constexpr int kDnBox = 32;               // H rows of a TMA box
 constexpr int kDnPitch = 128 * 2 + 16;   // staged token row
 constexpr int kDnStageOut = 32 * kDnPitch;
 constexpr size_t kDnRing = 172 * 1024;   // followed by 2 staging areas per set of epilogue warps
+constexpr int kDrStages = 4, kDrTileB = 256 * 128;  // tokens as the M operand: the W_down ring
 
 // Position in the pairs of a call: item `it` of tile rt is work item `sub` of
 // expert e.
@@ -705,38 +702,19 @@ struct DownPos {
     }
 };
 
-__global__ void __launch_bounds__(kDnThreads, 1)
-    down_gemm_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
-                     const int* __restrict__ cnt, const int* __restrict__ ltok, int T, int E, int d, int nrt,
-                     __nv_bfloat16* Y, long long ycap, float* yacc, unsigned* status, uint64_t lim) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t full[kDnStages], empty[kDnStages], tfull[kDnAcc], tempty[kDnAcc];
-    __shared__ uint32_t taddr_s;
-    __shared__ ItemTable tab;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kDnStages; i++) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
-        }
-        for (int i = 0; i < kDnAcc; i++) {
-            mbar_init(&tfull[i], 1);
-            mbar_init(&tempty[i], kDnEpi);
-        }
-        fence_mbar_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(&taddr_s, kDnAcc * 128);
-        tmem_relinquish();
-    }
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    tab.build(cnt, E);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = taddr_s;
+struct DownShared {
+    ItemTable tab;
+    uint32_t taddr;
+    uint64_t full[kDnStages], empty[kDnStages], tfull[kDnAcc], tempty[kDnAcc];    // down_tiles
+    uint64_t rfull[kDrStages], rempty[kDrStages], rtfull[2], rtempty[2], afull, aempty;  // down_rows
+};
+
+PP_DEVINL void down_tiles(const CUtensorMap& map_h, const CUtensorMap& map_wd, DownShared& sh, unsigned char* smem,
+                          uint32_t tmem, const int* __restrict__ ltok, int T, int d, __nv_bfloat16* Y, long long ycap,
+                          float* yacc, unsigned* status, uint64_t lim) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nrt = (d + 127) / 128;
+    const ItemTable& tab = sh.tab;
+    uint64_t *full = sh.full, *empty = sh.empty, *tfull = sh.tfull, *tempty = sh.tempty;
     const long long P = (long long)tab.n_items() * nrt;
     const long long p0 = P * blockIdx.x / gridDim.x;
     const int n = (int)(P * (blockIdx.x + 1) / gridDim.x - p0);
@@ -854,54 +832,22 @@ __global__ void __launch_bounds__(kDnThreads, 1)
         bulk_wait_all();  // the stores are done before the CTA's shared memory goes away
         __syncwarp();
     }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, kDnAcc * 128);
 }
 
-// Down projection of many tokens per expert (more than kDownRowsMinT tokens),
-// tokens as the M operand.  Persistent over work items: an item's H tile is loaded once and the njt
-// 256-wide slices of d stream through the B ring.  Two 256-column TMEM
-// accumulators overlap the reduction epilogue with the next slice's MMAs.
-__global__ void __launch_bounds__(kTcThreads, 1)
-    down_rows_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
-                     const __grid_constant__ CUtensorMap map_y, const int* __restrict__ cnt,
-                     const int* __restrict__ ltok, int T, int E, int d, int njt, __nv_bfloat16* Y, long long ycap,
-                     float* yacc, unsigned* status, uint64_t lim) {
-    constexpr int kStages = 4;
-    constexpr int kTileB = 256 * 128;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+// Tokens as the M operand.  Persistent over work items: an item's H tile is
+// loaded once and the 256-wide slices of d stream through the B ring.  Two
+// 256-column TMEM accumulators overlap the stores of one slice with the next
+// slice's MMAs.  Warp 0 loads, 1 issues the MMAs, 2-5 store.
+PP_DEVINL void down_rows(const CUtensorMap& map_h, const CUtensorMap& map_wd, const CUtensorMap& map_y, DownShared& sh,
+                         unsigned char* smem, uint32_t tmem, const int* __restrict__ ltok, int T, int d,
+                         __nv_bfloat16* Y, long long ycap, float* yacc, unsigned* status, uint64_t lim) {
+    constexpr int kStages = kDrStages;
+    constexpr int kTileB = kDrTileB;
     unsigned char* tileA = smem;
     unsigned char* ringB = smem + kTileBytesA;
-    __shared__ uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], afull, aempty;
-    __shared__ uint32_t taddr_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __shared__ ItemTable tab;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; i++) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
-        }
-        for (int i = 0; i < 2; i++) {
-            mbar_init(&tfull[i], 1);
-            mbar_init(&tempty[i], 4);
-        }
-        mbar_init(&afull, 1);
-        mbar_init(&aempty, 1);
-        fence_mbar_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(&taddr_s, 512);
-        tmem_relinquish();
-    }
-    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
-    pdl_launch_dependents();
-    tab.build(cnt, E);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = taddr_s;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, njt = (d + 255) / 256;
+    const ItemTable& tab = sh.tab;
+    uint64_t *full = sh.rfull, *empty = sh.rempty, *tfull = sh.rtfull, *tempty = sh.rtempty;
     const int n_items = tab.n_items();
 
     if (warp == 0) {
@@ -909,9 +855,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             int it = 0, ii = 0;
             for (int v = blockIdx.x; v < n_items; v += gridDim.x, ii++) {
                 const Item w = tab.item(v);
-                if (ii >= 1) mbar_wait(&aempty, (uint32_t)(ii - 1) & 1u, status, lim);
-                mbar_arrive_expect_tx(&afull, kTileBytesA);
-                tma_load_2d(tileA, &map_h, 0, w.a0, &afull);
+                if (ii >= 1) mbar_wait(&sh.aempty, (uint32_t)(ii - 1) & 1u, status, lim);
+                mbar_arrive_expect_tx(&sh.afull, kTileBytesA);
+                tma_load_2d(tileA, &map_h, 0, w.a0, &sh.afull);
                 for (int jt = 0; jt < njt; jt++, it++) {
                     const int s = it % kStages;
                     if (it >= kStages) mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, status, lim);
@@ -926,7 +872,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             constexpr uint32_t idesc = idesc_bf16_m128(256);
             int it = 0, acc = 0, ii = 0;
             for (int v = blockIdx.x; v < n_items; v += gridDim.x, ii++) {
-                mbar_wait(&afull, (uint32_t)ii & 1u, status, lim);
+                mbar_wait(&sh.afull, (uint32_t)ii & 1u, status, lim);
                 for (int jt = 0; jt < njt; jt++, it++, acc++) {
                     const int a = acc & 1;
                     if (acc >= 2) mbar_wait(&tempty[a], (uint32_t)((acc >> 1) - 1) & 1u, status, lim);
@@ -937,11 +883,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     umma_commit(&empty[s]);
                     umma_commit(&tfull[a]);
                 }
-                umma_commit(&aempty);
+                umma_commit(&sh.aempty);
             }
         }
         __syncwarp();
-    } else {
+    } else if (warp < 6) {
         const int q = warp & 3;
         const int row = 32 * q + lane;
         // this warp's staging area for bulk stores: four 64-column boxes of
@@ -1030,6 +976,66 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (lane == 0) bulk_wait_all();  // the stores are done before the CTA's shared memory goes away
         __syncwarp();
     }
+}
+
+// The form goes by the call's tokens per work item and by its items, which only
+// the device knows.  With tokens as M an item costs the same however few tokens
+// it has, and fewer items than SMs leave SMs idle; with weights as M an item
+// costs by its tokens.  Whole layers, us, weights / tokens as M (tokens an item):
+//   8B, 300 tokens    (32) 144/146   (48) 165/161   (80) 217/195   (86, 2 items an expert) 392/293
+//   13B, 2000 tokens  (28) 156/167   (46) 184/182   (83) 245/225
+//   GPT-2-medium, 600 tokens  (47, 64 items) 29/30   (81, 104 items) 40/38
+//   d = 4096, 12 experts, 300 tokens  (100, 12 items) 49/67
+// By the call's tokens alone (rows above 1024) dense prompts of 257 to 1024
+// tokens took up to half as long again: 13B, 1024 tokens, every expert 2577 us,
+// 1738 by this rule.
+constexpr int kDownRowsMinItem = 48;
+
+__global__ void __launch_bounds__(kDnThreads, 1)
+    down_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_wd,
+                const __grid_constant__ CUtensorMap map_h128, const __grid_constant__ CUtensorMap map_wd256,
+                const __grid_constant__ CUtensorMap map_y, const int* __restrict__ cnt, const int* __restrict__ ltok, int T,
+                int E, int d, __nv_bfloat16* Y, long long ycap, float* yacc, unsigned* status, uint64_t lim) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    __shared__ DownShared sh;
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kDnStages; i++) {
+            mbar_init(&sh.full[i], 1);
+            mbar_init(&sh.empty[i], 1);
+        }
+        for (int i = 0; i < kDnAcc; i++) {
+            mbar_init(&sh.tfull[i], 1);
+            mbar_init(&sh.tempty[i], kDnEpi);
+        }
+        for (int i = 0; i < kDrStages; i++) {
+            mbar_init(&sh.rfull[i], 1);
+            mbar_init(&sh.rempty[i], 1);
+        }
+        for (int i = 0; i < 2; i++) {
+            mbar_init(&sh.rtfull[i], 1);
+            mbar_init(&sh.rtempty[i], 4);
+        }
+        mbar_init(&sh.afull, 1);
+        mbar_init(&sh.aempty, 1);
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(&sh.taddr, 512);
+        tmem_relinquish();
+    }
+    pdl_wait();  // the previous kernel on the stream has completed (programmatic dependent launch)
+    pdl_launch_dependents();
+    sh.tab.build(cnt, E);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = sh.taddr;
+    if (sh.tab.n_pairs() >= kDownRowsMinItem * sh.tab.n_items() && 2 * sh.tab.n_items() >= (int)gridDim.x)
+        down_rows(map_h128, map_wd256, map_y, sh, smem, tmem, ltok, T, d, Y, ycap, yacc, status, lim);
+    else
+        down_tiles(map_h, map_wd, sh, smem, tmem, ltok, T, d, Y, ycap, yacc, status, lim);
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
@@ -1189,27 +1195,22 @@ cudaError_t grouped_ffn(const GroupedArgs& a, int sms, cudaStream_t st) {
         !encode_2d(&mh, a.H, 64, (uint64_t)g.nnz_max + 128, 64, kDnBox) ||
         !encode_2d(&mwd, a.Wd, rows, a.d, 64, 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
         return cudaErrorInvalidValue;
-    const size_t gu_smem = kGuRing + kGuSlack + 1024, dn_smem = kDnRing + 4 * kDnStageOut + 1024;
+    // (down: the larger of the two forms' rings and staging areas)
+    const size_t gu_smem = kGuRing + kGuSlack + 1024;
+    const size_t dn_smem =
+        std::max(kDnRing + 4 * kDnStageOut, (size_t)kTileBytesA + kDrStages * (size_t)kDrTileB + 4 * (size_t)16384) + 1024;
+    CUtensorMap mh128, mwd256, my;
+    if (!encode_2d(&mh128, a.H, 64, (uint64_t)g.nnz_max + 128, 64, 128) ||
+        !encode_2d(&mwd256, a.Wd, rows, a.d, 64, 256, CU_TENSOR_MAP_L2_PROMOTION_L2_128B) ||
+        !encode_2d(&my, a.Y, a.d, (uint64_t)g.ycap, 64, 32))
+        return cudaErrorInvalidValue;
     cudaError_t e;
-    if ((e = set_smem(gu_gemm_kernel, gu_smem)) != cudaSuccess || (e = set_smem(down_gemm_kernel, dn_smem)) != cudaSuccess)
+    if ((e = set_smem(gu_gemm_kernel, gu_smem)) != cudaSuccess || (e = set_smem(down_kernel, dn_smem)) != cudaSuccess)
         return e;
     PP_LAUNCH(gu_gemm_kernel, dim3(sms), dim3(kGuThreads), gu_smem, st, mx, mwg, mwu, a.cnt, a.ltok, a.lgate, a.offsets, a.T,
               a.E, a.d, g.nk, a.act, a.H, g.ycap, a.yacc, a.status, a.timeout_ns);
-    if (a.T <= kDownRowsMinT) {
-        PP_LAUNCH(down_gemm_kernel, dim3(sms), dim3(kDnThreads), dn_smem, st, mh, mwd, a.cnt, a.ltok, a.T, a.E, a.d,
-                  (a.d + 127) / 128, a.Y, g.ycap, a.yacc, a.status, a.timeout_ns);
-    } else {
-        // A tile, the 4-stage W_down ring, 4 x 16 KB store staging
-        const size_t smem = (size_t)kTileBytesA + 4 * (size_t)256 * 128 + 4 * (size_t)16384 + 1024;
-        CUtensorMap mh128, mwd256, my;
-        if (!encode_2d(&mh128, a.H, 64, (uint64_t)g.nnz_max + 128, 64, 128) ||
-            !encode_2d(&mwd256, a.Wd, rows, a.d, 64, 256, CU_TENSOR_MAP_L2_PROMOTION_L2_128B) ||
-            !encode_2d(&my, a.Y, a.d, (uint64_t)g.ycap, 64, 32))
-            return cudaErrorInvalidValue;
-        if ((e = set_smem(down_rows_kernel, smem)) != cudaSuccess) return e;
-        PP_LAUNCH(down_rows_kernel, dim3(sms), dim3(kTcThreads), smem, st, mh128, mwd256, my, a.cnt, a.ltok, a.T, a.E, a.d,
-                  (a.d + 255) / 256, a.Y, g.ycap, a.yacc, a.status, a.timeout_ns);
-    }
+    PP_LAUNCH(down_kernel, dim3(sms), dim3(kDnThreads), dn_smem, st, mh, mwd, mh128, mwd256, my, a.cnt, a.ltok, a.T, a.E, a.d,
+              a.Y, g.ycap, a.yacc, a.status, a.timeout_ns);
     PP_LAUNCH(combine_kernel, dim3(a.T, (a.d + 1023) / 1024), dim3(128), 0, st, a.bits, a.slot_of, a.offsets, a.Y, g.ycap,
               a.yacc, a.T, a.E, a.d, reinterpret_cast<__nv_bfloat16*>(a.y));
     return cudaGetLastError();
