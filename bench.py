@@ -275,8 +275,9 @@ def kernel_traffic(workload, p, B, kind="decode"):
 # source files each timed kernel is built from: a DRAM-traffic record stays
 # valid while these are unchanged
 KERNEL_SOURCES = {
-    "decode": ["decode.cu", "pp_common.cuh", "pp_select.cuh", "pp_kernels.h", "api.cu"],
-    "grouped": ["grouped.cu", "union.cu", "pp_common.cuh", "pp_launch.h", "pp_select.cuh", "pp_tc.cuh",
+    "decode": ["decode.cu", "pp_union.cuh", "pp_common.cuh", "pp_launch.h", "pp_select.cuh", "pp_tc.cuh",
+               "pp_kernels.h", "api.cu"],
+    "grouped": ["grouped.cu", "union.cu", "pp_union.cuh", "pp_common.cuh", "pp_launch.h", "pp_select.cuh", "pp_tc.cuh",
                 "pp_kernels.h", "api.cu"],
 }
 

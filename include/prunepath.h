@@ -154,7 +154,8 @@ pp_status pp_sparse_ffn(const pp_desc *desc, const void *x, int T, const void *W
                         void *ws, size_t ws_bytes, void *stream);
 
 /* pp_route followed by pp_sparse_ffn, fused where the token count allows.
-   sel_out may be NULL (the selection then stays in the workspace). */
+   The selection is pp_route's, to the last bit; y agrees with pp_sparse_ffn's
+   to rounding.  sel_out may be NULL (the selection is then not written). */
 pp_status pp_layer(const pp_desc *desc, const void *x, int T, const void *W_r, const void *W_gate,
                    const void *W_up, const void *W_down, float p, const pp_selection *sel_out,
                    void *y, void *ws, size_t ws_bytes, void *stream);
@@ -168,9 +169,9 @@ pp_status pp_layer(const pp_desc *desc, const void *x, int T, const void *W_r, c
    y_prev may be NULL (no residual term: the first layer) and gamma NULL
    (unit weights).  The sum and the mean square are fp32; x is stored in the
    desc dtype and the layer reads exactly that x.  Where the fused decode
-   kernel runs the layer (up to 4 bf16 / 8 fp32 tokens, but not 2 to 4 tokens
-   of a wide layer with a large p) it forms x in its prologue (one launch);
-   otherwise one more kernel runs first.  x and y must not overlap x_prev,
+   kernel runs the layer (up to 4 bf16 / 8 fp32 tokens, but not 2 to 4 tokens of
+   a wide layer) it forms x in its prologue (one launch); otherwise one more
+   kernel runs first.  x and y must not overlap x_prev,
    y_prev or each other (PP_ERR_INVALID_ARG); eps >= 0. */
 pp_status pp_layer_chained(const pp_desc *desc, const void *x_prev, const void *y_prev, const void *gamma,
                            float eps, int T, const void *W_r, const void *W_gate, const void *W_up,
@@ -183,7 +184,8 @@ pp_status pp_layer_chained(const pp_desc *desc, const void *x_prev, const void *
    that exposes no allocator.  The paper has no counterpart: this entry point
    exists only for those callers.
    Same computation and arguments as pp_layer, for T <= 4 tokens and without a
-   workspace.  Like pp_layer, it runs the tokens in slices when one fused
+   workspace (the same selection to the last bit; y to rounding where pp_layer
+   goes on with the tensor cores, 2 to 4 tokens that select many experts).  Like pp_layer, it runs the tokens in slices when one fused
    launch cannot hold them all (fp32 rows of a wide model).  Its scratch (status word, per-CTA launch counts, router
    logits and gate/up activations: 533,760 bytes) is one static
    device array that every GPU loading this library keeps until the process

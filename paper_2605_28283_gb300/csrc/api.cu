@@ -50,31 +50,29 @@ constexpr int kGroupedMinT = 5;
 
 bool use_grouped(const pp_desc& d, int T) { return d.dtype == PP_BF16 && T >= kGroupedMinT; }
 
-// Whole bf16 layers of 2 to 4 tokens that read enough weights for the union
-// kernel: it streams them at 5-6 TB/s behind about 26 us of phases, the fused
-// decode kernel at 1.9 TB/s (fp32 products of every token) behind 10.  How many
-// experts a call selects is known only on the device; the lines lie where the
-// two measured the same on the 7B, 8B and 13B shapes (270-425 MB of expert
-// weights, router logits with a spread of 2 to 4), in us, fused / union:
-//   8B, 4 tokens: p = 0.5 30/32, 0.7 44/37, 0.9 80/51, 1 146/77; top-4 31/33, top-12 48/39
-//   8B, 3 tokens: p = 0.7 32/34, 0.8 41/37, 0.9 58/45
-//   8B, 2 tokens: p = 0.9 38/41, 0.95 48/46, 1 94/77; top-12 26/34
-//   7B, 3 tokens: p = 0.8 36/36;  13B, 3 tokens: p = 0.8 37/36;  13B, 2 tokens: p = 0.95 43/45
-//   4 tokens, LTE at 0.95: 69/47; 3 tokens 50/43; 2 tokens 34/39
-// GPT-2-medium (17 MB) is faster fused up to p = 0.95 (4 tokens at 0.9: 18/23).
-constexpr size_t kUnionMinBytes = (size_t)128 << 20;
+// Whole bf16 layers of 2 to 4 tokens: the fused decode kernel makes the selection
+// and, where the tokens selected enough experts together, goes on with the union
+// kernel's phases, which read weights at 5-6 TB/s behind about 15 us more of
+// phases; the fused ones take fp32 products of every token (1.9 TB/s at four).
+// The line lies where the two measured the same, in bytes of the selected
+// experts' weights (8B and 13B shapes; experts (MiB), us a layer, fused / union):
+//   2 tokens: 8B  51 (76) 33/38, 224 (336) 94/78;          13B  29 (54) 30/37, 68 (128) 49/45
+//   3 tokens: 8B  25 (38) 28/33, 40 (60) 36/37, 70 (105) 50/43;  13B  29 (54) 39/39, 40 (75) 48/44
+//   4 tokens: 8B  31 (47) 33/36, 38 (57) 40/37, 89 (133) 68/48;  13B  21 (39) 34/37, 30 (56) 43/40
+// Chosen by the rule's parameter instead (from p = 0.65 at four tokens), a router
+// that selects one or two experts a token paid the union kernel's phases: 4 tokens,
+// p = 0.7, 5 experts together 31 us, now 16 (fused 19).
+constexpr size_t kUnionSmallMiB[kGroupedMinT] = {0, 0, 104, 62, 48};
 
-// Shapes and token counts of which some call may take the union kernel.
-bool union_small_shape(const pp_desc& d, int T) {
-    return d.dtype == PP_BF16 && T >= 2 && T < kGroupedMinT &&
-           (size_t)(d.act == PP_ACT_SWIGLU ? 3 : 2) * d.d_ff * d.d_model * 2 >= kUnionMinBytes;
+// Experts from which a call of 2 to 4 tokens takes the union phases.
+int union_small_min(const pp_desc& d, int T) {
+    const size_t expert = (size_t)(d.act == PP_ACT_SWIGLU ? 3 : 2) * kDExpert * d.d_model * 2;
+    return (int)(((kUnionSmallMiB[T] << 20) + expert - 1) / expert);
 }
 
-bool use_union_small(const pp_desc& d, int T, float p) {
-    if (!union_small_shape(d, T)) return false;
-    if (d.rule == PP_SEL_MIN_PREFIX || d.rule == PP_SEL_PAPER) return p >= (T == 4 ? 0.65f : T == 3 ? 0.8f : 0.97f);
-    if (d.rule == PP_SEL_TOPK) return T >= 3 && T * p >= 32.0f;
-    return T >= 3;  // LTE
+// Shapes and token counts of which some call may take the union phases.
+bool union_small_shape(const pp_desc& d, int T) {
+    return d.dtype == PP_BF16 && T >= 2 && T < kGroupedMinT && d.n_experts >= union_small_min(d, T);
 }
 
 // Workspace layout of calls with T tokens.  Its size never falls as T grows: a
@@ -105,11 +103,13 @@ Layout layout(const pp_desc& d, int T) {
     L.tlog = take(8 * E * 8);
     L.th = take(E * 8 * kDExpert * 8);
     L.stats = take((size_t)router_stats_blocks((int)Tn) * (E + 2) * 8);
-    if (use_grouped(d, T) || union_small_shape(d, T)) {
-        const GroupedPlan g = grouped_plan(T, d.d_model, d.n_experts, 152);
+    if (use_grouped(d, T)) {
         L.part = take(router_part_rows(T, d.d_model, 152) * E * 4);
         L.bits = take(Tn * 8 * 4);
         L.gexp = take(Tn * E * 4);
+    }
+    if (use_grouped(d, T) || union_small_shape(d, T)) {
+        const GroupedPlan g = grouped_plan(T, d.d_model, d.n_experts, 152);
         L.H = take(std::max((size_t)g.nnz_max + 128, 15 * E) * kDExpert * 2);  // three terms of up to 5 tokens
         // the union kernel's partial tiles, or the prompt path's lists and rows
         const size_t dpart = union_part_floats((int)Tn, d.d_model) * 4;
@@ -234,10 +234,10 @@ bool make_down_map(const pp_desc& d, const void* Wd, int R6, CUtensorMap* map) {
     return r == CUDA_SUCCESS;
 }
 
-DecodePlanIn plan_in(const pp_desc& d, int TS, bool chain = false) {
+DecodePlanIn plan_in(const pp_desc& d, int TS, bool chain = false, bool uni = false) {
     const DeviceInfo di = device_info();
     return DecodePlanIn{d.dtype, d.d_model, d.n_experts, TS, di.sms, d.act == PP_ACT_SWIGLU,
-                        di.smem_optin - kDecodeStaticSmemReserve, chain};
+                        di.smem_optin - kDecodeStaticSmemReserve - (uni ? kUnionStaticSmemReserve : 0), chain};
 }
 
 // The chained step's extra inputs (pp_layer_chained); NULL for a plain layer.
@@ -298,17 +298,23 @@ GroupedArgs grouped_args(const pp_desc& d, int T, void* ws, const void* x, const
     return a;
 }
 
-// One launch of the fused decode kernel over tokens [t0, t0 + n).
+// One launch of the fused decode kernel over tokens [t0, t0 + n).  `ws` (plain
+// layers, all of the call's tokens): the workspace, for the union phases.
 pp_status decode_call(const pp_desc& d, const void* x, int t0, int n, const void* Wr, const void* Wg,
                       const void* Wu, const void* Wd, float p, const pp_selection* sel, bool do_route,
                       bool do_ffn, void* y, const Ws& w, cudaStream_t st, const Chain* chain = nullptr,
-                      unsigned long long* tline = nullptr) {
+                      unsigned long long* tline = nullptr, void* ws = nullptr) {
     const DeviceInfo di = device_info();
     int TS = 1;
     while (TS < n) TS <<= 1;
     if (TS > decode_max_ts(d.dtype)) return PP_ERR_SHAPE;
     DecodePlan plan;
-    if (!decode_plan(plan_in(d, TS, chain != nullptr), &plan)) return PP_ERR_SHAPE;
+    bool use_uni = ws && union_small_shape(d, n) && di.sms <= kUnionMaxGrid;
+    if (use_uni) {
+        const DecodePlanIn in = plan_in(d, TS, false, true);
+        use_uni = decode_plan(in, &plan) && plan.off_union + (size_t)kDecodeUnionRing <= in.smem_limit;
+    }
+    if (!use_uni && !decode_plan(plan_in(d, TS, chain != nullptr), &plan)) return PP_ERR_SHAPE;
     DecodeArgs a;
     std::memset(&a, 0, sizeof a);
     const size_t esz = d.dtype == PP_BF16 ? 2 : 4;
@@ -353,6 +359,7 @@ pp_status decode_call(const pp_desc& d, const void* x, int t0, int n, const void
     a.off_ring6 = plan.off_ring6;
     a.off_ring4 = plan.off_ring4;
     a.off_chain = plan.off_chain;
+    a.off_union = plan.off_union;
     if (chain) {
         const size_t esz = d.dtype == PP_BF16 ? 2 : 4;
         a.chain = 1;
@@ -362,7 +369,14 @@ pp_status decode_call(const pp_desc& d, const void* x, int t0, int n, const void
         a.eps = chain->eps;
     }
     a.tline = tline;
-    return cuda_status(decode_launch(a, plan, d.dtype, TS, di.sms, st));
+    UnionFfn uni;
+    if (use_uni) {
+        std::memset(&uni, 0, sizeof uni);
+        const GroupedArgs g = grouped_args(d, n, ws, x, Wr, Wg, Wu, Wd, p, pp_selection{}, y);
+        if (!union_ffn_args(g, di.sms, &uni)) return PP_ERR_CUDA;
+        a.union_min = union_small_min(d, n);
+    }
+    return cuda_status(decode_launch(a, plan, d.dtype, TS, di.sms, use_uni ? &uni : nullptr, st));
 }
 
 RouteArgs route_args(const pp_desc& d, const void* x, int T, const void* Wr, float kp, const pp_selection& s, const Ws& w,
@@ -547,7 +561,7 @@ pp_status pp_layer(const pp_desc* desc, const void* x, int T, const void* W_r, c
     const Ws w = ws_views(*desc, T, ws);
     pp_selection s = sel_out ? *sel_out : pp_selection{w.ids, w.counts, w.gates, nullptr};
     const float kp = rule_kernel_param(desc->rule, p, desc->n_experts);
-    if (use_grouped(*desc, T) || use_union_small(*desc, T, p)) {
+    if (use_grouped(*desc, T)) {
         GroupedArgs a = grouped_args(*desc, T, ws, x, W_r, W_gate, W_up, W_down, kp, s, y);
         if (!sel_out) {  // nobody reads the rank order
             a.ids = a.counts = nullptr;
@@ -560,7 +574,8 @@ pp_status pp_layer(const pp_desc* desc, const void* x, int T, const void* W_r, c
     const int ts = decode_ts_limit(*desc);
     if (ts == 0) return PP_ERR_SHAPE;
     if (T <= ts)
-        return decode_call(*desc, x, 0, T, W_r, W_gate, W_up, W_down, kp, sel_out, true, true, y, w, st);
+        return decode_call(*desc, x, 0, T, W_r, W_gate, W_up, W_down, kp, sel_out, true, true, y, w, st, nullptr, nullptr,
+                           ws);
     if (desc->dtype == PP_F32) {
         RouteArgs r = route_args(*desc, x, T, W_r, kp, s, w, true);
         if (!sel_out) {  // nobody reads the rank order
@@ -604,8 +619,11 @@ pp_status pp_layer_chained(const pp_desc* desc, const void* x_prev, const void* 
     if (T == 0) return PP_OK;
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Ws w = ws_views(*desc, T, ws);
-    // fused: the decode kernel forms x in its prologue
-    if (!use_grouped(*desc, T) && !use_union_small(*desc, T, p)) {
+    // fused: the decode kernel forms x in its prologue; where the union phases may
+    // follow, which need x in memory, a kernel of its own forms it (8B, 4 tokens,
+    // us a layer: 49.7 at p = 0.9 and 22.6 at 0.3, against 53.4 and 24.1 with x
+    // formed by every CTA and handed over by CTA 0)
+    if (!use_grouped(*desc, T) && !union_small_shape(*desc, T)) {
         const int ts = decode_ts_limit(*desc);
         DecodePlan plan;
         int TS = 1;

@@ -27,9 +27,17 @@
 // (Control.epoch[b], the same in every CTA because every launch runs one CTA
 // per SM and each CTA adds 1 to its own count), so words of an earlier
 // launch never match.  Only the selected expert blocks are read from HBM.
+//
+// 2 to 4 tokens of wide bf16 layers (UNI): CTA t selects token t and publishes its
+// gate weights as tagged words, and where the tokens selected many experts together
+// the FFN is that of the union kernel (pp_union.cuh) instead of phases 4 and 6.
+#include <type_traits>
+
 #include "pp_common.cuh"
 #include "pp_kernels.h"
+#include "pp_launch.h"
 #include "pp_select.cuh"
+#include "pp_union.cuh"
 
 namespace pp {
 
@@ -99,13 +107,56 @@ PP_DEVINL void decode_select_cta(const DecodeArgs& a, unsigned tag, float* gw, u
     }
 }
 
+// The same of token t alone, published by this CTA.
+PP_DEVINL void decode_select_token(const DecodeArgs& a, unsigned tag, int t, float* gw, unsigned* mask, CtaSelScratch& sc) {
+    const int j = threadIdx.x, E = a.E;
+    bool on;
+    int r;
+    float g;
+    const unsigned long long* row = a.tlog + (size_t)t * E;
+    const int k = cta_select_fn([&](int i) { return wait_tagged(row + i, tag, a.status, a.timeout_ns); }, E, a.p, a.rule,
+                                a.sel_ids != nullptr, sc, a.status, &on, &r, &g);
+    if (j < E) {
+        const float gv = on ? (a.gate == PP_GATE_NONE ? 1.0f : sigmoidf_(g)) : 0.0f;
+        if (on) {
+            gw[t * E + j] = gv;
+            mask[j] |= 1u << t;
+        }
+        if (a.sel_ids) write_selection_row(a.sel_ids + (size_t)t * E, a.sel_gates + (size_t)t * E, j, E, k, on, r, gv);
+        if (a.sel_logits) a.sel_logits[(size_t)t * E + j] = g;
+    }
+    if (j == 0 && a.sel_counts) a.sel_counts[t] = k;
+    __syncthreads();
+}
+
+struct NoUnion {};
+
+struct DecodeUnionArgs : DecodeArgs {
+    UnionFfn uni;
+};
+
+// The FFN of a call that selected many experts (UNI instantiations): the
+// phases of the union kernel over the ring at `smem`, from the selection in
+// shared memory.  Out of line: the other calls never fetch it.
+static __device__ __noinline__ void union_ffn(const UnionFfn& f, UnionShared<4>& sh, const float* gw, unsigned char* smem,
+                                              int nU) {
+    const uint32_t cols = union_cols(f, 0), tmem = union_begin(f, sh, cols);
+    auto gate = [gw, E = f.E](int t, int e) { return gw[t * E + e]; };
+    gu_phase<kDecodeUnionRing>(f, sh, gate, smem, tmem, nU);
+    down_phase<kDecodeUnionRing>(f, sh, gate, smem, tmem, nU);
+    union_end(tmem, cols);
+}
+
 // CHAIN: the chained step's prologue (a.chain) is compiled only into its own
 // instantiations, so that the plain layer's kernel carries no extra code.
 // TL: the timeline instantiation, which also records the global timer at
 // the phase boundaries of every CTA into a.tline[CTA][kDecodeStamps] (a
 // diagnostic; the plain kernel has no such stores).
-template <typename TW, int TS, int RPL, bool CHAIN, bool TL>
-__global__ void __launch_bounds__(kDecThreads, 1) decode_layer_kernel(const __grid_constant__ DecodeArgs a) {
+// UNI: calls that select a.union_min experts or more do their FFN by the
+// union phases (2 to 4 tokens of wide bf16 layers; decode_launch).
+template <typename TW, int TS, int RPL, bool CHAIN, bool TL, bool UNI>
+__global__ void __launch_bounds__(kDecThreads, 1)
+    decode_layer_kernel(const __grid_constant__ std::conditional_t<UNI, DecodeUnionArgs, DecodeArgs> a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     using EL = Elem<TW>;
     constexpr int kEl = EL::kPer16B;
@@ -131,6 +182,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_layer_kernel(const __gr
     __shared__ int s_nU;
     __shared__ int s_wcount[kWarps];
     __shared__ unsigned s_tag;
+    __shared__ std::conditional_t<UNI, UnionShared<4>, NoUnion> ush;
     __shared__ int s_k[TS];  // activated experts per token (cumulative-mass cut)
     // timeline stamp i of this CTA (TL instantiation, called by thread 0 only):
     // the global timer at entry, then that plus the SM cycles since entry at
@@ -198,6 +250,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_layer_kernel(const __gr
         const unsigned ep = a.epochs[b];
         a.epochs[b] = ep + 1u;
         s_tag = ep + 1u;
+        if constexpr (UNI) ush.bar_target = grid_bar_base(a.uni.bar, G);
     }
     // every CTA waits for its copy of x here, so no bulk copy is ever still
     // in flight when a CTA that has no work left exits
@@ -317,7 +370,57 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_layer_kernel(const __gr
         }
         if (TL && tid == 0) stamp(kStRouter);
         const bool publish = b == 0;
-        if (mass_cut) {
+        if constexpr (UNI) {
+            // CTA t selects token t (all tokens in every CTA took 2 us each) and
+            // publishes its gate weights as tagged words, which every CTA reads: a
+            // word of +0 where the expert is not activated (a weight of zero is
+            // -0).  They lie in the half of th that T <= 4 tokens leave free.
+            unsigned long long* tg = a.th + (size_t)E * 4 * kDExpert;
+            if (b < T) {
+                const int t = b;
+                float* gr = gw + t * E;
+                if (mass_cut) {
+                    const float g = tid < E ? wait_tagged(a.tlog + (size_t)t * E + tid, tag, a.status, lim) : -INFINITY;
+                    const int k = group_mass_cut(
+                        g, E, a.p, a.rule, cut_sc[0], reinterpret_cast<WarpCand*>(ring6), a.status, 0, kDecThreads,
+                        [&](int r, int e, float ge) {
+                            const float gv = a.gate == PP_GATE_NONE ? 1.0f : sigmoidf_(ge);
+                            gr[e] = gv;
+                            mask[e] = 1u;
+                            if (a.sel_ids) {
+                                a.sel_ids[(size_t)t * E + r] = e;
+                                a.sel_gates[(size_t)t * E + r] = gv;
+                            }
+                        },
+                        [] {});
+                    if (a.sel_ids && tid >= k && tid < E) {
+                        a.sel_ids[(size_t)t * E + tid] = -1;
+                        a.sel_gates[(size_t)t * E + tid] = 0.0f;
+                    }
+                    if (a.sel_logits && tid < E) a.sel_logits[(size_t)t * E + tid] = g;
+                    if (tid == 0 && a.sel_counts) a.sel_counts[t] = k;
+                } else {
+                    decode_select_token(a, tag, t, gw, mask, sel_sc);
+                }
+                if (tid < E) st_tagged(tg + (size_t)t * E + tid, tag, mask[tid] && gr[tid] == 0.0f ? -0.0f : gr[tid]);
+                fence_proxy_async_smem();  // the candidate list in the ring is dead
+            }
+            if (tid < E) {
+                unsigned long long w[TS];
+                unsigned m = 0u;
+#pragma unroll
+                for (int t = 0; t < TS; t++) w[t] = t < T ? ld_relaxed_u64(tg + (size_t)t * E + tid) : 0ull;
+#pragma unroll
+                for (int t = 0; t < TS; t++) {
+                    if (t >= T) break;
+                    const float v = word_tag(w[t]) == tag ? word_value(w[t])
+                                                          : wait_tagged(tg + (size_t)t * E + tid, tag, a.status, lim);
+                    gw[t * E + tid] = v;
+                    if (__float_as_uint(v) != 0u) m |= 1u << t;
+                }
+                mask[tid] = m;
+            }
+        } else if (mass_cut) {
             // cumulative-mass cut of every token: the tokens are cut side by
             // side by groups of nt threads (the smallest of 32, 64, 128, 256
             // that holds E experts; up to TS groups, each with its own named
@@ -417,6 +520,13 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_layer_kernel(const __gr
     }
     const int nU = a.do_route && mass_cut && TS == 1 ? s_k[0] : s_nU;
     if (TL && tid == 0) stamp(kStUnion);
+    if constexpr (UNI) {
+        if (a.do_route && nU >= a.union_min) {
+            if (tid < nU) ush.ul[tid] = ulist[tid];
+            union_ffn(a.uni, ush, gw, smem + a.off_union, nU);
+            return;
+        }
+    }
 
     // phase-6 geometry: CTA b owns rows [r0, r0 + rows) of W_down and y;
     // warp w handles experts u = w + 8 i of U (i < nt_w)
@@ -705,8 +815,6 @@ bool decode_plan(const DecodePlanIn& in, DecodePlan* out) {
     const size_t stage4 = (size_t)(in.gated ? 2 : 1) * in.d * esz;
     const int rpc = (in.E + G - 1) / G;
     size_t off = align_up(kNumBars * 8, 128);
-    p.off_x = (uint32_t)off;
-    off = align_up(off + (size_t)TS * in.d * esz, 128);
     p.off_gw = (uint32_t)off;
     off = align_up(off + (size_t)TS * in.E * 4, 128);
     p.off_mask = (uint32_t)off;
@@ -716,7 +824,10 @@ bool decode_plan(const DecodePlanIn& in, DecodePlan* out) {
     p.off_red = (uint32_t)off;
     off = align_up(off + (size_t)kWarps * 2 * TS * 4, 128);
     p.off_red6 = (uint32_t)off;
-    off = align_up(off + (size_t)kWarps * p.R6 * TS * 4, 1024);
+    off = align_up(off + (size_t)kWarps * p.R6 * TS * 4, 128);
+    p.off_union = (uint32_t)align_up(off, 1024);  // (the union phases need x and the rings no more)
+    p.off_x = (uint32_t)off;
+    off = align_up(off + (size_t)TS * in.d * esz, 1024);
     const size_t budget = in.smem_limit;
     // dedicated phase-6 slots: 2 per warp when they fit comfortably, else 1
     p.ded6 = (off + 2 * kWarps * stage6 + 2 * stage4 <= budget) ? 2 : 1;
@@ -752,59 +863,52 @@ bool decode_plan(const DecodePlanIn& in, DecodePlan* out) {
     return true;
 }
 
-template <typename TW, int TS, int RPL, bool TL = false>
-static cudaError_t launch_one(const DecodeArgs& a, const DecodePlan& p, int grid, cudaStream_t st) {
-    auto kern = TL ? decode_layer_kernel<TW, TS, RPL, false, true>
-                   : (a.chain ? decode_layer_kernel<TW, TS, RPL, true, false> : decode_layer_kernel<TW, TS, RPL, false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+template <typename TW, int TS, int RPL, bool CHAIN, bool TL, bool UNI>
+static cudaError_t launch_kernel(const DecodeArgs& a, const DecodePlan& p, int grid, const UnionFfn* uni, cudaStream_t st) {
+    auto kern = decode_layer_kernel<TW, TS, RPL, CHAIN, TL, UNI>;
+    const size_t smem = UNI ? std::max(p.smem, (size_t)p.off_union + kDecodeUnionRing) : p.smem;
+    const cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(p.threads);
-    cfg.dynamicSmemBytes = p.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    e = cudaLaunchKernelEx(&cfg, kern, a);
-    if (e == cudaErrorNotSupported || e == cudaErrorInvalidValue) {
-        (void)cudaGetLastError();  // this runtime cannot combine the two attributes
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, kern, a);
-    }
-    return e;
+    if constexpr (UNI)
+        return launch_coop(kern, dim3(grid), dim3(p.threads), smem, st, DecodeUnionArgs{a, *uni});
+    else
+        return launch_coop(kern, dim3(grid), dim3(p.threads), smem, st, a);
+}
+
+template <typename TW, int TS, int RPL>
+static cudaError_t launch_one(const DecodeArgs& a, const DecodePlan& p, int grid, const UnionFfn* uni, cudaStream_t st) {
+    if constexpr (std::is_same_v<TW, __nv_bfloat16> && TS > 1)
+        if (uni) return launch_kernel<TW, TS, RPL, false, false, true>(a, p, grid, uni, st);
+    return a.chain ? launch_kernel<TW, TS, RPL, true, false, false>(a, p, grid, nullptr, st)
+                   : launch_kernel<TW, TS, RPL, false, false, false>(a, p, grid, nullptr, st);
 }
 
 template <typename TW, int TS>
-static cudaError_t launch_rpl(const DecodeArgs& a, const DecodePlan& p, int grid, cudaStream_t st) {
-    return p.RPL == 8 ? launch_one<TW, TS, 8>(a, p, grid, st) : launch_one<TW, TS, 16>(a, p, grid, st);
+static cudaError_t launch_rpl(const DecodeArgs& a, const DecodePlan& p, int grid, const UnionFfn* uni, cudaStream_t st) {
+    return p.RPL == 8 ? launch_one<TW, TS, 8>(a, p, grid, uni, st) : launch_one<TW, TS, 16>(a, p, grid, uni, st);
 }
 
 cudaError_t decode_launch(const DecodeArgs& a, const DecodePlan& p, int dtype, int TS, int grid,
-                          cudaStream_t st) {
+                          const UnionFfn* uni, cudaStream_t st) {
     if (grid < 1 || grid > kMaxGrid) return cudaErrorInvalidValue;  // one launch count per CTA
     if (a.tline) {  // the timeline instantiation exists for one bf16 token of a plain layer only
         if (dtype != PP_BF16 || TS != 1 || a.chain) return cudaErrorInvalidValue;
-        return p.RPL == 8 ? launch_one<__nv_bfloat16, 1, 8, true>(a, p, grid, st)
-                          : launch_one<__nv_bfloat16, 1, 16, true>(a, p, grid, st);
+        return p.RPL == 8 ? launch_kernel<__nv_bfloat16, 1, 8, false, true, false>(a, p, grid, nullptr, st)
+                          : launch_kernel<__nv_bfloat16, 1, 16, false, true, false>(a, p, grid, nullptr, st);
     }
     if (dtype == PP_BF16) {
         switch (TS) {
-            case 1: return launch_rpl<__nv_bfloat16, 1>(a, p, grid, st);
-            case 2: return launch_rpl<__nv_bfloat16, 2>(a, p, grid, st);
-            case 4: return launch_rpl<__nv_bfloat16, 4>(a, p, grid, st);
+            case 1: return launch_rpl<__nv_bfloat16, 1>(a, p, grid, nullptr, st);
+            case 2: return launch_rpl<__nv_bfloat16, 2>(a, p, grid, uni, st);
+            case 4: return launch_rpl<__nv_bfloat16, 4>(a, p, grid, uni, st);
             default: return cudaErrorInvalidValue;
         }
     }
     switch (TS) {
-        case 1: return launch_rpl<float, 1>(a, p, grid, st);
-        case 2: return launch_rpl<float, 2>(a, p, grid, st);
-        case 4: return launch_rpl<float, 4>(a, p, grid, st);
-        case 8: return launch_rpl<float, 8>(a, p, grid, st);
+        case 1: return launch_rpl<float, 1>(a, p, grid, nullptr, st);
+        case 2: return launch_rpl<float, 2>(a, p, grid, nullptr, st);
+        case 4: return launch_rpl<float, 4>(a, p, grid, nullptr, st);
+        case 8: return launch_rpl<float, 8>(a, p, grid, nullptr, st);
         default: return cudaErrorInvalidValue;
     }
 }

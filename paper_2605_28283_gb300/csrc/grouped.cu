@@ -179,7 +179,7 @@ PP_DEVINL void list_add(const Lists& l, int T, int E, int t, int e, float gv) {
 // until the rule stops, with the exact fixed-point masses of group_mass_cut, so
 // the decisions are the same.  An activated expert costs about 110 cycles and
 // nothing is sorted that is not activated: one CTA per token took 46 us for
-// 8192 tokens of 216 experts (7 activated each), this 20 us (under ncu).  ids and gates
+// 8192 tokens of 216 experts (6 activated each), this 20 us (under ncu).  ids and gates
 // (together), counts, logits_out may be NULL; so may bits with the lists.
 template <int S>
 __global__ void __launch_bounds__(256)

@@ -193,7 +193,7 @@ extern "C" pp_status pp_layer_noalloc(const pp_desc* desc, const void* x, int T,
             a.sel_gates = sel_out->gates + (size_t)t0 * E;
             a.sel_logits = sel_out->logits ? sel_out->logits + (size_t)t0 * E : nullptr;
         }
-        if (pp::decode_launch(a, plan, d.dtype, TS, ds->sms, st) != cudaSuccess) return PP_ERR_CUDA;
+        if (pp::decode_launch(a, plan, d.dtype, TS, ds->sms, nullptr, st) != cudaSuccess) return PP_ERR_CUDA;
     }
     if (status_out &&
         cudaMemcpyAsync(status_out, &ctl->status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, st) != cudaSuccess)

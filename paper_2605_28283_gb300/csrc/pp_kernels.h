@@ -37,7 +37,7 @@ struct DecodeArgs {
     float* sel_gates;
     float* sel_logits;     // route: optional output
     unsigned long long* tlog;  // [T][E] tagged logits
-    unsigned long long* th;    // [|U|][T][64] tagged gate/up activations
+    unsigned long long* th;    // [|U|][T][64] tagged gate/up activations ([E][8][64] words)
     unsigned* epochs;          // [grid] launch count per CTA (Control.epoch)
     unsigned* status;
     uint64_t timeout_ns;
@@ -46,7 +46,7 @@ struct DecodeArgs {
     float p;
     int do_route, do_ffn;
     int R6, NS4, ded6, slots6, hch;
-    uint32_t off_x, off_gw, off_mask, off_ulist, off_red, off_red6, off_ring6, off_ring4;
+    uint32_t off_x, off_gw, off_mask, off_ulist, off_red, off_red6, off_ring6, off_ring4, off_union;
     // chained step: x = RMSNorm(x_prev + y_prev) * gamma computed in the
     // prologue (a.x is then x_prev); y_prev and gamma staged in the phase-4
     // ring at off_chain (free until phase 4), x written to x_out by CTA 0
@@ -58,6 +58,22 @@ struct DecodeArgs {
     float eps;
     // timeline instantiation only: [grid][kDecodeStamps] global-timer stamps
     unsigned long long* tline;
+    int union_min;  // with a UnionFfn: the union kernel's phases do the FFN of this many experts or more
+};
+
+// The FFN over the union of a call's selected experts on the tensor cores
+// (pp_union.cuh).
+struct UnionFfn {
+    CUtensorMap map_x, map_wg, map_wu;  // gate/up
+    CUtensorMap map_h, map_wd;          // down
+    int T, E, d, N, terms, nk, ntile, slots, act;
+    __nv_bfloat16* H;  // [terms * T][E * 64]: activations at union position * 64 + neuron
+    float* dpart;
+    const __nv_bfloat16* Wd;
+    __nv_bfloat16* y;
+    unsigned long long* bar;
+    unsigned* status;
+    uint64_t lim;
 };
 
 // Phase boundaries recorded by the decode kernel's timeline instantiation,
@@ -96,6 +112,7 @@ struct DecodePlan {
     size_t smem;
     uint32_t off_x, off_gw, off_mask, off_ulist, off_red, off_red6, off_ring6, off_ring4;
     uint32_t off_chain;  // within the phase-4 ring: y_prev [TS][d] then gamma [d]
+    uint32_t off_union;  // ring of the union phases: x and everything after it
 };
 
 // Part of the per-block shared-memory limit left to the decode kernel's
@@ -103,9 +120,17 @@ struct DecodePlan {
 // the 1 KB alignment of the dynamic area).
 constexpr size_t kDecodeStaticSmemReserve = 6144;
 
+// The same for the barriers and tables of the union phases, in calls that may
+// take them.
+constexpr size_t kUnionStaticSmemReserve = 2048;
+// Ring of the union phases in the fused decode kernel: what every plan leaves
+// after its tables (DecodePlan.off_union).
+constexpr int kDecodeUnionRing = 200 * 1024;
+
 bool decode_plan(const DecodePlanIn& in, DecodePlan* out);
+// `uni` (NULL: none): the call may do its FFN by the union phases.
 cudaError_t decode_launch(const DecodeArgs& a, const DecodePlan& p, int dtype, int TS, int grid,
-                          cudaStream_t st);
+                          const UnionFfn* uni, cudaStream_t st);
 int decode_max_ts(int dtype);
 
 // --------------------------------------------------------- route / select
@@ -206,6 +231,8 @@ cudaError_t grouped_ffn(const GroupedArgs& a, int sms, cudaStream_t st);
 // The whole layer (do_route), or the FFN alone over a.bits / a.gexp, in one
 // cooperative launch; a.T <= kUnionMaxT.  a.ids, a.counts, a.gates may be NULL.
 cudaError_t union_layer(const GroupedArgs& a, bool do_route, int sms, cudaStream_t st);
+// The FFN part alone, for a kernel of `grid` CTAs (false: no tensor maps).
+bool union_ffn_args(const GroupedArgs& g, int grid, UnionFfn* a);
 // Columns of the router's MMA for E experts.
 inline int router_ne(int E) {
     return E <= 32 ? 32 : E <= 64 ? 64 : E <= 128 ? 128 : E <= 160 ? 160 : E <= 192 ? 192 : E <= 224 ? 224 : 256;

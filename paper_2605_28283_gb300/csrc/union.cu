@@ -1,5 +1,5 @@
-// Batched path for a few to a few hundred tokens (bf16, up to kUnionMaxT
-// tokens; below 5 where use_union in api.cu says so): one cooperative launch, one CTA per SM, for the whole layer, with
+// Batched path for a few to a few hundred tokens (bf16, 5 to kUnionMaxT
+// tokens): one cooperative launch, one CTA per SM, for the whole layer, with
 // the FFN evaluated over the union of the batch's selected experts.
 //
 // At these sizes the weights are the traffic (a 64-token Llama-3-8B call reads
@@ -33,99 +33,36 @@
 // Per layer of the 8B shape, against six kernels over 16-row items of whole
 // experts: 8 tokens 52 -> 39 us, 64 tokens 88 -> 75; GPT-2-medium, 16 tokens,
 // 28 -> 25.
-//
-// Warps: 0-3 producers of the gate/up ring and epilogues (TMEM lanes
-// 32 * warp ..), 4-5 MMA issue, 6 W_down producer, 7 H producer.
+//// The FFN phases are in pp_union.cuh.
 #include "pp_common.cuh"
 #include "pp_kernels.h"
 #include "pp_launch.h"
 #include "pp_select.cuh"
 #include "pp_tc.cuh"
+#include "pp_union.cuh"
 
 namespace pp {
 namespace {
 
-constexpr int kUnitRows = 16;                 // weight rows of a unit
-constexpr int kUnitBytes = kUnitRows * 128;   // per 64-wide K chunk
-constexpr int kPassUnits = 16;                // units of one pass: two M = 128 tiles
-constexpr int kTileUnits = 128 / kUnitRows;
-constexpr int kProd = 4;                      // producer / epilogue warps
-constexpr int kMmaWarp = 4;                   // first of the two MMA warps
-constexpr int kWdWarp = 6, kHWarp = 7;        // down projection: W_down and H producers
-constexpr int kThreads = 256;
-constexpr int kMaxStages = 16;
-constexpr int kTileW = 128 * 128;             // 128 rows x 64 bf16
 constexpr int kRouterStages = 4;
-// Dynamic shared memory: the ring of the phase that runs.  An MMA always reads
-// 128 weight rows, also where the last tile of a gate/up pass holds fewer
-// units, so that ring is followed by a tile's worth of slack.
-constexpr size_t kUnionSmem = 218 * 1024;
-constexpr size_t kGuSlack = kTileW - kUnitBytes;
-
-PP_DEVINL uint32_t tmem_cols(int n) { return n <= 32 ? 32u : n <= 64 ? 64u : n <= 128 ? 128u : n <= 256 ? 256u : 512u; }
-
-// Ring position: slot and phase parity, advanced without a division.
-struct Ring {
-    int s = 0;
-    uint32_t ph = 0;
-    PP_DEVINL void next(int n) {
-        if (++s == n) {
-            s = 0;
-            ph ^= 1u;
-        }
-    }
-};
-
-// The L = tiles * nU (row tile, union expert) pairs of the down projection (at
-// most 64 * 256) are cut into runs, one per CTA b < run_count; CTAs past it
-// have none.  A run has at least kMinRun pairs: every run ends in a partial
-// tile that the reduction reads back.
-constexpr int kMinRun = 2;
-PP_DEVINL int run_count(int L, int G) { return max(1, min(G, L / kMinRun)); }
-PP_DEVINL int run_begin(int L, int b, int R) { return b >= R ? L : L * b / R; }
-// The run that holds pair i: run_begin(b) <= i < run_begin(b + 1).
-PP_DEVINL int run_of(int L, int i, int R) { return ((i + 1) * R - 1) / L; }
+constexpr int kUnionSmem = 218 * 1024;  // dynamic: the ring of the phase that runs, aligned to 1 KB
 
 struct UnionArgs {
-    CUtensorMap map_rx, map_wr;        // router: x in 128-row boxes, W_r in rn-row boxes
-    CUtensorMap map_x, map_wg, map_wu; // gate/up
-    CUtensorMap map_h, map_wd;         // down
-    int T, E, d, N, terms, rn, nk, kpb, nsplit, mt, ntile, slots, act, gate, rule, do_route;
+    UnionFfn f;
+    CUtensorMap map_rx, map_wr;  // router: x in 128-row boxes, W_r in rn-row boxes
+    int rn, kpb, nsplit, mt, gate, rule, do_route;
     float p;
     float* part;            // router partials [nsplit][T][E]
     int32_t *ids, *counts;  // selection outputs (NULL: not wanted)
     float *gates, *logits;
     uint32_t* bits;
     float* gexp;
-    __nv_bfloat16* H;       // [terms * T][E * 64]: activations at union position * 64 + neuron
-    float* dpart;
-    const __nv_bfloat16* Wd;
-    __nv_bfloat16* y;
-    unsigned long long* bar;
-    unsigned* status;
-    uint64_t lim;
 };
 
-struct UnionShared {
-    uint64_t rfull[kRouterStages], rempty[kRouterStages], rdone;
-    uint64_t full[kMaxStages], empty[kMaxStages], tfull;             // gate/up
-    uint64_t dfull[kMaxStages], dempty[kMaxStages], dt[2], de[2];    // down
-    unsigned long long bar_target;  // arrivals that complete the last barrier this CTA has joined
-    uint32_t taddr, um[8];
-    int ul[kMaxExperts];
-    float gw[kPassUnits / 4 + 1][kUnionMaxT];  // gate weights of the pass's experts
+struct RouterShared {
+    uint64_t full[kRouterStages], empty[kRouterStages], done;
+    uint32_t um[8];  // the union's bits
 };
-
-// Every thread of the CTA: what it wrote is visible to every CTA's reads after.
-PP_DEVINL void grid_sync(const UnionArgs& a, UnionShared& sh) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        grid_arrive(a.bar);
-        sh.bar_target += gridDim.x;
-        grid_wait(a.bar, sh.bar_target, a.status, a.lim);
-    }
-    __syncthreads();
-}
 
 // Partial logits of (token tile, K split, group of rn experts): the chunks of a
 // split in the order of router_gemm_kernel, so a logit's sum is the same.  The
@@ -133,26 +70,26 @@ PP_DEVINL void grid_sync(const UnionArgs& a, UnionShared& sh) {
 // loads, MMAs (N = 32) and stores are a seventh (64 tokens: 6.1 -> 3.2 us).
 // The W_r tiles are requested before the previous kernel on the stream has
 // completed.
-PP_DEVINL void router_phase(const UnionArgs& a, UnionShared& sh, unsigned char* smem, uint32_t tmem) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ngrp = (a.E + a.rn - 1) / a.rn, tasks = a.mt * a.nsplit * ngrp, rstage = kTileW + a.rn * 128;
+PP_DEVINL void router_phase(const UnionArgs& a, RouterShared& sh, unsigned char* smem, uint32_t tmem) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ngrp = (a.f.E + a.rn - 1) / a.rn, tasks = a.mt * a.nsplit * ngrp, rstage = kTileW + a.rn * 128;
     uint32_t round = 0;
     int it0 = 0;  // chunks of this CTA's earlier rounds
     bool waited = false;
     for (int b = blockIdx.x; b < tasks; b += gridDim.x, round++) {
         const int e0 = (b % ngrp) * a.rn, m0 = (b / ngrp % a.mt) * 128, split = b / ngrp / a.mt;
-        const int k0 = split * a.kpb, n = min(a.nk, k0 + a.kpb) - k0;
+        const int k0 = split * a.kpb, n = min(a.f.nk, k0 + a.kpb) - k0;
         // warp w < 4 loads into stage w: chunk i of all the CTA's chunks is in stage i % 4
         if (warp < kRouterStages && lane == 0) {
             unsigned char* st = smem + (size_t)warp * rstage;
             for (int i = (warp - it0) & (kRouterStages - 1); i < n; i += kRouterStages) {
                 const int q = (it0 + i) / kRouterStages;
-                if (q > 0) mbar_wait(&sh.rempty[warp], (uint32_t)(q - 1) & 1u, a.status, a.lim);
-                mbar_arrive_expect_tx(&sh.rfull[warp], (uint32_t)rstage);
-                tma_load_2d(st + kTileW, &a.map_wr, (k0 + i) * 64, e0, &sh.rfull[warp]);
+                if (q > 0) mbar_wait(&sh.empty[warp], (uint32_t)(q - 1) & 1u, a.f.status, a.f.lim);
+                mbar_arrive_expect_tx(&sh.full[warp], (uint32_t)rstage);
+                tma_load_2d(st + kTileW, &a.map_wr, (k0 + i) * 64, e0, &sh.full[warp]);
                 if (!waited) pdl_wait();
                 waited = true;
-                tma_load_2d(st, &a.map_rx, (k0 + i) * 64, m0, &sh.rfull[warp]);
+                tma_load_2d(st, &a.map_rx, (k0 + i) * 64, m0, &sh.full[warp]);
             }
         }
         if (!waited) pdl_wait();
@@ -162,35 +99,35 @@ PP_DEVINL void router_phase(const UnionArgs& a, UnionShared& sh, unsigned char* 
             const uint32_t idesc = idesc_bf16_m128(a.rn);
             for (int i = 0; i < n; i++) {
                 const int s = (it0 + i) & (kRouterStages - 1);
-                mbar_wait(&sh.rfull[s], (uint32_t)((it0 + i) / kRouterStages) & 1u, a.status, a.lim);
+                mbar_wait(&sh.full[s], (uint32_t)((it0 + i) / kRouterStages) & 1u, a.f.status, a.f.lim);
                 tc_fence_after();
                 unsigned char* st = smem + (size_t)s * rstage;
                 umma_k64(tmem, st, st + kTileW, idesc, i > 0);
-                umma_commit(&sh.rempty[s]);
+                umma_commit(&sh.empty[s]);
             }
-            umma_commit(&sh.rdone);
+            umma_commit(&sh.done);
         }
         __syncwarp();
         it0 += n;
         // epilogue: lane = token row of TMEM lanes 32 * warp ..
         const int r0 = m0 + 32 * warp, t = r0 + lane;
-        if (warp < kProd && r0 < a.T) {
-            mbar_wait(&sh.rdone, round & 1u, a.status, a.lim);
+        if (warp < kProd && r0 < a.f.T) {
+            mbar_wait(&sh.done, round & 1u, a.f.status, a.f.lim);
             tc_fence_after();
-            for (int c = e0; c < min(e0 + a.rn, a.E); c += 32) {
+            for (int c = e0; c < min(e0 + a.rn, a.f.E); c += 32) {
                 uint32_t r[32];
                 tmem_ld32(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(c - e0), r);
                 tmem_ld_wait();
-                if (t >= a.T) continue;
-                float* row = a.part + ((size_t)split * a.T + t) * a.E + c;
-                if ((a.E & 3) == 0) {
+                if (t >= a.f.T) continue;
+                float* row = a.part + ((size_t)split * a.f.T + t) * a.f.E + c;
+                if ((a.f.E & 3) == 0) {
 #pragma unroll
                     for (int i = 0; i < 32; i += 4)
-                        if (c + i < a.E) *reinterpret_cast<uint4*>(row + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
+                        if (c + i < a.f.E) *reinterpret_cast<uint4*>(row + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
                 } else {
 #pragma unroll
                     for (int i = 0; i < 32; i++)
-                        if (c + i < a.E) row[i] = __uint_as_float(r[i]);
+                        if (c + i < a.f.E) row[i] = __uint_as_float(r[i]);
                 }
             }
             tc_fence_before();
@@ -202,17 +139,16 @@ PP_DEVINL void router_phase(const UnionArgs& a, UnionShared& sh, unsigned char* 
         pdl_wait();
         pdl_launch_dependents();
     }
-    if (tid == 32 * kHWarp) sh.bar_target = grid_bar_base(a.bar, gridDim.x);
 }
 
 // Selection of tokens b, b + G, ... from the summed partial logits.
 PP_DEVINL void select_phase(const UnionArgs& a, unsigned char* smem) {
     SelScratch& s = *reinterpret_cast<SelScratch*>(smem);
-    for (int t = blockIdx.x; t < a.T; t += gridDim.x) {
-        const size_t row = (size_t)t * a.E;
+    for (int t = blockIdx.x; t < a.f.T; t += gridDim.x) {
+        const size_t row = (size_t)t * a.f.E;
         auto logit = [&](int e) {  // partials added in split order, eight loads in flight
             const float* q = a.part + row + e;
-            const size_t stride = (size_t)a.T * a.E;
+            const size_t stride = (size_t)a.f.T * a.f.E;
             float v = 0.0f;
             int i = 0;
             for (; i + 8 <= a.nsplit; i += 8) {
@@ -227,469 +163,43 @@ PP_DEVINL void select_phase(const UnionArgs& a, unsigned char* smem) {
         };
         const SelOut o{a.ids ? a.ids + row : nullptr, a.counts ? a.counts + t : nullptr, a.gates ? a.gates + row : nullptr,
                        a.logits ? a.logits + row : nullptr, a.bits + (size_t)t * 8, a.gexp + row};
-        select_token_cta(logit, a.E, a.p, a.rule, a.gate, s, o, a.status);
+        select_token_cta(logit, a.f.E, a.p, a.rule, a.gate, s, o, a.f.status);
         __syncthreads();  // the scratch is reused by the next token
     }
 }
-
-// MMA warps of the down projection: two take a run's pairs in turn, each with
-// its own two accumulators (added in the epilogue); above 128 tokens the four
-// accumulators would not fit the tensor memory.
-PP_DEVINL int down_mma(int N) { return N <= 128 ? 2 : 1; }
-
-// Run of this CTA in the down projection.
-struct DownRun {
-    int R, n, tile0, first, stage, nst;
-    PP_DEVINL DownRun(const UnionArgs& a, int nU) {
-        const int L = a.ntile * nU;
-        R = run_count(L, gridDim.x);
-        const int i0 = run_begin(L, blockIdx.x, R);
-        n = run_begin(L, blockIdx.x + 1, R) - i0;
-        tile0 = n > 0 ? i0 / nU : 0;
-        first = n > 0 ? i0 % nU : 0;
-        stage = kTileW + a.N * 128;
-        nst = min(kMaxStages, (int)((kUnionSmem - 1024) / stage)) & ~1;  // even, as in gu_phase
-    }
-};
-
-PP_DEVINL void load_wd(const UnionArgs& a, UnionShared& sh, unsigned char* smem, const DownRun& d, int slot, int u, int tile) {
-    mbar_arrive_expect_tx(&sh.dfull[slot], (uint32_t)kTileW);
-    tma_load_2d(smem + (size_t)slot * d.stage, &a.map_wd, sh.ul[u] * kDExpert, tile * 128, &sh.dfull[slot]);
-}
-
-// The first W_down tiles of the run, one ring's worth (lane 0 of warp kWdWarp).
-PP_DEVINL void wd_prologue(const UnionArgs& a, UnionShared& sh, unsigned char* smem, int nU) {
-    if ((threadIdx.x & 31) == 0) {
-        const DownRun d(a, nU);
-        int u = d.first, tile = d.tile0;
-        for (int i = 0; i < min(d.n, d.nst); i++) {
-            load_wd(a, sh, smem, d, i, u, tile);
-            if (++u == nU) {
-                u = 0;
-                tile++;
-            }
-        }
-    }
-    __syncwarp();
-}
-
-// An activation in bf16, or as three bf16 terms (24 bits: the fp32 value) whose
-// rows are `next` elements apart.
-PP_DEVINL void store_h(__nv_bfloat16* p, float h, int terms, size_t next) {
-    const __nv_bfloat16 hi = __float2bfloat16_rn(h);
-    *p = hi;
-    if (terms == 1) return;
-    const float r = isfinite(h) ? h - __bfloat162float(hi) : 0.0f;
-    const __nv_bfloat16 mid = __float2bfloat16_rn(r);
-    p[next] = mid;
-    p[2 * next] = __float2bfloat16_rn(r - __bfloat162float(mid));
-}
-
-// Out of line: the epilogue runs once per launch and is bound by instruction
-// fetch (unrolled inline, 16 copies of the tanh form took 4.4 us at 16 tokens, 3.6 now).
-static __device__ __noinline__ float union_act(int act, float u, float g) { return act_h(act, u, g); }
-
-// h = act(gate, up) * gate weight of the pass's units [base, base + nun), bf16,
-// at H[t][union position * 64 + neuron].  Warps w and w + 4 share the TMEM lanes
-// 32 (w % 4) .. and take every other 16 tokens.  A token that did not select
-// the expert (most do not: 5 % of the pairs at 64 tokens of the 8B shape) costs
-// a store of zero and no activation.  `halves`: the sums are those of two
-// accumulators.
-// UN: how far the loops over the tokens are unrolled.  A column block of 16 that
-// is run once is bound by instruction fetch, so it is rolled (8 tokens of the 8B
-// shape: 321 -> 313 us for 8 layers); the four blocks of 64 tokens reuse the
-// unrolled code (604 against 612 us).
-template <int UN>
-PP_DEVINL void gu_epilogue(const UnionArgs& a, UnionShared& sh, uint32_t tmem, int base, int nun, int upe, bool halves) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3;
-    const int T = a.T, N = a.N, p0 = base / upe;
-    const bool gated = upe == 8;
-    const size_t ldh = (size_t)a.E * kDExpert;
-    for (int m = 0; m * kTileUnits < nun; m++) {
-        if (m * kTileUnits + q * 2 >= nun) break;  // no unit in this warp's lanes
-        const int ui = m * kTileUnits + q * 2 + (lane >> 4);  // this lane's unit of the pass
-        const bool live = ui < nun;
-        const int g = base + min(ui, nun - 1), p = g / upe;
-        const float* gt = sh.gw[p - p0];
-        const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(m * N);
-        // lane -> neuron: rows 0-7 of a gated unit are gate rows, 8-15 the up
-        // rows of the same neurons
-        __nv_bfloat16* Hn = a.H + (size_t)p * kDExpert + (gated ? (g % upe) * 8 + (lane & 7) : (g % upe) * 16 + (lane & 15));
-        for (int c = 16 * (warp >> 2); c < N; c += 32) {
-            uint32_t v[16];
-            tmem_ld16(ta + (uint32_t)c, v);
-            if (halves) {
-                uint32_t o[16];
-                tmem_ld16(ta + (uint32_t)(N + c), o);
-                tmem_ld_wait();
-#pragma unroll
-                for (int k = 0; k < 16; k++) v[k] = __float_as_uint(__uint_as_float(v[k]) + __uint_as_float(o[k]));
-            } else {
-                tmem_ld_wait();
-            }
-            if (gated) {
-                // gate lanes finish the even tokens, up lanes the odd ones
-                const bool up = (lane & 8) != 0;
-#pragma unroll UN
-                for (int k = 0; k < 8; k++) {
-                    const int t = c + 2 * k + (up ? 1 : 0);
-                    const float w = live && t < T ? gt[t] : 0.0f;
-                    float h = 0.0f;
-                    if (__any_sync(kFull, w != 0.0f)) {
-                        const float e0 = __uint_as_float(v[2 * k]), e1 = __uint_as_float(v[2 * k + 1]);
-                        const float o = __shfl_xor_sync(kFull, up ? e0 : e1, 8);
-                        if (w != 0.0f) h = union_act(PP_ACT_SWIGLU, up ? e1 : o, up ? o : e0) * w;
-                    }
-                    if (live && t < T) store_h(Hn + (size_t)t * ldh, h, a.terms, T * ldh);
-                }
-            } else {
-#pragma unroll UN
-                for (int k = 0; k < 16; k++) {
-                    const int t = c + k;
-                    const float w = live && t < T ? gt[t] : 0.0f;
-                    const float h = w != 0.0f ? union_act(a.act, __uint_as_float(v[k]), 0.0f) * w : 0.0f;
-                    if (live && t < T) store_h(Hn + (size_t)t * ldh, h, a.terms, T * ldh);
-                }
-            }
-        }
-    }
-    tc_fence_before();
-}
-
-// Gate/up over the union.  Bound: HBM (each selected gate/up row read once).
-// A TMA instruction costs a warp about 24 ns plus 1.3 ns per 128-byte line it
-// moves, so one warp issuing the 1 KB boxes of the units reaches 26 GB/s on its
-// SM and four warps 80 GB/s; an SM's share of HBM is 45 GB/s.  Units of 8
-// neurons keep every CTA within one unit of the mean (64 tokens of the 8B
-// shape: 1488 units on 152 CTAs, 10 at most against 9.8; whole experts left
-// two rounds for 186 experts).
-// One thread issues an MMA every 55 cycles at best and spends about 300 more on
-// a stage's wait and commit, so a single MMA warp took 250 ns per 64-wide chunk
-// (16 us of an 8-token call's 24).  Two warps share the work: one M = 128 tile
-// each, or, when every pass fits one tile, every other stage each (the two sums
-// are added in the epilogue).
-// The unused rows of a pass's last tile hold whatever the ring holds; their
-// sums stay in accumulator rows that are never read.
-PP_DEVINL void gu_phase(const UnionArgs& a, UnionShared& sh, unsigned char* smem, uint32_t tmem, int nU) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int T = a.T, E = a.E, N = a.N, nk = a.nk;
-    const bool gated = a.act == PP_ACT_SWIGLU;
-    const int upe = gated ? 8 : 4;  // units of an expert
-    const int units = nU * upe, G = gridDim.x;
-    const int u0 = units * (int)blockIdx.x / G, u1 = units * ((int)blockIdx.x + 1) / G;
-    const int most = min(kPassUnits, (units + G - 1) / G);
-    const bool two = most > kTileUnits;  // MMA warp m takes tile m; else every other stage
-    // a stage holds one K chunk, or two where at least four stages of two fit
-    const int xbytes = N * 128, chunk = xbytes + most * kUnitBytes, avail = (int)(kUnionSmem - 1024 - kGuSlack);
-    const int cps = avail / (2 * chunk) >= 4 ? 2 : 1;
-    // With the stages dealt to two MMA warps in turn, the ring is even: a slot is
-    // then always the same warp's, which has seen every earlier phase of its
-    // full barrier (a parity wait cannot tell a phase from the one two before).
-    const int stage = cps * chunk, fit = min(kMaxStages, avail / stage), nst = two ? fit : fit & ~1;
-    const int nks = (nk + cps - 1) / cps;
-    if (tid == 0) {
-        for (int i = 0; i < kMaxStages; i++) {
-            mbar_init(&sh.full[i], kProd);
-            mbar_init(&sh.empty[i], two ? 2 : 1);
-        }
-        mbar_init(&sh.tfull, 2);
-        fence_mbar_init();
-    }
-    fence_proxy_async_smem();  // the ring was ordinary shared memory before
-    __syncthreads();
-    if (u0 == u1 && warp == kWdWarp) wd_prologue(a, sh, smem, nU);
-    Ring rp, rm;          // producers' and MMA warps' positions
-    bool primed = false;  // the ring has been filled once
-    uint32_t pass = 0;
-    for (int base = u0; base < u1; base += kPassUnits, pass ^= 1u) {
-        const int nun = min(kPassUnits, u1 - base);
-        if (warp < kProd) {
-            // box i of a stage: 0 = the x tile, then the units' weight rows;
-            // box i goes out from lane i / 4 of warp i % 4
-            const int i = lane * kProd + warp, per = gated ? 2 : 1;
-            const int nbox = 1 + nun * per;
-            int row = 0, off = 0;
-            const CUtensorMap* map = &a.map_x;
-            if (i > 0 && i < nbox) {
-                const int g = base + (i - 1) / per, half = (i - 1) % per;
-                row = sh.ul[g / upe] * kDExpert + (g % upe) * (kDExpert / upe);
-                off = xbytes + (i - 1) * (kUnitBytes / per);
-                map = gated && half == 0 ? &a.map_wg : &a.map_wu;
-            }
-            const int nmine = nbox > warp ? (nbox - warp + kProd - 1) / kProd : 0;  // this warp's boxes
-            const uint32_t bytes = (uint32_t)(cps * (warp == 0 ? xbytes + (nmine - 1) * (kUnitBytes / per)
-                                                               : nmine * (kUnitBytes / per)));
-            for (int ks = 0; ks < nks; ks++) {
-                if (lane == 0) {
-                    if (primed) mbar_wait(&sh.empty[rp.s], rp.ph ^ 1u, a.status, a.lim);
-                    mbar_arrive_expect_tx(&sh.full[rp.s], bytes);
-                }
-                __syncwarp();
-                // (a chunk past the row end is filled with zeros)
-                if (i < nbox) {
-                    unsigned char* dst = smem + (size_t)rp.s * stage + off;
-                    tma_load_2d(dst, map, ks * cps * 64, row, &sh.full[rp.s]);
-                    if (cps == 2) tma_load_2d(dst + chunk, map, (ks * 2 + 1) * 64, row, &sh.full[rp.s]);
-                }
-                rp.next(nst);
-                if (rp.s == 0) primed = true;
-            }
-        } else if (warp < kMmaWarp + 2) {
-            const int m = warp - kMmaWarp;
-            const uint32_t idesc = idesc_bf16_m128(N), acc = tmem + (uint32_t)(m * N);
-            const int a0 = xbytes + (two ? m * kTileW : 0);
-            if (lane == 0) {
-                for (int ks = 0; ks < nks; ks++) {
-                    if (two || (ks & 1) == m) {
-                        mbar_wait(&sh.full[rm.s], rm.ph, a.status, a.lim);
-                        if (two && m * kTileUnits >= nun) {
-                            mbar_arrive(&sh.empty[rm.s]);  // no unit in this tile
-                        } else {
-                            tc_fence_after();
-                            unsigned char* st = smem + (size_t)rm.s * stage;
-                            umma_k64(acc, st + a0, st, idesc, ks > (two ? 0 : m));
-                            if (cps == 2) umma_k64(acc, st + chunk + a0, st + chunk, idesc, true);
-                            umma_commit(&sh.empty[rm.s]);
-                        }
-                    }
-                    rm.next(nst);
-                }
-                umma_commit(&sh.tfull);
-            }
-            __syncwarp();
-        }
-        // gate weights of the pass's experts, while the last stages land
-        const int p0 = base / upe, np = (base + nun - 1) / upe - p0 + 1;
-        if (warp >= kMmaWarp + 2)
-            for (int p = 0; p < np; p++)
-                for (int t = tid - 32 * (kMmaWarp + 2); t < T; t += 64) sh.gw[p][t] = __ldcg(a.gexp + (size_t)t * E + sh.ul[p0 + p]);
-        __syncthreads();
-        mbar_wait(&sh.tfull, pass, a.status, a.lim);
-        // the ring is free: the first W_down tiles may go out
-        if (warp == kWdWarp && base + kPassUnits >= u1) wd_prologue(a, sh, smem, nU);
-        tc_fence_after();
-        if (N == 16)
-            gu_epilogue<1>(a, sh, tmem, base, nun, upe, !two && nks > 1);
-        else
-            gu_epilogue<16>(a, sh, tmem, base, nun, upe, !two && nks > 1);
-        if (base + kPassUnits < u1) {  // the accumulators and gw are free for the next pass
-            __syncthreads();
-            tc_fence_after();
-        }
-    }
-}
-
-// y[t][row] without the experts that token t did not select: a zero activation
-// times a non-finite weight is NaN in the union's sums, so a non-finite result
-// is formed again from the token's own experts.
-static __device__ __noinline__ float own_experts_only(const UnionArgs& a, const int* ul, int nU, int t, int row) {
-    const size_t ld = (size_t)a.E * kDExpert;
-    float s = 0.0f;
-    for (int u = 0; u < nU; u++) {
-        const int e = ul[u];
-        if (__ldcg(a.gexp + (size_t)t * a.E + e) == 0.0f) continue;
-        for (int k = 0; k < kDExpert; k++)
-            for (int m = a.terms - 1; m >= 0; m--)
-                s = fmaf(__bfloat162float(a.H[(size_t)(m * a.T + t) * ld + u * kDExpert + k]),
-                         __bfloat162float(a.Wd[(size_t)row * ld + e * kDExpert + k]), s);
-    }
-    return s;
-}
-
-// Down projection over the union: D[128 rows x N] += W_down[tile, expert]
-// . H_expert^T, a tile's experts accumulated in TMEM.  Bound: HBM (each
-// selected column block of W_down read once; the 64-column block of a tile is
-// one 16 KB box).  A run crosses at most `slots - 1` tile boundaries, so CTA b
-// writes its i-th tile's sums to slot i of its partials [slots][T][128]; the
-// partials of a tile are then added in CTA order, a warp per (tile, token).
-// Only the H producer waits for the other CTAs' activations.
-PP_DEVINL void down_phase(const UnionArgs& a, UnionShared& sh, unsigned char* smem, uint32_t tmem, int nU) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int T = a.T, TT = a.terms * T, N = a.N, G = gridDim.x;  // TT columns are used
-    const DownRun d(a, nU);
-    const int mm = down_mma(N);
-    const int L = a.ntile * nU, R = d.R, n = d.n, tile0 = d.tile0, first = d.first, stage = d.stage, nst = d.nst;
-    __syncthreads();  // this CTA's activations are written
-    if (tid == 32 * kHWarp) grid_arrive(a.bar);
-
-    if (warp < kProd) {
-        const int nseg = n > 0 ? (first + n - 1) / nU + 1 : 0;
-        for (int sg = 0; sg < nseg; sg++) {
-            const int acc = sg & 1;
-            mbar_wait(&sh.dt[acc], (uint32_t)(sg >> 1) & 1u, a.status, a.lim);
-            tc_fence_after();
-            float* out = a.dpart + ((size_t)blockIdx.x * a.slots + sg) * TT * 128 + 32 * warp + lane;
-            const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(acc * mm * N);
-            // pairs [s0, s1) of the run; a single pair is in the accumulator of its own MMA warp
-            const int s0 = max(0, sg * nU - first), s1 = min(n, (sg + 1) * nU - first);
-            const bool both = mm == 2 && s1 - s0 > 1;
-            const uint32_t tb = both || mm == 1 ? ta : ta + (uint32_t)((s0 & 1) * N);
-            for (int c = 0; c < N; c += 16) {
-                uint32_t v[16];
-                tmem_ld16(tb + (uint32_t)c, v);
-                if (both) {
-                    uint32_t o[16];
-                    tmem_ld16(ta + (uint32_t)(N + c), o);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int k = 0; k < 16; k++) v[k] = __float_as_uint(__uint_as_float(v[k]) + __uint_as_float(o[k]));
-                } else {
-                    tmem_ld_wait();
-                }
-#pragma unroll
-                for (int k = 0; k < 16; k++)
-                    if (c + k < TT) out[(size_t)(c + k) * 128] = __uint_as_float(v[k]);
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.de[acc]);
-        }
-    } else if (warp < kMmaWarp + mm) {
-        if (lane == 0) {
-            const int m = warp - kMmaWarp;
-            const uint32_t idesc = idesc_bf16_m128(N);
-            Ring r;
-            int u = first, acc = 0;
-            bool fresh = true;  // no pair of this segment yet
-            for (int i = 0; i < n; i++) {
-                const int c = acc & 1;
-                if (acc >= 2 && u == 0) mbar_wait(&sh.de[c], (uint32_t)((acc >> 1) - 1) & 1u, a.status, a.lim);
-                if ((i & (mm - 1)) == m) {
-                    mbar_wait(&sh.dfull[r.s], r.ph, a.status, a.lim);
-                    tc_fence_after();
-                    unsigned char* st = smem + (size_t)r.s * stage;
-                    umma_k64(tmem + (uint32_t)((c * mm + m) * N), st, st + kTileW, idesc, !fresh);
-                    umma_commit(&sh.dempty[r.s]);
-                    fresh = false;
-                }
-                r.next(nst);
-                if (++u == nU || i + 1 == n) {
-                    umma_commit(&sh.dt[c]);
-                    acc++;
-                    u = 0;
-                    fresh = true;
-                }
-            }
-        }
-        __syncwarp();
-    } else if (warp == kWdWarp) {
-        if (lane == 0) {  // after the first ring's worth (wd_prologue)
-            Ring r;
-            int i = min(n, nst), u = first + i, tile = tile0;
-            for (; u >= nU && nU > 0; u -= nU) tile++;
-            for (; i < n; i++) {
-                mbar_wait(&sh.dempty[r.s], r.ph, a.status, a.lim);
-                load_wd(a, sh, smem, d, r.s, u, tile);
-                r.next(nst);
-                if (++u == nU) {
-                    u = 0;
-                    tile++;
-                }
-            }
-        }
-        __syncwarp();
-    } else if (warp == kHWarp) {
-        if (lane == 0) {
-            sh.bar_target += G;
-            grid_wait(a.bar, sh.bar_target, a.status, a.lim);
-            fence_proxy_async_global();  // H was written by ordinary stores
-            const int hbytes = N * 128;
-            Ring r;
-            int u = first;
-            for (int i = 0; i < n; i++) {
-                if (i >= nst) mbar_wait(&sh.dempty[r.s], r.ph ^ 1u, a.status, a.lim);
-                mbar_arrive_expect_tx(&sh.dfull[r.s], (uint32_t)hbytes);
-                tma_load_2d(smem + (size_t)r.s * stage + kTileW, &a.map_h, u * kDExpert, 0, &sh.dfull[r.s]);
-                r.next(nst);
-                if (++u == nU) u = 0;
-            }
-        }
-        __syncwarp();
-    }
-    grid_sync(a, sh);
-    for (int q = blockIdx.x * (kThreads / 32) + warp; q < a.ntile * T; q += G * (kThreads / 32)) {
-        const int tile = q / T, t = q - tile * T, row = tile * 128 + lane * 4;
-        if (row >= a.d) continue;
-        float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (nU > 0) {
-            const int j0 = tile * nU, b0 = run_of(L, j0, R), b1 = run_of(L, j0 + nU - 1, R);
-            // the first run may have begun in an earlier tile; every other run
-            // of the tile begins inside it (slot 0)
-            const int slot0 = tile - run_begin(L, b0, R) / nU;
-            for (int m = a.terms - 1; m >= 0; m--) {  // the smallest term first
-                const float* base = a.dpart + (size_t)(m * T + t) * 128 + lane * 4;
-                for (int b = b0; b <= b1; b += 8) {
-                    float4 v[8];
-#pragma unroll
-                    for (int k = 0; k < 8; k++)
-                        if (b + k <= b1)
-                            v[k] = __ldcg(reinterpret_cast<const float4*>(
-                                base + ((size_t)(b + k) * a.slots + (b + k == b0 ? slot0 : 0)) * TT * 128));
-#pragma unroll
-                    for (int k = 0; k < 8; k++)
-                        if (b + k <= b1) {
-                            s[0] += v[k].x;
-                            s[1] += v[k].y;
-                            s[2] += v[k].z;
-                            s[3] += v[k].w;
-                        }
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (!isfinite(s[k])) s[k] = own_experts_only(a, sh.ul, nU, t, row + k);
-        }
-        *reinterpret_cast<uint2*>(a.y + (size_t)t * a.d + row) = make_uint2(pack_bf16x2(s[0], s[1]), pack_bf16x2(s[2], s[3]));
-    }
-}
-
-__global__ void __launch_bounds__(kThreads, 1) union_layer_kernel(const __grid_constant__ UnionArgs a) {
+__global__ void __launch_bounds__(kUnionThreads, 1) union_layer_kernel(const __grid_constant__ UnionArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    __shared__ UnionShared sh;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const uint32_t cols = tmem_cols(max(a.rn, a.N * (down_mma(a.N) > 1 ? 4 : 2)));
+    __shared__ UnionShared<kUnionMaxT> sh;
+    __shared__ RouterShared rs;
+    const int tid = threadIdx.x;
+    const int T = a.f.T, E = a.f.E;
     if (tid == 0) {
         for (int i = 0; i < kRouterStages; i++) {
-            mbar_init(&sh.rfull[i], 1);
-            mbar_init(&sh.rempty[i], 1);
+            mbar_init(&rs.full[i], 1);
+            mbar_init(&rs.empty[i], 1);
         }
-        mbar_init(&sh.rdone, 1);
-        for (int i = 0; i < kMaxStages; i++) {
-            mbar_init(&sh.dfull[i], 2);
-            mbar_init(&sh.dempty[i], 1);
-        }
-        for (int i = 0; i < 2; i++) {
-            mbar_init(&sh.dt[i], down_mma(a.N));
-            mbar_init(&sh.de[i], kProd);
-        }
-        fence_mbar_init();
+        mbar_init(&rs.done, 1);
     }
-    if (tid < 8) sh.um[tid] = 0u;
-    if (warp == kMmaWarp) {
-        tmem_alloc(&sh.taddr, cols);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = sh.taddr;
+    if (tid < 8) rs.um[tid] = 0u;
+    const uint32_t cols = union_cols(a.f, a.rn), tmem = union_begin(a.f, sh, cols);
     if (a.do_route) {
-        router_phase(a, sh, smem, tmem);
-        grid_sync(a, sh);
+        router_phase(a, rs, smem, tmem);
+        if (tid == 32 * kHWarp) sh.bar_target = grid_bar_base(a.f.bar, gridDim.x);
+        grid_sync(a.f, sh);
         tc_fence_after();
         select_phase(a, smem);
-        grid_sync(a, sh);
+        grid_sync(a.f, sh);
     } else {
         pdl_wait();
         pdl_launch_dependents();
-        if (tid == 0) sh.bar_target = grid_bar_base(a.bar, gridDim.x);
+        if (tid == 0) sh.bar_target = grid_bar_base(a.f.bar, gridDim.x);
     }
     // the union of the tokens' experts, ascending
     uint32_t own = 0u;
-    for (int t = tid >> 3; t < a.T; t += kThreads / 8) own |= __ldcg(a.bits + (size_t)t * 8 + (tid & 7));
-    if (own) atomicOr(&sh.um[tid & 7], own);
+    for (int t = tid >> 3; t < T; t += kUnionThreads / 8) own |= __ldcg(a.bits + (size_t)t * 8 + (tid & 7));
+    if (own) atomicOr(&rs.um[tid & 7], own);
     __syncthreads();
     int nU = 0;
     {
@@ -698,7 +208,7 @@ __global__ void __launch_bounds__(kThreads, 1) union_layer_kernel(const __grid_c
 #pragma unroll
         for (int w = 0; w < 8; w++) {
             // experts past E (a selection that is not this call's, after an error) are dropped
-            const uint32_t m = 32 * w + 32 <= a.E ? sh.um[w] : 32 * w < a.E ? sh.um[w] & ((1u << (a.E & 31)) - 1u) : 0u;
+            const uint32_t m = 32 * w + 32 <= E ? rs.um[w] : 32 * w < E ? rs.um[w] & ((1u << (E & 31)) - 1u) : 0u;
             nU += __popc(m);
             if (w < (e >> 5)) before += __popc(m);
             if (w == (e >> 5)) {
@@ -708,11 +218,10 @@ __global__ void __launch_bounds__(kThreads, 1) union_layer_kernel(const __grid_c
         }
     }
     __syncthreads();
-    gu_phase(a, sh, smem, tmem, nU);
-    down_phase(a, sh, smem, tmem, nU);
-    tc_fence_before();
-    __syncthreads();
-    if (warp == kMmaWarp) tmem_dealloc(tmem, cols);
+    auto gate = [gexp = a.gexp, E](int t, int e) { return __ldcg(gexp + (size_t)t * E + e); };
+    gu_phase<kUnionSmem - 1024>(a.f, sh, gate, smem, tmem, nU);
+    down_phase<kUnionSmem - 1024>(a.f, sh, gate, smem, tmem, nU);
+    union_end(tmem, cols);
 }
 
 int pad16(int T) { return (T + 15) / 16 * 16; }
@@ -725,28 +234,44 @@ size_t union_part_floats(int T, int d) {
     return rows * 128 * (size_t)std::min(std::max(T, 16), kUnionMaxT);
 }
 
+bool union_ffn_args(const GroupedArgs& g, int grid, UnionFfn* a) {
+    const bool gated = g.act == PP_ACT_SWIGLU;
+    const uint64_t rows = (uint64_t)g.E * kDExpert;
+    a->T = g.T;
+    a->E = g.E;
+    a->d = g.d;
+    a->N = pad16(g.T);
+    a->terms = 3 * g.T <= 16 ? 3 : 1;  // the terms fit the MMA's 16 columns
+    a->nk = g.plan.nk;
+    a->ntile = (g.d + 127) / 128;
+    // tiles that a run can touch: ceil(pairs / CTAs) consecutive pairs, or 3
+    // pairs where there are fewer than kMinRun pairs per CTA
+    a->slots = std::max(a->ntile / grid + 2, 3);
+    a->act = g.act;
+    a->H = g.H;
+    a->dpart = g.dpart;
+    a->Wd = static_cast<const __nv_bfloat16*>(g.Wd);
+    a->y = static_cast<__nv_bfloat16*>(g.y);
+    a->bar = g.bar;
+    a->status = g.status;
+    a->lim = g.timeout_ns;
+    const uint32_t box = gated ? 8 : 16;
+    return encode_2d(&a->map_x, g.x, g.d, g.T, 64, a->N) && encode_2d(&a->map_wu, g.Wu, g.d, rows, 64, box) &&
+           encode_2d(&a->map_wg, gated ? g.Wg : g.Wu, g.d, rows, 64, box) &&
+           encode_2d(&a->map_h, g.H, rows, (uint64_t)a->terms * g.T, 64, a->N) &&
+           encode_2d(&a->map_wd, g.Wd, rows, g.d, 64, 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+}
+
 cudaError_t union_layer(const GroupedArgs& g, bool do_route, int sms, cudaStream_t st) {
     UnionArgs a;
     std::memset(&a, 0, sizeof a);
-    const bool gated = g.act == PP_ACT_SWIGLU;
-    const uint64_t rows = (uint64_t)g.E * kDExpert;
     const int grid = std::min(sms, kUnionMaxGrid);
-    a.T = g.T;
-    a.E = g.E;
-    a.d = g.d;
-    a.N = pad16(g.T);
-    a.terms = 3 * g.T <= 16 ? 3 : 1;  // the terms fit the MMA's 16 columns
-    a.nk = g.plan.nk;
+    if (!union_ffn_args(g, grid, &a.f)) return cudaErrorInvalidValue;
     a.mt = (g.T + 127) / 128;
     a.kpb = g.plan.kpb;
     a.nsplit = g.plan.nsplit;
     // experts of a router task: 32, or 64 where the tasks of 32 would not fit one round
     a.rn = a.mt * a.nsplit * ((g.E + 31) / 32) <= grid ? 32 : 64;
-    a.ntile = (g.d + 127) / 128;
-    // tiles that a run can touch: ceil(pairs / CTAs) consecutive pairs, or 3
-    // pairs where there are fewer than kMinRun pairs per CTA
-    a.slots = std::max(a.ntile / grid + 2, 3);
-    a.act = g.act;
     a.gate = g.gate;
     a.rule = g.rule;
     a.do_route = do_route ? 1 : 0;
@@ -758,22 +283,11 @@ cudaError_t union_layer(const GroupedArgs& g, bool do_route, int sms, cudaStream
     a.logits = do_route ? g.logits_out : nullptr;
     a.bits = g.bits;
     a.gexp = g.gexp;
-    a.H = g.H;
-    a.dpart = g.dpart;
-    a.Wd = static_cast<const __nv_bfloat16*>(g.Wd);
-    a.y = static_cast<__nv_bfloat16*>(g.y);
-    a.bar = g.bar;
-    a.status = g.status;
-    a.lim = g.timeout_ns;
-    const uint32_t box = gated ? 8 : 16;
-    if ((do_route && (!encode_2d(&a.map_rx, g.x, g.d, g.T, 64, 128) || !encode_2d(&a.map_wr, g.Wr, g.d, g.E, 64, a.rn))) ||
-        !encode_2d(&a.map_x, g.x, g.d, g.T, 64, a.N) || !encode_2d(&a.map_wu, g.Wu, g.d, rows, 64, box) ||
-        !encode_2d(&a.map_wg, gated ? g.Wg : g.Wu, g.d, rows, 64, box) || !encode_2d(&a.map_h, g.H, rows, (uint64_t)a.terms * g.T, 64, a.N) ||
-        !encode_2d(&a.map_wd, g.Wd, rows, g.d, 64, 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))
+    if (do_route && (!encode_2d(&a.map_rx, g.x, g.d, g.T, 64, 128) || !encode_2d(&a.map_wr, g.Wr, g.d, g.E, 64, a.rn)))
         return cudaErrorInvalidValue;
     cudaError_t e = set_smem(union_layer_kernel, kUnionSmem);
     if (e != cudaSuccess) return e;
-    return launch_coop(union_layer_kernel, dim3(grid), dim3(kThreads), kUnionSmem, st, a);
+    return launch_coop(union_layer_kernel, dim3(grid), dim3(kUnionThreads), kUnionSmem, st, a);
 }
 
 }  // namespace pp
