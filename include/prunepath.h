@@ -154,6 +154,11 @@ pp_status pp_sparse_ffn(const pp_desc *desc, const void *x, int T, const void *W
                         void *ws, size_t ws_bytes, void *stream);
 
 /* pp_route followed by pp_sparse_ffn, fused where the token count allows.
+   Up to 256 bf16 tokens (4 tokens and fewer: the fused kernel; 8 for fp32) the
+   layer is one cooperative launch that starts when all its CTAs, one per SM,
+   can be resident: work that other streams have on the GPU's SMs delays it.
+   On a stream that owns fewer SMs (a green context) 5 to 256 tokens run on a
+   smaller grid; the fused kernel needs every SM (PP_ERR_CUDA).
    The selection is pp_route's, to the last bit; y agrees with pp_sparse_ffn's
    to rounding.  sel_out may be NULL (the selection is then not written). */
 pp_status pp_layer(const pp_desc *desc, const void *x, int T, const void *W_r, const void *W_gate,

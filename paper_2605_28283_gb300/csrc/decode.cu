@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kDecThreads, 1)
         const unsigned ep = a.epochs[b];
         a.epochs[b] = ep + 1u;
         s_tag = ep + 1u;
-        if constexpr (UNI) ush.bar_target = grid_bar_base(a.uni.bar, G);
+        if constexpr (UNI) ush.bar_target = grid_bar_base(a.uni.bar);
     }
     // every CTA waits for its copy of x here, so no bulk copy is ever still
     // in flight when a CTA that has no work left exits

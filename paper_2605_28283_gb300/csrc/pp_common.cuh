@@ -214,20 +214,24 @@ PP_DEVINL float wait_tagged(const unsigned long long* p, unsigned tag, unsigned*
 }
 
 // --------------------------------------------------------------- grid barrier
-// Barrier of all CTAs of a cooperative launch on one 64-bit arrival counter
-// (it only grows: every launch adds a multiple of its CTA count).  One thread
-// of a CTA reads the counter once, early in the launch (grid_bar_base), and
-// keeps the target of the next barrier; an arrival is one reduction without a
-// reply, and the waiters poll the counter itself.  What the CTA wrote before
-// its arrival (and a barrier of the CTA) is visible to what it reads after the
-// wait.  Waits are bounded.
-PP_DEVINL unsigned long long grid_bar_base(const unsigned long long* count, unsigned nctas) {
-    const unsigned long long v = ld_relaxed_u64(count);
-    return v - v % nctas;  // at most nctas - 1 of this launch's CTAs have arrived so far
+// Barrier of all CTAs of a cooperative launch on one 64-bit arrival counter.
+// Every barrier adds kBarrierSum to it, whatever the grid (CTA 0 arrives for the
+// CTAs that a full one has more), so launches of several grids share a counter.
+// One thread of a CTA reads the counter once, early in the launch
+// (grid_bar_base), and keeps the target of the next barrier; an arrival is one
+// reduction without a reply, and the waiters poll the counter itself.  What the
+// CTA wrote before its arrival (and a barrier of the CTA) is visible to what it
+// reads after the wait.  Waits are bounded.
+constexpr unsigned kBarrierSum = kMaxGrid;
+
+PP_DEVINL unsigned long long grid_bar_base(const unsigned long long* count) {
+    // this CTA has not arrived, so the launch's first barrier has less than its sum
+    return ld_relaxed_u64(count) & ~(unsigned long long)(kBarrierSum - 1);
 }
 
 PP_DEVINL void grid_arrive(unsigned long long* count) {
-    asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(count) : "memory");
+    const unsigned long long n = blockIdx.x == 0 ? kBarrierSum + 1 - gridDim.x : 1u;
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(count), "l"(n) : "memory");
 }
 
 PP_DEVINL bool grid_wait(const unsigned long long* count, unsigned long long target, unsigned* status,

@@ -70,7 +70,7 @@ PP_DEVINL void grid_sync(const UnionFfn& a, UnionShared<MaxT>& sh) {
     __syncthreads();
     if (threadIdx.x == 0) {
         grid_arrive(a.bar);
-        sh.bar_target += gridDim.x;
+        sh.bar_target += kBarrierSum;
         grid_wait(a.bar, sh.bar_target, a.status, a.lim);
     }
     __syncthreads();
@@ -439,7 +439,7 @@ PP_DEVINL void down_phase(const UnionFfn& a, UnionShared<MaxT>& sh, Gate gate, u
         __syncwarp();
     } else if (warp == kHWarp) {
         if (lane == 0) {
-            sh.bar_target += G;
+            sh.bar_target += kBarrierSum;
             grid_wait(a.bar, sh.bar_target, a.status, a.lim);
             fence_proxy_async_global();  // H was written by ordinary stores
             const int hbytes = N * 128;

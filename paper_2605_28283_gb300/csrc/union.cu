@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kUnionThreads, 1) union_layer_kernel(const __g
     const uint32_t cols = union_cols(a.f, a.rn), tmem = union_begin(a.f, sh, cols);
     if (a.do_route) {
         router_phase(a, rs, smem, tmem);
-        if (tid == 32 * kHWarp) sh.bar_target = grid_bar_base(a.f.bar, gridDim.x);
+        if (tid == 32 * kHWarp) sh.bar_target = grid_bar_base(a.f.bar);
         grid_sync(a.f, sh);
         tc_fence_after();
         select_phase(a, smem);
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kUnionThreads, 1) union_layer_kernel(const __g
     } else {
         pdl_wait();
         pdl_launch_dependents();
-        if (tid == 0) sh.bar_target = grid_bar_base(a.f.bar, gridDim.x);
+        if (tid == 0) sh.bar_target = grid_bar_base(a.f.bar);
     }
     // the union of the tokens' experts, ascending
     uint32_t own = 0u;
@@ -262,32 +262,37 @@ bool union_ffn_args(const GroupedArgs& g, int grid, UnionFfn* a) {
            encode_2d(&a->map_wd, g.Wd, rows, g.d, 64, 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
+// A stream may own fewer SMs than the device has (a green context): the grid
+// then shrinks until it is resident at once (each CTA takes more units and runs).
 cudaError_t union_layer(const GroupedArgs& g, bool do_route, int sms, cudaStream_t st) {
-    UnionArgs a;
-    std::memset(&a, 0, sizeof a);
-    const int grid = std::min(sms, kUnionMaxGrid);
-    if (!union_ffn_args(g, grid, &a.f)) return cudaErrorInvalidValue;
-    a.mt = (g.T + 127) / 128;
-    a.kpb = g.plan.kpb;
-    a.nsplit = g.plan.nsplit;
-    // experts of a router task: 32, or 64 where the tasks of 32 would not fit one round
-    a.rn = a.mt * a.nsplit * ((g.E + 31) / 32) <= grid ? 32 : 64;
-    a.gate = g.gate;
-    a.rule = g.rule;
-    a.do_route = do_route ? 1 : 0;
-    a.p = g.p;
-    a.part = g.part;
-    a.ids = do_route ? g.ids : nullptr;
-    a.counts = do_route ? g.counts : nullptr;
-    a.gates = do_route ? g.gates : nullptr;
-    a.logits = do_route ? g.logits_out : nullptr;
-    a.bits = g.bits;
-    a.gexp = g.gexp;
-    if (do_route && (!encode_2d(&a.map_rx, g.x, g.d, g.T, 64, 128) || !encode_2d(&a.map_wr, g.Wr, g.d, g.E, 64, a.rn)))
-        return cudaErrorInvalidValue;
     cudaError_t e = set_smem(union_layer_kernel, kUnionSmem);
     if (e != cudaSuccess) return e;
-    return launch_coop(union_layer_kernel, dim3(grid), dim3(kUnionThreads), kUnionSmem, st, a);
+    for (int grid = std::min(sms, kUnionMaxGrid);; grid = (grid + 1) / 2) {
+        UnionArgs a;
+        std::memset(&a, 0, sizeof a);
+        if (!union_ffn_args(g, grid, &a.f)) return cudaErrorInvalidValue;
+        a.mt = (g.T + 127) / 128;
+        a.kpb = g.plan.kpb;
+        a.nsplit = g.plan.nsplit;
+        // experts of a router task: 32, or 64 where the tasks of 32 would not fit one round
+        a.rn = a.mt * a.nsplit * ((g.E + 31) / 32) <= grid ? 32 : 64;
+        a.gate = g.gate;
+        a.rule = g.rule;
+        a.do_route = do_route ? 1 : 0;
+        a.p = g.p;
+        a.part = g.part;
+        a.ids = do_route ? g.ids : nullptr;
+        a.counts = do_route ? g.counts : nullptr;
+        a.gates = do_route ? g.gates : nullptr;
+        a.logits = do_route ? g.logits_out : nullptr;
+        a.bits = g.bits;
+        a.gexp = g.gexp;
+        if (do_route && (!encode_2d(&a.map_rx, g.x, g.d, g.T, 64, 128) || !encode_2d(&a.map_wr, g.Wr, g.d, g.E, 64, a.rn)))
+            return cudaErrorInvalidValue;
+        e = launch_coop(union_layer_kernel, dim3(grid), dim3(kUnionThreads), kUnionSmem, st, a);
+        if (e != cudaErrorCooperativeLaunchTooLarge || grid == 1) return e;
+        (void)cudaGetLastError();
+    }
 }
 
 }  // namespace pp
