@@ -68,17 +68,23 @@ struct RouterShared {
 // split in the order of router_gemm_kernel, so a logit's sum is the same.  The
 // expert groups make 112 CTAs of what would be 16 (d = 4096, E = 224): a CTA's
 // loads, MMAs (N = 32) and stores are a seventh (64 tokens: 6.1 -> 3.2 us).
-// The W_r tiles are requested before the previous kernel on the stream has
-// completed.
+// Before the previous kernel on the stream has completed, the W_r tiles are only
+// prefetched into L2 (where that kernel's writes arrive too): it may be the one
+// that writes W_r.
 PP_DEVINL void router_phase(const UnionArgs& a, RouterShared& sh, unsigned char* smem, uint32_t tmem) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ngrp = (a.f.E + a.rn - 1) / a.rn, tasks = a.mt * a.nsplit * ngrp, rstage = kTileW + a.rn * 128;
     uint32_t round = 0;
     int it0 = 0;  // chunks of this CTA's earlier rounds
-    bool waited = false;
     for (int b = blockIdx.x; b < tasks; b += gridDim.x, round++) {
         const int e0 = (b % ngrp) * a.rn, m0 = (b / ngrp % a.mt) * 128, split = b / ngrp / a.mt;
         const int k0 = split * a.kpb, n = min(a.f.nk, k0 + a.kpb) - k0;
+        if (round == 0) {
+            if (warp < kRouterStages && lane == 0)
+                for (int i = warp; i < n; i += kRouterStages) tma_prefetch_2d(&a.map_wr, (k0 + i) * 64, e0);
+            pdl_wait();
+            pdl_launch_dependents();
+        }
         // warp w < 4 loads into stage w: chunk i of all the CTA's chunks is in stage i % 4
         if (warp < kRouterStages && lane == 0) {
             unsigned char* st = smem + (size_t)warp * rstage;
@@ -87,14 +93,9 @@ PP_DEVINL void router_phase(const UnionArgs& a, RouterShared& sh, unsigned char*
                 if (q > 0) mbar_wait(&sh.empty[warp], (uint32_t)(q - 1) & 1u, a.f.status, a.f.lim);
                 mbar_arrive_expect_tx(&sh.full[warp], (uint32_t)rstage);
                 tma_load_2d(st + kTileW, &a.map_wr, (k0 + i) * 64, e0, &sh.full[warp]);
-                if (!waited) pdl_wait();
-                waited = true;
                 tma_load_2d(st, &a.map_rx, (k0 + i) * 64, m0, &sh.full[warp]);
             }
         }
-        if (!waited) pdl_wait();
-        waited = true;
-        if (round == 0) pdl_launch_dependents();
         if (warp == kMmaWarp && lane == 0) {
             const uint32_t idesc = idesc_bf16_m128(a.rn);
             for (int i = 0; i < n; i++) {
@@ -135,7 +136,7 @@ PP_DEVINL void router_phase(const UnionArgs& a, RouterShared& sh, unsigned char*
         __syncthreads();  // the accumulator is free for the next round
         tc_fence_after();
     }
-    if (!waited) {
+    if (round == 0) {  // no task
         pdl_wait();
         pdl_launch_dependents();
     }

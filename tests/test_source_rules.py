@@ -21,3 +21,14 @@ def test_aligned_instructions_follow_a_syncwarp():
                 (os.path.basename(path), text[start:m.start() + 60])
             found += 1
     assert found >= 9
+
+
+def test_union_kernel_reads_nothing_before_the_previous_kernel_is_done():
+    """Launched with programmatic dependent launch, the union kernel may run while
+    the previous kernel on the stream writes any of its inputs, W_r among them: up
+    to pdl_wait() it only prefetches into L2."""
+    text = open(os.path.join(build.CSRC, "union.cu")).read()
+    router = re.sub(r"//[^\n]*", "", text[text.index("PP_DEVINL void router_phase("):text.index("PP_DEVINL void select_phase(")])
+    before = router[:router.index("pdl_wait()")]
+    assert "tma_prefetch_2d(&a.map_wr" in before
+    assert not re.search(r"tma_load_2d|bulk_g2s|ld_relaxed|__ldg|__ldcg|\ba\.part\b", before)
