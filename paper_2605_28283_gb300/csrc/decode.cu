@@ -141,7 +141,8 @@ struct DecodeUnionArgs : DecodeArgs {
 static __device__ __noinline__ void union_ffn(const UnionFfn& f, UnionShared<4>& sh, const float* gw, unsigned char* smem,
                                               int nU) {
     const uint32_t cols = union_cols(f, 0), tmem = union_begin(f, sh, cols);
-    auto gate = [gw, E = f.E](int t, int e) { return gw[t * E + e]; };
+    // (a weight of zero takes no activation here, as in phase 4)
+    auto gate = [gw, E = f.E](int t, int e) { return gw[t * E + e] + 0.0f; };
     gu_phase<kDecodeUnionRing>(f, sh, gate, smem, tmem, nU);
     down_phase<kDecodeUnionRing>(f, sh, gate, smem, tmem, nU);
     union_end(tmem, cols);

@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(256) select_part_cta_kernel(const float* __res
 
 // ================================================================== dispatch
 // bits[t][w]: bit (e % 32) of word e / 32 set when token t activated e;
-// gexp[t][e]: the gate weight of that assignment (gates of a repeated id
-// add up), 0 where e is not activated.  Invalid ids and counts are recorded
+// gexp[t][e]: gexp_entry of that assignment's gate weight (gates of a repeated
+// id add up), +0 where e is not activated.  Invalid ids and counts are recorded
 // and skipped.
 __global__ void __launch_bounds__(256) dispatch_bits_kernel(const int32_t* __restrict__ ids,
                                                             const int32_t* __restrict__ counts,
@@ -364,6 +364,8 @@ __global__ void __launch_bounds__(256) dispatch_bits_kernel(const int32_t* __res
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v |= __shfl_xor_sync(kFull, v, o);
         if (lane == i) bits[(size_t)t * 8 + i] = v;
+        // (the entries that this lane has summed)
+        if ((v >> lane) & 1u && grow[32 * i + lane] == 0.0f) grow[32 * i + lane] = gexp_entry(0.0f);
     }
 }
 

@@ -603,10 +603,15 @@ PP_DEVINL void write_selection_row(int32_t* ids, float* gates, int j, int E, int
 // The whole selection of one token by a CTA of 256 threads, written in both
 // forms: rank order for the caller (ids, counts, gates, logits: the token's
 // rows, each may be NULL but ids and gates only together) and per expert for
-// the FFN kernels (bits: E bits in 8 words; gexp: the gate weight, 0 where the
-// expert is not activated; NULL when no FFN follows).  `load(j)` returns logit
+// the FFN kernels (bits: E bits in 8 words; gexp: gexp_entry of the gate weight,
+// +0 where the expert is not activated; NULL when no FFN follows).  `load(j)` returns logit
 // j.  The cumulative-mass rules below p = 1 take the three-barrier cut, the
 // others the counting selection.
+// An activated expert's gate weight may be zero (a sigmoid that underflows, a
+// caller's zero): it is kept as -0, so that its activation, infinities and NaN
+// included, is still multiplied by it.
+PP_DEVINL float gexp_entry(float gate) { return gate == 0.0f ? -0.0f : gate; }
+
 struct SelOut {
     int32_t* ids;
     int32_t* count;
@@ -640,7 +645,7 @@ PP_DEVINL void select_token_cta(Load load, int E, float p, int rule, int gate, S
                 o.ids[r] = e;
                 o.gates[r] = gv;
             }
-            s.gx[e] = gv;
+            s.gx[e] = gexp_entry(gv);
             atomicOr(&s.bw[e >> 5], 1u << (e & 31));
         }, [] {});  // its last barrier orders gx and bw before the reads below
         if (o.ids)
@@ -655,7 +660,7 @@ PP_DEVINL void select_token_cta(Load load, int E, float p, int rule, int gate, S
         const float gv = on ? (gate == PP_GATE_NONE ? 1.0f : sigmoidf_(g)) : 0.0f;
         if (o.ids) write_selection_row(o.ids, o.gates, j, E, k, on, r, gv);
         if (on) {
-            s.gx[j] = gv;
+            s.gx[j] = gexp_entry(gv);
             atomicOr(&s.bw[j >> 5], 1u << (j & 31));
         }
         __syncthreads();

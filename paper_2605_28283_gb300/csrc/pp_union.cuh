@@ -52,8 +52,11 @@ PP_DEVINL int run_begin(int L, int b, int R) { return b >= R ? L : L * b / R; }
 // The run that holds pair i: run_begin(b) <= i < run_begin(b + 1).
 PP_DEVINL int run_of(int L, int i, int R) { return ((i + 1) * R - 1) / L; }
 
-// kRing: bytes of shared memory for a phase's ring.  `gate(t, e)` in the functions below is the gate weight of token t for expert
-// e, 0 where the token did not select it.
+// kRing: bytes of shared memory for a phase's ring.  `gate(t, e)` in the functions
+// below is the gate weight of token t for expert e, +0 where the token did not
+// select it (a weight of zero is -0).
+PP_DEVINL bool selected(float gate) { return __float_as_uint(gate) != 0u; }
+
 template <int MaxT>
 struct UnionShared {
     uint64_t full[kMaxStages], empty[kMaxStages], tfull;             // gate/up
@@ -181,10 +184,10 @@ PP_DEVINL void gu_epilogue(const UnionFfn& a, UnionShared<MaxT>& sh, uint32_t tm
                     const int t = c + 2 * k + (up ? 1 : 0);
                     const float w = live && t < T ? gt[t] : 0.0f;
                     float h = 0.0f;
-                    if (__any_sync(kFull, w != 0.0f)) {
+                    if (__any_sync(kFull, selected(w))) {
                         const float e0 = __uint_as_float(v[2 * k]), e1 = __uint_as_float(v[2 * k + 1]);
                         const float o = __shfl_xor_sync(kFull, up ? e0 : e1, 8);
-                        if (w != 0.0f) h = union_act(PP_ACT_SWIGLU, up ? e1 : o, up ? o : e0) * w;
+                        if (selected(w)) h = union_act(PP_ACT_SWIGLU, up ? e1 : o, up ? o : e0) * w;
                     }
                     if (live && t < T) store_h(Hn + (size_t)t * ldh, h, a.terms, T * ldh);
                 }
@@ -193,7 +196,7 @@ PP_DEVINL void gu_epilogue(const UnionFfn& a, UnionShared<MaxT>& sh, uint32_t tm
                 for (int k = 0; k < 16; k++) {
                     const int t = c + k;
                     const float w = live && t < T ? gt[t] : 0.0f;
-                    const float h = w != 0.0f ? union_act(a.act, __uint_as_float(v[k]), 0.0f) * w : 0.0f;
+                    const float h = selected(w) ? union_act(a.act, __uint_as_float(v[k]), 0.0f) * w : 0.0f;
                     if (live && t < T) store_h(Hn + (size_t)t * ldh, h, a.terms, T * ldh);
                 }
             }
@@ -335,7 +338,7 @@ __device__ __noinline__ float own_experts_only(const UnionFfn& a, Gate gate, con
     float s = 0.0f;
     for (int u = 0; u < nU; u++) {
         const int e = ul[u];
-        if (gate(t, e) == 0.0f) continue;
+        if (!selected(gate(t, e))) continue;
         for (int k = 0; k < kDExpert; k++)
             for (int m = a.terms - 1; m >= 0; m--)
                 s = fmaf(__bfloat162float(a.H[(size_t)(m * a.T + t) * ld + u * kDExpert + k]),
