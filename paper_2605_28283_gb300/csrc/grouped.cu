@@ -43,7 +43,8 @@ constexpr int kTileBytesA = 128 * 128;  // 128 rows x 64 bf16
 
 // ====================================================================== router
 // Grid (m-tiles, splits).  CTA (m, s): D[128 tokens x NE] over K chunks
-// [s*kpb, min((s+1)*kpb, nk)); partial logits to part[s][t][e].
+// [s*kpb, min((s+1)*kpb, nk)), one at least (grouped_plan); partial logits to
+// part[s][t][e].
 template <int NE>
 __global__ void __launch_bounds__(kTcThreads, 1)
     router_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_wr,
@@ -123,12 +124,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
                 for (int i = 0; i < 32; i += 4)
                     if (c + i < E)
-                        *reinterpret_cast<uint4*>(row + c + i) =
-                            k1 > k0 ? make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]) : make_uint4(0u, 0u, 0u, 0u);
+                        *reinterpret_cast<uint4*>(row + c + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
             } else {
 #pragma unroll
                 for (int i = 0; i < 32; i++)
-                    if (c + i < E) row[c + i] = k1 > k0 ? __uint_as_float(r[i]) : 0.0f;
+                    if (c + i < E) row[c + i] = __uint_as_float(r[i]);
             }
         }
     }
