@@ -258,6 +258,15 @@ def path_kind(w, B):
     return "decode" if (B <= 4 or w.dtype == "f32") else "grouped"
 
 
+def kernels_per_call(w, B):
+    """Kernels that one pp_layer call launches: one up to 8 fp32 or 256 bf16
+    tokens, else routing, gate/up and down (fp32), or router, selection, gate/up,
+    down and combine (bf16)."""
+    if w.dtype == "f32":
+        return 1 if B <= 8 else 3
+    return 1 if B <= 256 else 5
+
+
 def kernel_traffic(workload, p, B, kind="decode"):
     """DRAM bytes per layer call measured by ncu (committed summary), valid
     only while the kernel's sources are unchanged; None otherwise."""
@@ -613,7 +622,6 @@ def main():
     desc, ws, layers = head["desc"], head["ws"], head["layers"]
     value, ms_per_step, roof = head["tokens_per_s"], head["ms_per_step"], head["roofline"]
     head_rec = public(head)
-    kernels_per_layer = 1 if path_kind(w, B) == "decode" else 9
 
     if args.skip_extras:
         if rank == 0:
@@ -800,7 +808,7 @@ def main():
                     flush, world)
         rec = public(m)
         rec["config"] = config_dict(cw, cB, cp, cpool, world, args.no_flush)
-        rec["gpu_launches"] = m["launches"] * (1 if path_kind(cw, cB) == "decode" else 9)
+        rec["gpu_launches"] = m["launches"] * kernels_per_call(cw, cB)
         if cw.n_layers != full_layers:
             rec["model_tokens_per_s"] = m["tokens_per_s"] * cw.n_layers / full_layers
             rec["scaling_note"] = ("timed on %d of the model's %d layers (same shape, independently drawn); "
@@ -823,7 +831,7 @@ def main():
            "hbm_gbs_total": head_rec["total_gbs"], "tflops": head_rec["tflops"],
            "p_sweep": sweep, "rules": rules, "chained": chained, "router_stats": router_stats,
            "moefy_permute": moefy_permute, "warm_l2_tokens_per_s": warm_tok_s,
-           "e2e": e2e, "gpu_launches": args.steps * w.n_layers * kernels_per_layer, "clocks": head_rec["clocks"],
+           "e2e": e2e, "gpu_launches": args.steps * w.n_layers * kernels_per_call(w, B), "clocks": head_rec["clocks"],
            "configs": configs}
     if rank == 0 and world == 1:
         try:
